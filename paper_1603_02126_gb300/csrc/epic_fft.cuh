@@ -139,6 +139,90 @@ __device__ __forceinline__ Cb2 twiddle(Cb2 v) {
   }
 }
 
+// Two FP32 values in one 64-bit register pair; add, subtract, multiply and
+// fused multiply-add act on both in one instruction (the FP32 rate is that of
+// the scalar forms, the issue slots half).
+using f32x2 = unsigned long long;
+
+__device__ __forceinline__ f32x2 f2_pack(float lo, float hi) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ f32x2 f2_splat(float v) { return f2_pack(v, v); }
+__device__ __forceinline__ float2 f2_unpack(f32x2 v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ f32x2 f2_add(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 f2_sub(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 f2_mul(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 f2_fma(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+// The same complex sample of two independent FP32 transforms (two frames):
+// re = (re_0, re_1), im = (im_0, im_1), 16 bytes.
+struct __align__(16) Cf2 {
+  f32x2 re, im;
+};
+
+// Butterfly of a Cf2: the quarter turn costs no multiply, the eighth turns
+// two adds and four fused multiply-adds, every other angle six fused
+// multiply-adds: with w = c + i s, w o = c ((o.re - (s/c) o.im) +
+// i (o.im + (s/c) o.re)), or the same with s and c/s factored out, whichever
+// ratio is at most 1 in size.
+template <int R, int K>
+__device__ __forceinline__ void butterfly(Cf2 (&x)[R], const Cf2 (&e)[R / 2], const Cf2 (&o)[R / 2]) {
+  constexpr int m = ((K * (32 / R)) % 32 + 32) % 32;
+  const Cf2 a = e[K], b = o[K];
+  if constexpr (m == 0) {
+    x[K] = Cf2{f2_add(a.re, b.re), f2_add(a.im, b.im)};
+    x[K + R / 2] = Cf2{f2_sub(a.re, b.re), f2_sub(a.im, b.im)};
+  } else if constexpr (m == 8) {
+    x[K] = Cf2{f2_sub(a.re, b.im), f2_add(a.im, b.re)};
+    x[K + R / 2] = Cf2{f2_add(a.re, b.im), f2_sub(a.im, b.re)};
+  } else if constexpr (m == 4) {
+    const f32x2 u = f2_sub(b.re, b.im), v = f2_add(b.re, b.im);
+    const f32x2 p = f2_splat(cos32(4)), n = f2_splat(-cos32(4));
+    x[K] = Cf2{f2_fma(u, p, a.re), f2_fma(v, p, a.im)};
+    x[K + R / 2] = Cf2{f2_fma(u, n, a.re), f2_fma(v, n, a.im)};
+  } else if constexpr (m == 12) {
+    const f32x2 u = f2_sub(b.re, b.im), v = f2_add(b.re, b.im);
+    const f32x2 p = f2_splat(cos32(4)), n = f2_splat(-cos32(4));
+    x[K] = Cf2{f2_fma(v, n, a.re), f2_fma(u, p, a.im)};
+    x[K + R / 2] = Cf2{f2_fma(v, p, a.re), f2_fma(u, n, a.im)};
+  } else {
+    constexpr float c = cos32(m), s = cos32(8 - m);
+    if constexpr (m < 4 || m > 12) {
+      constexpr float t = s / c;
+      const f32x2 u = f2_fma(b.im, f2_splat(-t), b.re), v = f2_fma(b.re, f2_splat(t), b.im);
+      x[K] = Cf2{f2_fma(u, f2_splat(c), a.re), f2_fma(v, f2_splat(c), a.im)};
+      x[K + R / 2] = Cf2{f2_fma(u, f2_splat(-c), a.re), f2_fma(v, f2_splat(-c), a.im)};
+    } else {
+      constexpr float t = c / s;                 // u = -(t re - im), v = re + t im, times s
+      const f32x2 u = f2_fma(b.re, f2_splat(-t), b.im), v = f2_fma(b.im, f2_splat(t), b.re);
+      x[K] = Cf2{f2_fma(u, f2_splat(-s), a.re), f2_fma(v, f2_splat(s), a.im)};
+      x[K + R / 2] = Cf2{f2_fma(u, f2_splat(s), a.re), f2_fma(v, f2_splat(-s), a.im)};
+    }
+  }
+}
+
 // Radix-2 combination x[k] = e[k] + w^k o[k], x[k + R/2] = e[k] - w^k o[k]
 // for k = 0 .. R/2 - 1, expanded at compile time.
 template <int R, int K, typename T>

@@ -53,6 +53,17 @@ struct ImageArgs {
   const uint2* ptab;       // [COLROUNDS][BT] (slot mask, first tap index) per thread
   const float2* pph;       // [C][npix] window-coordinate phase of each pixel
   float2* ptap;            // [T][C][npix] pixel taps of the call
+  // frame-pair form (epic_pair.cu): gridding as per-cell tap lists in slices
+  // of 32 cells, most taps first
+  int pair;                // 1: frame-pair form
+  const int* pcell;        // grid cell (row * gs + column) of each list, 32 per slice; -1 = none
+  const int2* pslice;      // (first entry relative to the channel's, taps) of each slice
+  const uint2* pent;       // entries (byte offset of E'_a, weight bits), [tap][32] per slice
+  const int* psbase;       // [C + 1] first slice of each channel
+  const int* pebase;       // [C + 1] first entry of each channel
+  const int* pcost;        // [C + 1] prefix sums of the channels' cost per frame pair
+  int gs;                  // row stride of the grid (16-byte cells)
+  int max_slices, max_ent; // most slices / entries of one channel (0: lists not in shared memory)
 };
 
 // Shape facts of the fused image kernel for grid side n.
@@ -167,6 +178,20 @@ int image_fft_lanes(int n);
 // Opt in to the shared memory and report resident CTAs per SM.
 cudaError_t image_kernel_prepare(int n, size_t smem, int n_ant, int steps, int* ctas_per_sm);
 cudaError_t launch_image(int n, const ImageArgs& a, cudaStream_t s);
+
+// Frame-pair fused form (N = 16..128): two frames per FP32 pair through
+// gridding and both transforms.
+constexpr int kPairMaxAnt = 4;   // antennas per thread
+int pair_threads(int n);
+// Row stride of the spectra for at most rows occupied rows.
+int pair_rs(int n, int rows);
+// Dynamic shared memory, with the tap lists when max_slices > 0.
+size_t pair_smem_bytes(int n, int n_ant, int rows, int gs, int max_slices, int max_ent);
+cudaError_t pair_prepare(int n, int n_ant, bool table, size_t smem, int* ctas_per_sm);
+cudaError_t launch_pair(int n, const ImageArgs& a, cudaStream_t s);
+// Owner of image pixel (kx, ky) in the column phase.
+bool pair_pixel_owner(int n, int kx, int ky, PixelOwner* out);
+int pair_col_rounds(int n);
 
 // Warp-specialised fused form (N = 64, 128): producer warps grid and row-FFT
 // frame t + 1 while consumer warps column-FFT frame t (two spectra slots).

@@ -794,6 +794,7 @@ cudaError_t image_kernel_prepare(int n, size_t smem, int n_ant, int steps, int* 
 }
 
 cudaError_t launch_image(int n, const ImageArgs& a, cudaStream_t s) {
+  if (a.pair) return launch_pair(n, a, s);
   if (a.piped) return launch_piped(n, a, s);
   switch (n) {
     case 16: return launch_n<16>(a, s);

@@ -1,0 +1,549 @@
+// Frame-pair forms of the fused imaging kernel (sm_103a, N = 16..128): two
+// consecutive frames of one channel go through gain correction, gridding,
+// both transforms and the square together, each value of the two frames one
+// FP32 pair (fft::Cf2), so that every add and multiply of both frames is one
+// packed instruction and every weight, twiddle and list entry is read once
+// for both.
+//
+// A 1-D transform of length N = 16 NR of an input with L occupied entries is
+// NR independent tasks, one per output residue r: with n = n' + 16 q and
+// k = NR m + r,
+//   X[NR m + r] = sum_n' e^{2 pi i m n' / 16} ( e^{2 pi i r n' / N}
+//                 sum_q x[n' + 16 q] e^{2 pi i r q / NR} ),
+// a sum over the L / 16 occupied blocks, 15 twiddles and one 16-point DFT in
+// registers, for any L.  The tasks of a transform read the same L inputs
+// (shared-memory broadcasts: the NR lanes of one transform are neighbours)
+// and exchange nothing.
+//
+// One persistent launch images a batch.  Every CTA takes an equal share of
+// the estimated cost of the (channel, frame pair) list, so that no last wave
+// is left and an image block is flushed once per channel and share.  Shared
+// memory holds the grid of a frame pair, its row spectra and E' = E / g.
+// Gridding (Eq. 9) gives each lane one grid cell, the cells sorted by their
+// number of taps so that the 32 lanes of a slice run equally long.
+//
+// What bounds it: the FP32 pipe.  A packed instruction takes two cycles (the
+// scalar rate) and three with three distinct operands; one transform task of
+// 40 inputs takes 252 SM cycles with 16 warps resident (DFT 75, twiddles 37,
+// square 20, the rest the input sum and its shared-memory loads), 42 tasks
+// per pair of the 256-antenna, 128 x 128 station.  64 channels x 10^4 4-bit
+// samples: 15.3 ms against 19.3 for one frame per FP32 value with an
+// exchange through shared memory (63 % of the issue slots, 42 % of the FP32
+// pipe); 128 samples 0.254 against 0.361 ms; 248 antennas, 64 x 64, 15
+// channels, 1023 complex64 samples 0.297 against 0.426; 32 antennas, 32 x 32,
+// 2000 samples 37.6 against 53.9 us (with the update).
+#include "epic_fft.cuh"
+#include "epic_internal.h"
+
+#include <cstdint>
+
+namespace epic {
+namespace {
+
+using fft::Cf2;
+using fft::cmul;
+using fft::f2_fma;
+using fft::f2_mul;
+using fft::f2_pack;
+using fft::f2_splat;
+using fft::f2_unpack;
+using fft::f32x2;
+
+// Frame pairs per FP32 partial image (FP64 across): 128 roundings of a running
+// sum, image error 0.9e-7 against 64 bits over 10^4 samples (1.4e-7 at 256).
+constexpr int kPairRun = 128;
+
+// y[j] += x[j] a for four complex pairs and one complex factor a given as
+// splats; consecutive instructions share the factor's operand.
+__device__ __forceinline__ void cmadd4(Cf2* y, const Cf2* __restrict__ x, f32x2 ar, f32x2 ai, f32x2 nai) {
+  Cf2 v[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) v[j] = x[j];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) y[j].re = f2_fma(v[j].re, ar, y[j].re);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) y[j].im = f2_fma(v[j].im, ar, y[j].im);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) y[j].re = f2_fma(v[j].im, nai, y[j].re);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) y[j].im = f2_fma(v[j].re, ai, y[j].im);
+}
+
+// Task r of a transform of src[0 .. len4), len4 a multiple of 4 and uniform
+// over the CTA: y[m] = X[NR m + r].  tw: [16][NR] e^{2 pi i r n' / N};
+// wq: [16][NR] e^{2 pi i r q / NR}.
+template <int NR>
+__device__ __forceinline__ void dft_task(const Cf2* __restrict__ src, int len4, int r, const float2* tw,
+                                         const float2* wq, Cf2 (&y)[16]) {
+#pragma unroll
+  for (int b = 0; b < 4; ++b) {
+    if (4 * b < len4) {
+#pragma unroll
+      for (int j = 4 * b; j < 4 * b + 4; ++j) y[j] = src[j];
+    } else {
+#pragma unroll
+      for (int j = 4 * b; j < 4 * b + 4; ++j) y[j] = Cf2{0ull, 0ull};
+    }
+  }
+  for (int q = 1; 16 * q < len4; ++q) {
+    const float2 a = wq[q * NR + r];
+    const f32x2 ar = f2_splat(a.x), ai = f2_splat(a.y), nai = f2_splat(-a.y);
+    const Cf2* s = src + 16 * q;
+    const int left = len4 - 16 * q;
+#pragma unroll
+    for (int b = 0; b < 4; ++b)
+      if (4 * b < left) cmadd4(&y[4 * b], s + 4 * b, ar, ai, nai);
+  }
+  if constexpr (NR > 1) {
+#pragma unroll
+    for (int j = 1; j < 16; ++j) {
+      const float2 t = tw[j * NR + r];
+      const f32x2 c = f2_splat(t.x), s = f2_splat(t.y), ns = f2_splat(-t.y);
+      const Cf2 v = y[j];
+      y[j].re = f2_fma(v.im, ns, f2_mul(v.re, c));
+      y[j].im = f2_fma(v.re, s, f2_mul(v.im, c));
+    }
+  }
+  fft::Dft<16>::run(y);
+}
+
+// Scaled voltage of the 4-bit sample in the low byte of b.
+__device__ __forceinline__ float2 unpack_ci4(unsigned b, float vs) {
+  const int re = static_cast<int>(b << 24) >> 28;
+  const int im = static_cast<int>(b << 28) >> 28;
+  return make_float2(static_cast<float>(re) * vs, static_cast<float>(im) * vs);
+}
+
+template <int FMT>
+__device__ __forceinline__ float2 pair_volt(const void* volt, size_t idx, float vs) {
+  if constexpr (FMT == 0) {
+    return unpack_ci4(__ldg(static_cast<const unsigned char*>(volt) + idx), vs);
+  } else {
+    const float2 e = __ldg(static_cast<const float2*>(volt) + idx);
+    return make_float2(e.x * vs, e.y * vs);
+  }
+}
+
+// Gridding of one frame pair: slices of 32 cells, one cell per lane.
+template <int BT>
+__device__ __forceinline__ void grid_pair(const int* __restrict__ cell, const int2* __restrict__ slice,
+                                          const uint2* __restrict__ ent, int nslice, const Cf2* Es, Cf2* grid) {
+  const int lane = threadIdx.x & 31;
+  for (int sl = threadIdx.x >> 5; sl < nslice; sl += BT / 32) {
+    const int2 s = slice[sl];
+    const int at = cell[sl * 32 + lane];
+    const uint2* e = ent + s.x + lane;
+    Cf2 sum{0ull, 0ull};
+#pragma unroll 2
+    for (int k = 0; k < s.y; ++k) {
+      const uint2 en = e[k * 32];
+      const Cf2 x = *reinterpret_cast<const Cf2*>(reinterpret_cast<const unsigned char*>(Es) + en.x);
+      const f32x2 w = f2_splat(__uint_as_float(en.y));
+      sum.re = f2_fma(w, x.re, sum.re);
+      sum.im = f2_fma(w, x.im, sum.im);
+    }
+    if (at >= 0) grid[at] = sum;
+  }
+}
+
+// |E|^2 of the 16 outputs of a column task, both frames, into the running
+// sums (one rounding of a sum per pair).
+__device__ __forceinline__ void square_add(const Cf2 (&y)[16], float (&acc)[16]) {
+#pragma unroll
+  for (int m = 0; m < 16; ++m) {
+    const float2 re = f2_unpack(y[m].re), im = f2_unpack(y[m].im);
+    acc[m] += fmaf(re.x, re.x, fmaf(im.x, im.x, fmaf(re.y, re.y, im.y * im.y)));
+  }
+}
+
+// Output slot `slot` of both frames times the phase ph.
+__device__ __forceinline__ void store_pixel(const Cf2 (&y)[16], int slot, float2 ph, float2* p0, float2* p1) {
+#pragma unroll
+  for (int m = 0; m < 16; ++m)
+    if (m == slot) {
+      const float2 re = f2_unpack(y[m].re), im = f2_unpack(y[m].im);
+      *p0 = cmul(make_float2(re.x, im.x), ph);
+      if (p1) *p1 = cmul(make_float2(re.y, im.y), ph);
+    }
+}
+
+// Multiple-pixel EPICal: the calibration pixels among a thread's outputs
+// (slot mask, index of its first tap) of frame pair p.
+__device__ __forceinline__ void store_taps(const ImageArgs& A, const Cf2 (&y)[16], int entry, long long p, int c) {
+  const uint2 tb = __ldg(A.ptab + entry);
+  if (!tb.x) return;
+  float2* d0 = A.ptap + (static_cast<size_t>(2 * p) * A.n_chan + c) * A.npix;
+  float2* d1 = 2 * p + 1 < A.n_time ? d0 + static_cast<size_t>(A.n_chan) * A.npix : nullptr;
+  const float2* ph = A.pph + static_cast<size_t>(c) * A.npix;
+#pragma unroll
+  for (int m = 0; m < 16; ++m)
+    if ((tb.x >> m) & 1u) {
+      const int pi = static_cast<int>(tb.y) + __popc(tb.x & ((1u << m) - 1u));
+      store_pixel(y, m, __ldg(ph + pi), d0 + pi, d1 ? d1 + pi : nullptr);
+    }
+}
+
+// Bring the voltages of frame pair p of channel c into L1.
+template <int FMT, int BT>
+__device__ __forceinline__ void prefetch_pair(const ImageArgs& A, long long p, int c) {
+  constexpr int esz = FMT == 0 ? 1 : 8;
+  const size_t bytes = static_cast<size_t>(A.n_ant) * esz;
+#pragma unroll
+  for (int f = 0; f < 2; ++f)
+    if (2 * p + f < A.n_time) {
+      const uintptr_t b0 = reinterpret_cast<uintptr_t>(A.volt) +
+                           (static_cast<size_t>(2 * p + f) * A.n_chan + c) * bytes;
+      for (uintptr_t q = (b0 & ~static_cast<uintptr_t>(127)) + static_cast<uintptr_t>(threadIdx.x) * 128; q < b0 + bytes;
+           q += BT * 128)
+        asm volatile("prefetch.global.L1 [%0];" ::"l"(q));
+    }
+}
+
+// The share of one CTA in the cost of all (channel, frame pair)s: positions
+// [lo, hi) of the list of channels, cost[c + 1] - cost[c] per pair.
+struct Share {
+  long long lo, hi, pairs;
+  const int* cost;
+  __device__ __forceinline__ Share(const ImageArgs& A) : pairs((A.n_time + 1) / 2), cost(A.pcost) {
+    const long long total = static_cast<long long>(__ldg(cost + A.n_chan)) * pairs, g = gridDim.x, b = blockIdx.x;
+    lo = total / g * b + total % g * b / g;
+    hi = total / g * (b + 1) + total % g * (b + 1) / g;
+  }
+  __device__ __forceinline__ long long before(int c) const { return static_cast<long long>(__ldg(cost + c)) * pairs; }
+  // first pair of channel c at or after position pos
+  __device__ __forceinline__ long long pair_at(long long pos, int c) const {
+    const long long w = __ldg(cost + c + 1) - __ldg(cost + c);
+    const long long p = (pos - before(c) + w - 1) / w;
+    return p < 0 ? 0 : (p > pairs ? pairs : p);
+  }
+};
+
+// A channel's tables and geometry, its tap lists in shared memory (TS) or
+// read through L1.
+struct Chan {
+  int R, R4, W4, nslice;
+  const int2* slice;
+  const int* cell;
+  const uint2* ent;
+  float vs;
+  float2 pph;
+  const float2* wg;
+};
+
+template <bool TS>
+__device__ __forceinline__ Chan channel(const ImageArgs& A, int c, const int2* sslice, const int* scell,
+                                        const uint2* sent) {
+  Chan q;
+  const int4 wn = __ldg(A.win4 + c);                       // (y0, rows, x0, cols)
+  q.R = wn.y;
+  q.R4 = (wn.y + 3) & ~3;
+  q.W4 = (wn.w + 3) & ~3;
+  const int sb = __ldg(A.psbase + c), eb = __ldg(A.pebase + c);
+  q.nslice = __ldg(A.psbase + c + 1) - sb;
+  q.slice = TS ? sslice : A.pslice + sb;
+  q.cell = TS ? scell : A.pcell + static_cast<size_t>(sb) * 32;
+  q.ent = TS ? sent : A.pent + eb;
+  q.vs = A.vscale ? __ldg(A.vscale + c) : 1.0f;
+  q.pph = A.do_cal ? __ldg(A.pixph + c) : make_float2(1.f, 0.f);
+  q.wg = A.wgain + static_cast<size_t>(c) * A.n_ant;
+  return q;
+}
+
+template <int BT>
+__device__ __forceinline__ void load_lists(const ImageArgs& A, int c, int2* sslice, int* scell, uint2* sent) {
+  const int sb = __ldg(A.psbase + c), eb = __ldg(A.pebase + c);
+  const int ns = __ldg(A.psbase + c + 1) - sb, ne = __ldg(A.pebase + c + 1) - eb;
+  for (int i = threadIdx.x; i < ns; i += BT) sslice[i] = __ldg(A.pslice + sb + i);
+  for (int i = threadIdx.x; i < ns * 32; i += BT) scell[i] = __ldg(A.pcell + static_cast<size_t>(sb) * 32 + i);
+  for (int i = threadIdx.x; i < ne; i += BT) sent[i] = __ldg(A.pent + eb + i);
+}
+
+// One antenna's EPICal sums over a run (FP32; FP64 across runs).
+struct Corr {
+  float2 k;
+  float p;
+  __device__ __forceinline__ void add(float2 e, float2 q) {
+    k.x += e.x * q.x + e.y * q.y;
+    k.y += e.y * q.x - e.x * q.y;
+    p += e.x * e.x + e.y * e.y;
+  }
+  __device__ __forceinline__ void flush(const ImageArgs& A, int c, int a) const {
+    const size_t o = static_cast<size_t>(c) * A.n_ant + a;
+    if (__ldg(A.cellf + o) < 0) return;
+    atomicAdd(&A.kacc[o].x, static_cast<double>(k.x));
+    atomicAdd(&A.kacc[o].y, static_cast<double>(k.y));
+    atomicAdd(A.pacc + o, static_cast<double>(p));
+  }
+};
+
+template <int N> struct PCfg;
+template <> struct PCfg<16>  { static constexpr int BT = 32,  PER_SM = 8; };
+template <> struct PCfg<32>  { static constexpr int BT = 64,  PER_SM = 8; };
+template <> struct PCfg<64>  { static constexpr int BT = 256, PER_SM = 2; };
+template <> struct PCfg<128> { static constexpr int BT = 512, PER_SM = 1; };
+
+template <int N>
+struct PGeo {
+  static constexpr int BT = PCfg<N>::BT;
+  static constexpr int NR = N / 16;                  // residues = lanes per transform
+  static constexpr int TASKS = N * NR;               // column tasks
+  static constexpr int ROUNDS = TASKS < BT ? 1 : TASKS / BT;
+  static_assert(TASKS < BT || TASKS % BT == 0, "column tasks must fill the CTA");
+};
+
+// Two phases per frame pair, a CTA barrier after each:
+//   rows      tasks (grid row, r): grid -> spectra; the last warps also
+//             correlate the previous pair with the calibrator pixel (Eqs. 12,
+//             15) and form E' of the next pair (Eq. 8);
+//   columns   tasks (column kx, r): spectra -> |E|^2 in registers (Eq. 10),
+//             calibrator pixel stored; then the next pair is gridded.
+template <int N, int FMT, int MAXA, bool TS>
+__global__ void __launch_bounds__(PCfg<N>::BT, PCfg<N>::PER_SM) epic_image_pair(const ImageArgs A) {
+  using G = PGeo<N>;
+  constexpr int BT = G::BT, NR = G::NR, TASKS = G::TASKS, ROUNDS = G::ROUNDS;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int rs = A.rs, gs = A.gs, Na = A.n_ant;
+  Cf2* Tt = reinterpret_cast<Cf2*>(smem_raw);              // [N][rs] row spectra, transposed
+  Cf2* grid = Tt + N * rs;                                 // [rows_alloc][gs]
+  Cf2* Es = grid + A.rows_alloc * gs;                      // [Na + 1] E' (entry Na is zero)
+  float2* tw = reinterpret_cast<float2*>(Es + Na + 1);     // [16][NR]
+  float2* wq = tw + N;                                     // [16][NR]
+  float2* pixs = wq + N;                                   // [2] calibrator pixel of the pair
+  int2* sslice = reinterpret_cast<int2*>(pixs + 2);        // [max_slices] (TS)
+  uint2* sent = reinterpret_cast<uint2*>(sslice + A.max_slices);   // [max_ent] (TS)
+  int* scell = reinterpret_cast<int*>(sent + A.max_ent);   // [max_slices * 32] (TS)
+
+  const int tid = threadIdx.x;
+  const int aw = (BT - 32 - (tid & ~31)) + (tid & 31);     // antenna of this thread: the last warps first
+  for (int i = tid; i < N; i += BT) {
+    const int n = i / NR, r = i % NR;                      // also (q, r) of wq
+    tw[i] = A.twid[(n * r) & (N - 1)];
+    wq[i] = A.twid[(16 * n * r) & (N - 1)];
+  }
+  if (tid == 0) Es[Na] = Cf2{0ull, 0ull};
+
+  const long long T = A.n_time;
+  const int C = A.n_chan;
+  const Share share(A);
+  int c = 0;
+  while (c < C && share.before(c + 1) <= share.lo) ++c;
+  int cur = -1;
+  for (; c < C && share.before(c) < share.hi; ++c) {
+    const long long p_lo = share.pair_at(share.lo, c), p_hi = share.pair_at(share.hi, c);
+    const Chan ch = channel<TS>(A, c, sslice, scell, sent);
+    for (long long pa = p_lo; pa < p_hi; pa += kPairRun) {
+      const long long pb = pa + kPairRun < p_hi ? pa + kPairRun : p_hi;
+      __syncthreads();                                     // the previous run's shared memory is free
+      if (cur != c) {
+        if (TS) load_lists<BT>(A, c, sslice, scell, sent);
+        for (int i = tid; i < A.rows_alloc * gs; i += BT) grid[i] = Cf2{0ull, 0ull};   // cells without taps stay zero
+        const int pad = ch.R4 - ch.R;
+        for (int i = tid; i < N * pad; i += BT) Tt[(i / pad) * rs + ch.R + i % pad] = Cf2{0ull, 0ull};
+        cur = c;
+      }
+      Corr corr[MAXA];
+      unsigned hist[MAXA];                                 // 4-bit voltages of the last two pairs, 16 bits each
+#pragma unroll
+      for (int i = 0; i < MAXA; ++i) {
+        corr[i] = Corr{make_float2(0.f, 0.f), 0.f};
+        hist[i] = 0;
+      }
+      // E' of pair p (a missing second frame is zero)
+      auto form_e = [&](long long p) {
+#pragma unroll
+        for (int i = 0; i < MAXA; ++i) {
+          const int a = aw + BT * i;
+          hist[i] <<= 16;
+          if (a < Na && p < pb) {
+            const size_t idx = (static_cast<size_t>(2 * p) * C + c) * Na + a, next = static_cast<size_t>(C) * Na;
+            const bool two = 2 * p + 1 < T;
+            const float2 w = __ldg(ch.wg + a);
+            float2 v0, v1 = make_float2(0.f, 0.f);
+            if (FMT == 0) {
+              const unsigned char* v = static_cast<const unsigned char*>(A.volt) + idx;
+              const unsigned b = __ldg(v) | (two ? static_cast<unsigned>(__ldg(v + next)) << 8 : 0u);
+              hist[i] |= b;
+              v0 = unpack_ci4(b, ch.vs);
+              v1 = unpack_ci4(b >> 8, ch.vs);
+            } else {
+              v0 = pair_volt<FMT>(A.volt, idx, ch.vs);
+              if (two) v1 = pair_volt<FMT>(A.volt, idx + next, ch.vs);
+            }
+            const float2 e0 = cmul(v0, w), e1 = cmul(v1, w);
+            Es[a] = Cf2{f2_pack(e0.x, e1.x), f2_pack(e0.y, e1.y)};
+          }
+        }
+      };
+      // correlation of pair p, the last but one formed, with the calibrator
+      // pixel (Eqs. 12, 15); a missing second frame adds zero
+      auto correlate = [&](long long p) {
+#pragma unroll
+        for (int i = 0; i < MAXA; ++i) {
+          const int a = aw + BT * i;
+          if (a < Na) {
+#pragma unroll
+            for (int f = 0; f < 2; ++f) {
+              if (FMT == 0)
+                corr[i].add(unpack_ci4(hist[i] >> (16 + 8 * f), ch.vs), pixs[f]);
+              else if (2 * p + f < T)
+                corr[i].add(pair_volt<FMT>(A.volt, (static_cast<size_t>(2 * p + f) * C + c) * Na + a, ch.vs), pixs[f]);
+            }
+          }
+        }
+      };
+      float acc[ROUNDS][16];
+#pragma unroll
+      for (int i = 0; i < ROUNDS; ++i)
+#pragma unroll
+        for (int m = 0; m < 16; ++m) acc[i][m] = 0.f;
+
+      form_e(pa);
+      __syncthreads();
+      grid_pair<BT>(ch.cell, ch.slice, ch.ent, ch.nslice, Es, grid);
+      __syncthreads();
+      for (long long p = pa; p < pb; ++p) {
+        if (p + 2 < pb) prefetch_pair<FMT, BT>(A, p + 2, c);
+        // ---- rows ----
+        for (int task = tid; task < ch.R * NR; task += BT) {
+          const int row = task / NR, r = task % NR;
+          Cf2 y[16];
+          dft_task<NR>(grid + row * gs, ch.W4, r, tw, wq, y);
+#pragma unroll
+          for (int m = 0; m < 16; ++m) Tt[(NR * m + r) * rs + row] = y[m];
+        }
+        if (A.do_cal && p > pa) correlate(p - 1);
+        form_e(p + 1);
+        __syncthreads();
+        // ---- columns ----
+#pragma unroll
+        for (int i = 0; i < ROUNDS; ++i) {
+          const int task = tid + BT * i;
+          if (TASKS >= BT || task < TASKS) {
+            const int kx = task / NR, r = task % NR;
+            Cf2 y[16];
+            dft_task<NR>(Tt + kx * rs, ch.R4, r, tw, wq, y);
+            square_add(y, acc[i]);
+            if (A.do_cal && kx == A.k0x && r == A.k0y % NR) store_pixel(y, A.k0y / NR, ch.pph, pixs, pixs + 1);
+            if (A.npix) store_taps(A, y, task, p, c);
+          }
+        }
+        if (p + 1 < pb) grid_pair<BT>(ch.cell, ch.slice, ch.ent, ch.nslice, Es, grid);
+        __syncthreads();
+      }
+      if (A.do_cal) correlate(pb - 1);
+
+      // flush the run's partial sums (FP32 over the run, FP64 across)
+      double* img = A.image + static_cast<size_t>(c) * N * N;
+#pragma unroll
+      for (int i = 0; i < ROUNDS; ++i) {
+        const int task = tid + BT * i;
+        if (TASKS >= BT || task < TASKS) {
+          const int kx = task / NR, r = task % NR;
+#pragma unroll
+          for (int m = 0; m < 16; ++m)
+            atomicAdd(img + (NR * m + r) * N + kx, static_cast<double>(acc[i][m]) * A.img_scale);
+        }
+      }
+      if (A.do_cal) {
+#pragma unroll
+        for (int i = 0; i < MAXA; ++i)
+          if (aw + BT * i < Na) corr[i].flush(A, c, aw + BT * i);
+      }
+    }
+  }
+}
+
+using PairKernel = void (*)(const ImageArgs);
+
+template <int N, int FMT>
+PairKernel pair_kernel_nf(bool many, bool table) {
+  if (many) return table ? epic_image_pair<N, FMT, kPairMaxAnt, true> : epic_image_pair<N, FMT, kPairMaxAnt, false>;
+  return table ? epic_image_pair<N, FMT, 1, true> : epic_image_pair<N, FMT, 1, false>;
+}
+
+template <int N>
+PairKernel pair_kernel_n(int fmt, bool many, bool table) {
+  return fmt ? pair_kernel_nf<N, 1>(many, table) : pair_kernel_nf<N, 0>(many, table);
+}
+
+PairKernel pair_kernel(int n, int fmt, bool many, bool table) {
+  switch (n) {
+    case 16: return pair_kernel_n<16>(fmt, many, table);
+    case 32: return pair_kernel_n<32>(fmt, many, table);
+    case 64: return pair_kernel_n<64>(fmt, many, table);
+    case 128: return pair_kernel_n<128>(fmt, many, table);
+    default: return nullptr;
+  }
+}
+
+}  // namespace
+
+int pair_threads(int n) {
+  switch (n) {
+    case 16: return PCfg<16>::BT;
+    case 32: return PCfg<32>::BT;
+    case 64: return PCfg<64>::BT;
+    case 128: return PCfg<128>::BT;
+    default: return 0;
+  }
+}
+
+int pair_col_rounds(int n) {
+  const int bt = pair_threads(n);
+  if (!bt) return 0;
+  const int tasks = n * n / 16;
+  return tasks < bt ? 1 : tasks / bt;
+}
+
+bool pair_pixel_owner(int n, int kx, int ky, PixelOwner* out) {
+  const int bt = pair_threads(n);
+  if (!bt || kx < 0 || ky < 0 || kx >= n || ky >= n) return false;
+  const int nr = n / 16, task = kx * nr + ky % nr;
+  out->round = task / bt;
+  out->thread = task % bt;
+  out->slot = ky / nr;
+  return true;
+}
+
+// Row stride of the spectra: room for the rows rounded up to 4, and a
+// stride that keeps the row phase's stores free of bank conflicts (a quarter
+// warp stores NR columns of 8 / NR neighbouring rows, 16 bytes each).
+int pair_rs(int n, int rows) {
+  const int nr = n / 16;
+  int rs = (rows + 3) & ~3;
+  const int step = 8 / nr;                       // rows per quarter warp
+  while (!(nr == 1 || (rs % step == 0 && (rs / step) % 2 == 1))) ++rs;
+  return rs;
+}
+
+size_t pair_smem_bytes(int n, int n_ant, int rows, int gs, int max_slices, int max_ent) {
+  const size_t cells = static_cast<size_t>(n) * pair_rs(n, rows) + static_cast<size_t>(rows) * gs + n_ant + 1;
+  return cells * 16 + (2 * static_cast<size_t>(n) + 2) * sizeof(float2) +
+         static_cast<size_t>(max_slices) * (sizeof(int2) + 32 * sizeof(int)) +
+         static_cast<size_t>(max_ent) * sizeof(uint2);
+}
+
+cudaError_t pair_prepare(int n, int n_ant, bool table, size_t smem, int* ctas_per_sm) {
+  // the attribute belongs to the kernel, not to a plan: always the device's
+  // limit, so that plans of different footprints can live side by side
+  int dev = 0, most = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  const int bt = pair_threads(n);
+  for (int fmt = 0; fmt < 2; ++fmt) {
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(pair_kernel(n, fmt, n_ant > bt, table), cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  }
+  if (e != cudaSuccess) return e;
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, pair_kernel(n, 0, n_ant > bt, table), bt, smem);
+}
+
+cudaError_t launch_pair(int n, const ImageArgs& a, cudaStream_t s) {
+  const int bt = pair_threads(n);
+  const PairKernel k = pair_kernel(n, a.input_fmt, a.n_ant > bt, a.gsmem != 0);
+  if (!k) return cudaErrorInvalidValue;
+  k<<<a.grid, bt, a.smem, s>>>(a);
+  return cudaGetLastError();
+}
+
+}  // namespace epic

@@ -127,6 +127,13 @@ struct epic_plan_s {
   int gsmem = 0;                // fused gather table held in shared memory
   bool piped = false;           // fused path in its warp-specialised form
   int steps = 1;                // fused form: frames per step
+  bool pair = false;            // fused path in its frame-pair form
+  int gs = 0;                   // frame-pair form: row stride of the grid, 16-byte cells
+  int max_slices = 0, max_ent = 0;   // most slices / entries of one channel
+  DevBuf<int> d_pcell;          // frame-pair gridding: grid cell of each list, 32 per slice
+  DevBuf<int2> d_pslice;        // (first entry, taps) of each slice
+  DevBuf<uint2> d_pent;         // entries (byte offset of E'_a, weight bits)
+  DevBuf<int> d_psbase, d_pebase, d_pcost;   // [C + 1] first slice / first entry / cost prefix
   DevBuf<float2> d_pixph;       // [C] calibrator-pixel phase in window coordinates
   std::vector<int> x0, cols;    // [C] first occupied column, occupied columns
   int rs_fused = 0;
@@ -403,7 +410,128 @@ epic_status build_gather(epic_plan_t p, const std::vector<float>& wts, int N1, b
   return EPIC_OK;
 }
 
-// Arguments of one fused launch over a device batch.// Arguments of one fused launch over a device batch.
+// Gridding of Eq. 9 as one tap list per occupied grid cell (frame-pair
+// form): the cells of a channel sorted by their number of taps, most first,
+// in slices of 32 (one per lane) as long as their longest list; entry k of
+// the slice's lanes is contiguous.  Shorter lists and lanes without a cell
+// read the zero voltage behind the last antenna with weight 0.
+struct CellTables {
+  std::vector<int> cell, sbase, ebase, cost;
+  std::vector<int2> slice;
+  std::vector<uint2> ent;
+  int max_slices = 0, max_ent = 0;
+};
+
+void build_cells(const epic_plan_s* p, const std::vector<float>& wts, int gs, CellTables* t) {
+  const int C = p->nc, Na = p->na, N = p->n, K = p->k, KK = K * K, h = (K - 1) / 2;
+  std::vector<int> count, order, place, start, sorted;
+  std::vector<unsigned char> bank;         // 16-byte bank of a cell's first antenna
+  for (int c = 0; c < C; ++c) {
+    t->sbase.push_back(static_cast<int>(t->slice.size()));
+    t->ebase.push_back(static_cast<int>(t->ent.size()));
+    const int R = p->rows[c];
+    count.assign(static_cast<size_t>(R) * gs, 0);
+    bank.assign(count.size(), 0);
+    auto each_tap = [&](auto&& f) {
+      for (int a = 0; a < Na; ++a) {
+        if (p->flags[a]) continue;
+        const size_t ob = (static_cast<size_t>(c) * Na + a) * 2;
+        const int r0 = p->base[ob + 1] - h - p->y0[c], x0 = p->base[ob] - h - p->x0[c];
+        const float* wf = &wts[(static_cast<size_t>(c) * Na + a) * KK];
+        for (int dy = 0; dy < K; ++dy)
+          for (int dx = 0; dx < K; ++dx)
+            if (wf[dy * K + dx] != 0.0f) f(a, (r0 + dy) * gs + x0 + dx, wf[dy * K + dx]);
+      }
+    };
+    int most = 0;
+    long long taps = 0;
+    each_tap([&](int a, int cell, float) {
+      if (!count[cell]) bank[cell] = static_cast<unsigned char>(a % 8);
+      most = std::max(most, ++count[cell]);
+      ++taps;
+    });
+    // counting sort of the occupied cells, most taps first
+    start.assign(most + 2, 0);
+    for (int n : count) ++start[most - n];
+    int cells = 0;
+    for (int i = 0; i < most; ++i) {
+      const int n = start[i];
+      start[i] = cells;
+      cells += n;
+    }
+    sorted.assign(cells, 0);
+    for (size_t i = 0; i < count.size(); ++i)
+      if (count[i]) sorted[start[most - count[i]]++] = static_cast<int>(i);
+    // cells of equal length taken in turn from the 8 banks
+    order.clear();
+    for (int lo = 0; lo < cells;) {
+      int hi = lo;
+      std::vector<int> by[8];
+      for (; hi < cells && count[sorted[hi]] == count[sorted[lo]]; ++hi) by[bank[sorted[hi]]].push_back(sorted[hi]);
+      for (size_t k = 0; order.size() < static_cast<size_t>(hi); ++k)
+        for (const auto& b : by)
+          if (k < b.size()) order.push_back(b[k]);
+      lo = hi;
+    }
+    place.assign(count.size(), -1);
+    for (int i = 0; i < cells; ++i) place[order[i]] = i;
+    const int slices = (cells + 31) / 32;
+    const size_t s0 = t->slice.size(), e0 = t->ent.size();
+    int ne = 0;
+    for (int s = 0; s < slices; ++s) {
+      const int m = count[order[32 * s]];
+      t->slice.push_back(make_int2(ne, m));
+      ne += 32 * m;
+    }
+    t->cell.resize((s0 + slices) * 32, -1);
+    for (int i = 0; i < cells; ++i) t->cell[s0 * 32 + i] = order[i];
+    t->ent.resize(e0 + ne, make_uint2(static_cast<unsigned>(Na) * 16u, 0u));
+    std::fill(count.begin(), count.end(), 0);
+    each_tap([&](int a, int cell, float w) {
+      const int i = place[cell];
+      uint2& q = t->ent[e0 + t->slice[s0 + i / 32].x + static_cast<size_t>(count[cell]++) * 32 + i % 32];
+      q.x = static_cast<unsigned>(a) * 16u;
+      std::memcpy(&q.y, &w, sizeof w);
+    });
+    // the order of a list's taps is free: let the 8 lanes of a quarter warp
+    // read different 16-byte banks of E' at each step where they can
+    for (int i = 0; i < slices * 32; i += 8) {
+      const int2 sl = t->slice[s0 + i / 32];
+      for (int k = 0; k < sl.y; ++k) {
+        unsigned used = 0;
+        for (int l = i; l < i + 8 && l < cells; ++l) {
+          uint2* e = &t->ent[e0 + sl.x + l % 32];
+          const int n = count[order[l]];
+          for (int m = k; m < n; ++m)
+            if (!((used >> (e[static_cast<size_t>(m) * 32].x / 16 % 8)) & 1u)) {
+              std::swap(e[static_cast<size_t>(m) * 32], e[static_cast<size_t>(k) * 32]);
+              break;
+            }
+          if (k < n) used |= 1u << (e[static_cast<size_t>(k) * 32].x / 16 % 8);
+        }
+      }
+    }
+    t->max_slices = std::max(t->max_slices, slices);
+    t->max_ent = std::max(t->max_ent, ne);
+    // cost of one frame pair, in packed FP32 instructions of a thread: a
+    // transform task of length L is about 290 + 5 (L - 16); a tap 12
+    const auto task = [](int L) { return 290 + 5 * std::max(0, ((L + 3) & ~3) - 16); };
+    const long long work = static_cast<long long>(N) * (N / 16) * task(R) +
+                           static_cast<long long>(R) * (N / 16) * task(p->cols[c]) + 12 * taps + 20 * Na;
+    t->cost.push_back(static_cast<int>(std::max<long long>(1, work / 256)));
+  }
+  t->sbase.push_back(static_cast<int>(t->slice.size()));
+  t->ebase.push_back(static_cast<int>(t->ent.size()));
+  int sum = 0;
+  for (int& v : t->cost) {
+    const int w = v;
+    v = sum;
+    sum += w;
+  }
+  t->cost.push_back(sum);
+}
+
+// Arguments of one fused launch over a device batch.
 epic::ImageArgs fused_args(epic_plan_t p, const void* d_volt, long long n_time, double* d_image,
                            double img_scale) {
   epic::ImageArgs a{};
@@ -446,6 +574,22 @@ epic::ImageArgs fused_args(epic_plan_t p, const void* d_volt, long long n_time, 
   a.smem = p->smem;
   a.npix = 0;                              // epic_image arms the pixel taps itself
   a.wait_limit = p->wait_limit;
+  if (p->pair) {
+    a.pair = 1;
+    a.pcell = p->d_pcell.p;
+    a.pslice = p->d_pslice.p;
+    a.pent = p->d_pent.p;
+    a.psbase = p->d_psbase.p;
+    a.pebase = p->d_pebase.p;
+    a.pcost = p->d_pcost.p;
+    a.gs = p->gs;
+    a.max_slices = p->max_slices;
+    a.max_ent = p->max_ent;
+    a.rs = epic::pair_rs(p->n, p->rows_alloc);
+    // at least tune_units frame pairs per CTA
+    const long long pairs = static_cast<long long>(p->nc) * ((n_time + 1) / 2);
+    a.grid = static_cast<int>(std::max<long long>(1, std::min<long long>(pairs / p->tune_units, p->ctas)));
+  }
   return a;
 }
 
@@ -858,7 +1002,8 @@ epic_status build_grid_tables(epic_plan_s* p, std::vector<int>& cell0, std::vect
 // FP16/BF16, else the fused kernel's frames per step and gather-table
 // placement (or the warp-specialised form), the cluster form when asked
 // for, else the plain unfused path; CTAs per launch.
-epic_status choose_path(epic_plan_s* p, const epic_plan_desc* d, bool fused_shape, bool unfused_ok) {
+epic_status choose_path(epic_plan_s* p, const epic_plan_desc* d, bool fused_shape, bool unfused_ok,
+                        const std::vector<float>& wts, CellTables* cells) {
   const int Na = p->na, N = p->n, KK = p->k * p->k;
   p->rs = epic::image_rs(p->rows_alloc);
   int dev = 0;
@@ -897,7 +1042,25 @@ epic_status choose_path(epic_plan_s* p, const epic_plan_desc* d, bool fused_shap
   }
   if (d->path == EPIC_PATH_PIPED && !p->piped)
     return fail(EPIC_ERR_UNSUPPORTED, "warp-specialised fused path: array footprint exceeds shared memory");
-  if (fused && !p->piped) {
+  if (fused && d->path != EPIC_PATH_PIPED) {
+    // frame-pair form: grid, spectra and E' of one pair in shared memory,
+    // with the tap lists beside them when they fit, else read through L1
+    const int W4 = (*std::max_element(p->cols.begin(), p->cols.end()) + 3) & ~3;
+    p->gs = W4 + 1;                          // odd: neighbouring rows in different banks
+    const size_t s0 = epic::pair_smem_bytes(N, Na, p->rows_alloc, p->gs, 0, 0);
+    if (Na <= epic::kPairMaxAnt * epic::pair_threads(N) && s0 <= static_cast<size_t>(smem_optin)) {
+      build_cells(p, wts, p->gs, cells);
+      const size_t s1 = epic::pair_smem_bytes(N, Na, p->rows_alloc, p->gs, cells->max_slices, cells->max_ent);
+      p->gsmem = s1 <= static_cast<size_t>(smem_optin) ? 1 : 0;
+      if (p->gsmem) {
+        p->max_slices = cells->max_slices;
+        p->max_ent = cells->max_ent;
+      }
+      p->smem = p->gsmem ? s1 : s0;
+      p->pair = true;
+    }
+  }
+  if (fused && !p->piped && !p->pair) {
     // shape preference: two frames per step, then one; the gather table in
     // shared memory when it fits (entries per channel <= Na K^2 taps), else
     // read through L1
@@ -955,6 +1118,7 @@ epic_status choose_path(epic_plan_s* p, const epic_plan_desc* d, bool fused_shap
   } else if (fused) {
     int per_sm = 0;
     e = p->piped ? epic::piped_prepare(N, p->smem, p->gsmem != 0, &per_sm)
+        : p->pair ? epic::pair_prepare(N, Na, p->gsmem != 0, p->smem, &per_sm)
                  : epic::image_kernel_prepare(N, p->smem, Na, p->steps, &per_sm);
     if (e != cudaSuccess || per_sm < 1)
       return e != cudaSuccess ? cuda_fail(e, "image kernel attributes")
@@ -1052,7 +1216,8 @@ epic_status epic_plan_create(epic_plan_t* out, const epic_plan_desc* d) {
   const int Na = p->na, C = p->nc, N = p->n, K = p->k, h = (K - 1) / 2;
 
   // ---- launch shape ----
-  if (epic_status st = choose_path(p, d, fused_shape, unfused_ok)) {
+  CellTables cells;
+  if (epic_status st = choose_path(p, d, fused_shape, unfused_ok, wts, &cells)) {
     delete p;
     return st;
   }
@@ -1082,7 +1247,7 @@ epic_status epic_plan_create(epic_plan_t* out, const epic_plan_desc* d) {
   std::vector<int> gofs, gbase, ugofs, ugbase;
   std::vector<uint4> gcnt, ugcnt;
   std::vector<uint2> gent, ugent;
-  if (p->path == EPIC_PATH_FUSED || p->path == EPIC_PATH_UNFUSED) {
+  if ((p->path == EPIC_PATH_FUSED && !p->pair) || p->path == EPIC_PATH_UNFUSED) {
     const int n1 = p->path == EPIC_PATH_FUSED ? epic::image_fft_lanes(N) : epic::unfused_fft_lanes(N);
     if (epic_status st = build_gather(p, wts, n1, true, gofs, gcnt, gent, gbase)) {
       epic_plan_destroy(p);
@@ -1116,7 +1281,9 @@ epic_status epic_plan_create(epic_plan_t* out, const epic_plan_desc* d) {
                       up(p->d_order, order), up(p->d_ranges, ranges), up(p->d_gofs, gofs),
                       up(p->d_gent, gent), up(p->d_gbase, gbase), up(p->d_gcnt, gcnt),
                       up(p->d_ugofs, ugofs), up(p->d_ugcnt, ugcnt), up(p->d_ugent, ugent),
-                      up(p->d_ugbase, ugbase)};
+                      up(p->d_ugbase, ugbase), up(p->d_pcell, cells.cell), up(p->d_pslice, cells.slice),
+                      up(p->d_pent, cells.ent), up(p->d_psbase, cells.sbase), up(p->d_pebase, cells.ebase),
+                      up(p->d_pcost, cells.cost)};
   for (cudaError_t x : es)
     if (x != cudaSuccess) {
       epic_plan_destroy(p);
@@ -1191,6 +1358,12 @@ epic_status epic_plan_destroy(epic_plan_t p) {
   p->d_xe_z.release();
   p->d_phase.release();
   p->d_bx.release();
+  p->d_pcell.release();
+  p->d_pslice.release();
+  p->d_pent.release();
+  p->d_psbase.release();
+  p->d_pebase.release();
+  p->d_pcost.release();
   p->d_uv.release();
   p->d_iters.release();
   if (p->graph_exec) cudaGraphExecDestroy(p->graph_exec);
@@ -1509,9 +1682,10 @@ epic_status epical_configure_pixels(epic_plan_t p, int n_pix, const double* pix_
   if (p->path != EPIC_PATH_FUSED || p->piped || p->precision != EPIC_PREC_FP32)
     return fail(EPIC_ERR_UNSUPPORTED, "multiple-pixel EPICal needs the fused FP32 path (N <= 128)");
   const int Na = p->na, C = p->nc, N = p->n;
-  const int rounds = epic::image_col_rounds(N);
+  const int rounds = p->pair ? epic::pair_col_rounds(N) : epic::image_col_rounds(N);
   epic::ImageKernelShape sh{};
   epic::image_kernel_shape(N, &sh);
+  if (p->pair) sh.threads = epic::pair_threads(N);
   // owner of every pixel; taps ordered by (round, thread, slot) so that a
   // thread's taps of one round are consecutive
   struct Tap { int round, thread, slot, user, kx, ky; };
@@ -1521,7 +1695,7 @@ epic_status epical_configure_pixels(epic_plan_t p, int n_pix, const double* pix_
     if (!nearest_pixel(p, pix_lm[2 * i], pix_lm[2 * i + 1], &kx, &ky))
       return fail(EPIC_ERR_INVALID_ARG, "calibration pixel outside the image");
     epic::PixelOwner o{};
-    if (!epic::image_pixel_owner(N, kx, ky, &o)) return fail(EPIC_ERR_UNSUPPORTED, "grid size");
+    if (!(p->pair ? epic::pair_pixel_owner(N, kx, ky, &o) : epic::image_pixel_owner(N, kx, ky, &o))) return fail(EPIC_ERR_UNSUPPORTED, "grid size");
     taps[i] = {o.round, o.thread, o.slot, i, kx, ky};
   }
   std::sort(taps.begin(), taps.end(), [](const Tap& x, const Tap& y) {
