@@ -303,6 +303,26 @@ struct UnfusedArgs {
 bool persistent_supported(int n);
 cudaError_t launch_unfused_persistent(const UnfusedArgs& a, long long n_time, int nt_batch, unsigned* bar, int sms,
                                       cudaStream_t s);
+// Frame-pair form of the plain path (N = 256, 512), epic_wide.cu.
+struct WideArgs {
+  UnfusedArgs u;           // spec: [pair][nc][N][rs] 16-byte frame pairs; gather tables unused
+  int c0, nc;              // channels of this launch
+  const int4* win4;        // [C] (y0, rows, x0, cols)
+  const unsigned char* lists;   // row blocks' tap lists
+  const int2* lists_at;    // [C][nb_max] (offset, bytes) / 16 of each block's lists
+  int nb_max, max_lists;   // most blocks of a channel, most bytes of one block's lists
+  int gs;                  // row stride of the grid block (16-byte cells)
+  const int* row_cost;     // [C + 1] prefix sums of the row kernel's cost per pair
+  const int* col_cost;     // [C + 1] prefix sums of the column kernel's cost per pair and block
+  int rows_ctas, cols_ctas;
+};
+bool wide_supported(int n);
+int wide_row_block(int n);   // grid rows per block of lists
+// Resident CTAs per SM of both kernels; 0 when one does not fit.
+cudaError_t wide_prepare(const WideArgs& w, int fmt, int* rows_per_sm, int* cols_per_sm);
+// Row and column kernels of channels [c0, c0 + nc), samples [t0, t0 + nt).
+cudaError_t launch_wide_batch(const WideArgs& w, long long t0, int nt, cudaStream_t s);
+
 bool unfused_supported(int n);
 // Lanes per row FFT (N1) of the unfused kernels: absolute column x is gather
 // group j = x / N1 of lane x % N1.

@@ -5,15 +5,7 @@
 // packed instruction and every weight, twiddle and list entry is read once
 // for both.
 //
-// A 1-D transform of length N = 16 NR of an input with L occupied entries is
-// NR independent tasks, one per output residue r: with n = n' + 16 q and
-// k = NR m + r,
-//   X[NR m + r] = sum_n' e^{2 pi i m n' / 16} ( e^{2 pi i r n' / N}
-//                 sum_q x[n' + 16 q] e^{2 pi i r q / NR} ),
-// a sum over the L / 16 occupied blocks, 15 twiddles and one 16-point DFT in
-// registers, for any L.  The tasks of a transform read the same L inputs
-// (shared-memory broadcasts: the NR lanes of one transform are neighbours)
-// and exchange nothing.
+// The transforms are residue tasks (epic_residue.cuh) of 16 outputs.
 //
 // One persistent launch images a batch.  Every CTA takes an equal share of
 // the estimated cost of the (channel, frame pair) list, so that no last wave
@@ -34,6 +26,7 @@
 // 2000 samples 37.6 against 53.9 us (with the update).
 #include "epic_fft.cuh"
 #include "epic_internal.h"
+#include "epic_residue.cuh"
 
 #include <cstdint>
 
@@ -43,86 +36,13 @@ namespace {
 using fft::Cf2;
 using fft::cmul;
 using fft::f2_fma;
-using fft::f2_mul;
 using fft::f2_pack;
 using fft::f2_splat;
-using fft::f2_unpack;
 using fft::f32x2;
 
 // Frame pairs per FP32 partial image (FP64 across): 128 roundings of a running
 // sum, image error 0.9e-7 against 64 bits over 10^4 samples (1.4e-7 at 256).
 constexpr int kPairRun = 128;
-
-// y[j] += x[j] a for four complex pairs and one complex factor a given as
-// splats; consecutive instructions share the factor's operand.
-__device__ __forceinline__ void cmadd4(Cf2* y, const Cf2* __restrict__ x, f32x2 ar, f32x2 ai, f32x2 nai) {
-  Cf2 v[4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) v[j] = x[j];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) y[j].re = f2_fma(v[j].re, ar, y[j].re);
-#pragma unroll
-  for (int j = 0; j < 4; ++j) y[j].im = f2_fma(v[j].im, ar, y[j].im);
-#pragma unroll
-  for (int j = 0; j < 4; ++j) y[j].re = f2_fma(v[j].im, nai, y[j].re);
-#pragma unroll
-  for (int j = 0; j < 4; ++j) y[j].im = f2_fma(v[j].re, ai, y[j].im);
-}
-
-// Task r of a transform of src[0 .. len4), len4 a multiple of 4 and uniform
-// over the CTA: y[m] = X[NR m + r].  tw: [16][NR] e^{2 pi i r n' / N};
-// wq: [16][NR] e^{2 pi i r q / NR}.
-template <int NR>
-__device__ __forceinline__ void dft_task(const Cf2* __restrict__ src, int len4, int r, const float2* tw,
-                                         const float2* wq, Cf2 (&y)[16]) {
-#pragma unroll
-  for (int b = 0; b < 4; ++b) {
-    if (4 * b < len4) {
-#pragma unroll
-      for (int j = 4 * b; j < 4 * b + 4; ++j) y[j] = src[j];
-    } else {
-#pragma unroll
-      for (int j = 4 * b; j < 4 * b + 4; ++j) y[j] = Cf2{0ull, 0ull};
-    }
-  }
-  for (int q = 1; 16 * q < len4; ++q) {
-    const float2 a = wq[q * NR + r];
-    const f32x2 ar = f2_splat(a.x), ai = f2_splat(a.y), nai = f2_splat(-a.y);
-    const Cf2* s = src + 16 * q;
-    const int left = len4 - 16 * q;
-#pragma unroll
-    for (int b = 0; b < 4; ++b)
-      if (4 * b < left) cmadd4(&y[4 * b], s + 4 * b, ar, ai, nai);
-  }
-  if constexpr (NR > 1) {
-#pragma unroll
-    for (int j = 1; j < 16; ++j) {
-      const float2 t = tw[j * NR + r];
-      const f32x2 c = f2_splat(t.x), s = f2_splat(t.y), ns = f2_splat(-t.y);
-      const Cf2 v = y[j];
-      y[j].re = f2_fma(v.im, ns, f2_mul(v.re, c));
-      y[j].im = f2_fma(v.re, s, f2_mul(v.im, c));
-    }
-  }
-  fft::Dft<16>::run(y);
-}
-
-// Scaled voltage of the 4-bit sample in the low byte of b.
-__device__ __forceinline__ float2 unpack_ci4(unsigned b, float vs) {
-  const int re = static_cast<int>(b << 24) >> 28;
-  const int im = static_cast<int>(b << 28) >> 28;
-  return make_float2(static_cast<float>(re) * vs, static_cast<float>(im) * vs);
-}
-
-template <int FMT>
-__device__ __forceinline__ float2 pair_volt(const void* volt, size_t idx, float vs) {
-  if constexpr (FMT == 0) {
-    return unpack_ci4(__ldg(static_cast<const unsigned char*>(volt) + idx), vs);
-  } else {
-    const float2 e = __ldg(static_cast<const float2*>(volt) + idx);
-    return make_float2(e.x * vs, e.y * vs);
-  }
-}
 
 // Gridding of one frame pair: slices of 32 cells, one cell per lane.
 template <int BT>
@@ -144,27 +64,6 @@ __device__ __forceinline__ void grid_pair(const int* __restrict__ cell, const in
     }
     if (at >= 0) grid[at] = sum;
   }
-}
-
-// |E|^2 of the 16 outputs of a column task, both frames, into the running
-// sums (one rounding of a sum per pair).
-__device__ __forceinline__ void square_add(const Cf2 (&y)[16], float (&acc)[16]) {
-#pragma unroll
-  for (int m = 0; m < 16; ++m) {
-    const float2 re = f2_unpack(y[m].re), im = f2_unpack(y[m].im);
-    acc[m] += fmaf(re.x, re.x, fmaf(im.x, im.x, fmaf(re.y, re.y, im.y * im.y)));
-  }
-}
-
-// Output slot `slot` of both frames times the phase ph.
-__device__ __forceinline__ void store_pixel(const Cf2 (&y)[16], int slot, float2 ph, float2* p0, float2* p1) {
-#pragma unroll
-  for (int m = 0; m < 16; ++m)
-    if (m == slot) {
-      const float2 re = f2_unpack(y[m].re), im = f2_unpack(y[m].im);
-      *p0 = cmul(make_float2(re.x, im.x), ph);
-      if (p1) *p1 = cmul(make_float2(re.y, im.y), ph);
-    }
 }
 
 // Multiple-pixel EPICal: the calibration pixels among a thread's outputs
@@ -198,25 +97,6 @@ __device__ __forceinline__ void prefetch_pair(const ImageArgs& A, long long p, i
         asm volatile("prefetch.global.L1 [%0];" ::"l"(q));
     }
 }
-
-// The share of one CTA in the cost of all (channel, frame pair)s: positions
-// [lo, hi) of the list of channels, cost[c + 1] - cost[c] per pair.
-struct Share {
-  long long lo, hi, pairs;
-  const int* cost;
-  __device__ __forceinline__ Share(const ImageArgs& A) : pairs((A.n_time + 1) / 2), cost(A.pcost) {
-    const long long total = static_cast<long long>(__ldg(cost + A.n_chan)) * pairs, g = gridDim.x, b = blockIdx.x;
-    lo = total / g * b + total % g * b / g;
-    hi = total / g * (b + 1) + total % g * (b + 1) / g;
-  }
-  __device__ __forceinline__ long long before(int c) const { return static_cast<long long>(__ldg(cost + c)) * pairs; }
-  // first pair of channel c at or after position pos
-  __device__ __forceinline__ long long pair_at(long long pos, int c) const {
-    const long long w = __ldg(cost + c + 1) - __ldg(cost + c);
-    const long long p = (pos - before(c) + w - 1) / w;
-    return p < 0 ? 0 : (p > pairs ? pairs : p);
-  }
-};
 
 // A channel's tables and geometry, its tap lists in shared memory (TS) or
 // read through L1.
@@ -315,20 +195,14 @@ __global__ void __launch_bounds__(PCfg<N>::BT, PCfg<N>::PER_SM) epic_image_pair(
 
   const int tid = threadIdx.x;
   const int aw = (BT - 32 - (tid & ~31)) + (tid & 31);     // antenna of this thread: the last warps first
-  for (int i = tid; i < N; i += BT) {
-    const int n = i / NR, r = i % NR;                      // also (q, r) of wq
-    tw[i] = A.twid[(n * r) & (N - 1)];
-    wq[i] = A.twid[(16 * n * r) & (N - 1)];
-  }
+  residue_tables<N, NR>(A.twid, tw, wq, BT);
   if (tid == 0) Es[Na] = Cf2{0ull, 0ull};
 
   const long long T = A.n_time;
   const int C = A.n_chan;
-  const Share share(A);
-  int c = 0;
-  while (c < C && share.before(c + 1) <= share.lo) ++c;
+  const Share share(A.pcost, A.n_chan, 1, (A.n_time + 1) / 2);
   int cur = -1;
-  for (; c < C && share.before(c) < share.hi; ++c) {
+  for (int c = share.first(C); c < C && share.before(c) < share.hi; ++c) {
     const long long p_lo = share.pair_at(share.lo, c), p_hi = share.pair_at(share.hi, c);
     const Chan ch = channel<TS>(A, c, sslice, scell, sent);
     for (long long pa = p_lo; pa < p_hi; pa += kPairRun) {
@@ -407,7 +281,7 @@ __global__ void __launch_bounds__(PCfg<N>::BT, PCfg<N>::PER_SM) epic_image_pair(
         for (int task = tid; task < ch.R * NR; task += BT) {
           const int row = task / NR, r = task % NR;
           Cf2 y[16];
-          dft_task<NR>(grid + row * gs, ch.W4, r, tw, wq, y);
+          dft_task<16, NR>(grid + row * gs, ch.W4, r, tw, wq, y);
 #pragma unroll
           for (int m = 0; m < 16; ++m) Tt[(NR * m + r) * rs + row] = y[m];
         }
@@ -421,7 +295,7 @@ __global__ void __launch_bounds__(PCfg<N>::BT, PCfg<N>::PER_SM) epic_image_pair(
           if (TASKS >= BT || task < TASKS) {
             const int kx = task / NR, r = task % NR;
             Cf2 y[16];
-            dft_task<NR>(Tt + kx * rs, ch.R4, r, tw, wq, y);
+            dft_task<16, NR>(Tt + kx * rs, ch.R4, r, tw, wq, y);
             square_add(y, acc[i]);
             if (A.do_cal && kx == A.k0x && r == A.k0y % NR) store_pixel(y, A.k0y / NR, ch.pph, pixs, pixs + 1);
             if (A.npix) store_taps(A, y, task, p, c);

@@ -158,6 +158,13 @@ struct epic_plan_s {
   int ctas = 0;
   int sms = 0;
 
+  // plain path in its frame-pair form (N = 256, 512)
+  bool wide = false;
+  DevBuf<unsigned char> d_wlists;   // row blocks' tap lists
+  DevBuf<int2> d_wat;               // [C][nb_max] (offset, bytes) / 16 of each block's lists
+  DevBuf<int> d_wrcost, d_wccost;   // [C + 1] cost prefixes of the row and column kernels
+  int w_nb_max = 0, w_max_lists = 0, w_gs = 0, w_rows_ctas = 0, w_cols_ctas = 0;
+
   // host-API staging
   DevBuf<unsigned char> d_stage_in;
   DevBuf<double> d_stage_img;
@@ -410,11 +417,133 @@ epic_status build_gather(epic_plan_t p, const std::vector<float>& wts, int N1, b
   return EPIC_OK;
 }
 
-// Gridding of Eq. 9 as one tap list per occupied grid cell (frame-pair
-// form): the cells of a channel sorted by their number of taps, most first,
-// in slices of 32 (one per lane) as long as their longest list; entry k of
-// the slice's lanes is contiguous.  Shorter lists and lanes without a cell
-// read the zero voltage behind the last antenna with weight 0.
+// Gridding of Eq. 9 as one tap list per grid cell (frame-pair forms): the
+// cells sorted by their number of taps, most first, in slices of 32 (one per
+// lane) as long as their longest list; entry k of a slice's lanes is
+// contiguous.  Shorter lists and lanes without a cell read the zero voltage
+// behind the last antenna with weight 0.
+struct Tap {
+  int cell, ant;
+  float w;
+};
+
+struct SliceLists {
+  std::vector<int> cell;        // 32 per slice, -1 = none
+  std::vector<int2> slice;      // (first entry, taps)
+  std::vector<uint2> ent;       // (byte offset of E'_a, weight bits)
+  std::vector<int> count, order, place, start, sorted;   // scratch
+  std::vector<unsigned char> bank;                       // 16-byte bank of a cell's first antenna
+};
+
+// Lists of the taps on n_cells cells; empty: cells without taps are listed
+// too where empty[cell] is set.
+void slice_lists(const std::vector<Tap>& taps, int n_cells, const std::vector<unsigned char>* empty, int n_ant,
+                 SliceLists* t) {
+  std::vector<int>&count = t->count, &order = t->order, &start = t->start, &sorted = t->sorted;
+  count.assign(n_cells, 0);
+  t->bank.assign(n_cells, 0);
+  int most = 0;
+  for (const Tap& q : taps) {
+    if (!count[q.cell]) t->bank[q.cell] = static_cast<unsigned char>(q.ant % 8);
+    most = std::max(most, ++count[q.cell]);
+  }
+  // counting sort, most taps first
+  const auto listed = [&](int i) { return count[i] > 0 || (empty && (*empty)[i]); };
+  start.assign(most + 1, 0);
+  for (int i = 0; i < n_cells; ++i)
+    if (listed(i)) ++start[most - count[i]];
+  int cells = 0;
+  for (int& v : start) {
+    const int n = v;
+    v = cells;
+    cells += n;
+  }
+  sorted.assign(cells, 0);
+  for (int i = 0; i < n_cells; ++i)
+    if (listed(i)) sorted[start[most - count[i]]++] = i;
+  // cells of equal length taken in turn from the 8 banks
+  order.clear();
+  for (int lo = 0; lo < cells;) {
+    int hi = lo;
+    std::vector<int> by[8];
+    for (; hi < cells && count[sorted[hi]] == count[sorted[lo]]; ++hi) by[t->bank[sorted[hi]]].push_back(sorted[hi]);
+    for (size_t k = 0; order.size() < static_cast<size_t>(hi); ++k)
+      for (const auto& b : by)
+        if (k < b.size()) order.push_back(b[k]);
+    lo = hi;
+  }
+  t->place.assign(n_cells, -1);
+  for (int i = 0; i < cells; ++i) t->place[order[i]] = i;
+  const int slices = (cells + 31) / 32;
+  t->slice.clear();
+  int ne = 0;
+  for (int s = 0; s < slices; ++s) {
+    const int m = count[order[32 * s]];
+    t->slice.push_back(make_int2(ne, m));
+    ne += 32 * m;
+  }
+  t->cell.assign(static_cast<size_t>(slices) * 32, -1);
+  std::copy(order.begin(), order.end(), t->cell.begin());
+  t->ent.assign(ne, make_uint2(static_cast<unsigned>(n_ant) * 16u, 0u));
+  std::fill(count.begin(), count.end(), 0);
+  for (const Tap& q : taps) {
+    const int i = t->place[q.cell];
+    uint2& e = t->ent[t->slice[i / 32].x + static_cast<size_t>(count[q.cell]++) * 32 + i % 32];
+    e.x = static_cast<unsigned>(q.ant) * 16u;
+    std::memcpy(&e.y, &q.w, sizeof q.w);
+  }
+  // the order of a list's taps is free: let the 8 lanes of a quarter warp
+  // read different 16-byte banks of E' at each step where they can
+  for (int i = 0; i < slices * 32; i += 8) {
+    const int2 sl = t->slice[i / 32];
+    for (int k = 0; k < sl.y; ++k) {
+      unsigned used = 0;
+      for (int l = i; l < i + 8 && l < cells; ++l) {
+        uint2* e = &t->ent[sl.x + l % 32];
+        const int n = count[order[l]];
+        for (int m = k; m < n; ++m)
+          if (!((used >> (e[static_cast<size_t>(m) * 32].x / 16 % 8)) & 1u)) {
+            std::swap(e[static_cast<size_t>(m) * 32], e[static_cast<size_t>(k) * 32]);
+            break;
+          }
+        if (k < n) used |= 1u << (e[static_cast<size_t>(k) * 32].x / 16 % 8);
+      }
+    }
+  }
+}
+
+// Taps of channel c by blocks of rb window rows, cell = (row in block) * gs + window column.
+void block_taps(const epic_plan_s* p, const std::vector<float>& wts, int c, int gs, int rb,
+                std::vector<std::vector<Tap>>* blocks) {
+  const int Na = p->na, K = p->k, KK = K * K, h = (K - 1) / 2;
+  blocks->resize((p->rows[c] + rb - 1) / rb);
+  for (auto& b : *blocks) b.clear();
+  for (int a = 0; a < Na; ++a) {
+    if (p->flags[a]) continue;
+    const size_t ob = (static_cast<size_t>(c) * Na + a) * 2;
+    const int r0 = p->base[ob + 1] - h - p->y0[c], x0 = p->base[ob] - h - p->x0[c];
+    const float* wf = &wts[(static_cast<size_t>(c) * Na + a) * KK];
+    for (int dy = 0; dy < K; ++dy)
+      for (int dx = 0; dx < K; ++dx)
+        if (wf[dy * K + dx] != 0.0f)
+          (*blocks)[(r0 + dy) / rb].push_back(Tap{(r0 + dy) % rb * gs + x0 + dx, a, wf[dy * K + dx]});
+  }
+}
+
+void prefix_sums(std::vector<int>* v) {
+  int sum = 0;
+  for (int& x : *v) {
+    const int w = x;
+    x = sum;
+    sum += w;
+  }
+  v->push_back(sum);
+}
+
+// Cost of one transform task of P outputs from L inputs and of the whole
+// transform of an N-point axis, in packed FP32 instructions of a thread.
+long long task_cost(int P, int L) { return 18LL * P + 5LL * std::max(0, ((L + 3) & ~3) - P); }
+
 struct CellTables {
   std::vector<int> cell, sbase, ebase, cost;
   std::vector<int2> slice;
@@ -423,112 +552,83 @@ struct CellTables {
 };
 
 void build_cells(const epic_plan_s* p, const std::vector<float>& wts, int gs, CellTables* t) {
-  const int C = p->nc, Na = p->na, N = p->n, K = p->k, KK = K * K, h = (K - 1) / 2;
-  std::vector<int> count, order, place, start, sorted;
-  std::vector<unsigned char> bank;         // 16-byte bank of a cell's first antenna
-  for (int c = 0; c < C; ++c) {
+  const int N = p->n;
+  SliceLists l;
+  std::vector<std::vector<Tap>> taps;
+  for (int c = 0; c < p->nc; ++c) {
     t->sbase.push_back(static_cast<int>(t->slice.size()));
     t->ebase.push_back(static_cast<int>(t->ent.size()));
     const int R = p->rows[c];
-    count.assign(static_cast<size_t>(R) * gs, 0);
-    bank.assign(count.size(), 0);
-    auto each_tap = [&](auto&& f) {
-      for (int a = 0; a < Na; ++a) {
-        if (p->flags[a]) continue;
-        const size_t ob = (static_cast<size_t>(c) * Na + a) * 2;
-        const int r0 = p->base[ob + 1] - h - p->y0[c], x0 = p->base[ob] - h - p->x0[c];
-        const float* wf = &wts[(static_cast<size_t>(c) * Na + a) * KK];
-        for (int dy = 0; dy < K; ++dy)
-          for (int dx = 0; dx < K; ++dx)
-            if (wf[dy * K + dx] != 0.0f) f(a, (r0 + dy) * gs + x0 + dx, wf[dy * K + dx]);
-      }
-    };
-    int most = 0;
-    long long taps = 0;
-    each_tap([&](int a, int cell, float) {
-      if (!count[cell]) bank[cell] = static_cast<unsigned char>(a % 8);
-      most = std::max(most, ++count[cell]);
-      ++taps;
-    });
-    // counting sort of the occupied cells, most taps first
-    start.assign(most + 2, 0);
-    for (int n : count) ++start[most - n];
-    int cells = 0;
-    for (int i = 0; i < most; ++i) {
-      const int n = start[i];
-      start[i] = cells;
-      cells += n;
-    }
-    sorted.assign(cells, 0);
-    for (size_t i = 0; i < count.size(); ++i)
-      if (count[i]) sorted[start[most - count[i]]++] = static_cast<int>(i);
-    // cells of equal length taken in turn from the 8 banks
-    order.clear();
-    for (int lo = 0; lo < cells;) {
-      int hi = lo;
-      std::vector<int> by[8];
-      for (; hi < cells && count[sorted[hi]] == count[sorted[lo]]; ++hi) by[bank[sorted[hi]]].push_back(sorted[hi]);
-      for (size_t k = 0; order.size() < static_cast<size_t>(hi); ++k)
-        for (const auto& b : by)
-          if (k < b.size()) order.push_back(b[k]);
-      lo = hi;
-    }
-    place.assign(count.size(), -1);
-    for (int i = 0; i < cells; ++i) place[order[i]] = i;
-    const int slices = (cells + 31) / 32;
-    const size_t s0 = t->slice.size(), e0 = t->ent.size();
-    int ne = 0;
-    for (int s = 0; s < slices; ++s) {
-      const int m = count[order[32 * s]];
-      t->slice.push_back(make_int2(ne, m));
-      ne += 32 * m;
-    }
-    t->cell.resize((s0 + slices) * 32, -1);
-    for (int i = 0; i < cells; ++i) t->cell[s0 * 32 + i] = order[i];
-    t->ent.resize(e0 + ne, make_uint2(static_cast<unsigned>(Na) * 16u, 0u));
-    std::fill(count.begin(), count.end(), 0);
-    each_tap([&](int a, int cell, float w) {
-      const int i = place[cell];
-      uint2& q = t->ent[e0 + t->slice[s0 + i / 32].x + static_cast<size_t>(count[cell]++) * 32 + i % 32];
-      q.x = static_cast<unsigned>(a) * 16u;
-      std::memcpy(&q.y, &w, sizeof w);
-    });
-    // the order of a list's taps is free: let the 8 lanes of a quarter warp
-    // read different 16-byte banks of E' at each step where they can
-    for (int i = 0; i < slices * 32; i += 8) {
-      const int2 sl = t->slice[s0 + i / 32];
-      for (int k = 0; k < sl.y; ++k) {
-        unsigned used = 0;
-        for (int l = i; l < i + 8 && l < cells; ++l) {
-          uint2* e = &t->ent[e0 + sl.x + l % 32];
-          const int n = count[order[l]];
-          for (int m = k; m < n; ++m)
-            if (!((used >> (e[static_cast<size_t>(m) * 32].x / 16 % 8)) & 1u)) {
-              std::swap(e[static_cast<size_t>(m) * 32], e[static_cast<size_t>(k) * 32]);
-              break;
-            }
-          if (k < n) used |= 1u << (e[static_cast<size_t>(k) * 32].x / 16 % 8);
-        }
-      }
-    }
-    t->max_slices = std::max(t->max_slices, slices);
-    t->max_ent = std::max(t->max_ent, ne);
-    // cost of one frame pair, in packed FP32 instructions of a thread: a
-    // transform task of length L is about 290 + 5 (L - 16); a tap 12
-    const auto task = [](int L) { return 290 + 5 * std::max(0, ((L + 3) & ~3) - 16); };
-    const long long work = static_cast<long long>(N) * (N / 16) * task(R) +
-                           static_cast<long long>(R) * (N / 16) * task(p->cols[c]) + 12 * taps + 20 * Na;
+    block_taps(p, wts, c, gs, R, &taps);
+    slice_lists(taps[0], R * gs, nullptr, p->na, &l);
+    t->cell.insert(t->cell.end(), l.cell.begin(), l.cell.end());
+    t->slice.insert(t->slice.end(), l.slice.begin(), l.slice.end());
+    t->ent.insert(t->ent.end(), l.ent.begin(), l.ent.end());
+    t->max_slices = std::max(t->max_slices, static_cast<int>(l.slice.size()));
+    t->max_ent = std::max(t->max_ent, static_cast<int>(l.ent.size()));
+    // cost of one frame pair: the transform tasks, 12 per tap, 20 per antenna
+    const long long work = static_cast<long long>(N) * (N / 16) * task_cost(16, R) +
+                           static_cast<long long>(R) * (N / 16) * task_cost(16, p->cols[c]) +
+                           12LL * static_cast<long long>(taps[0].size()) + 20LL * p->na;
     t->cost.push_back(static_cast<int>(std::max<long long>(1, work / 256)));
   }
   t->sbase.push_back(static_cast<int>(t->slice.size()));
   t->ebase.push_back(static_cast<int>(t->ent.size()));
-  int sum = 0;
-  for (int& v : t->cost) {
-    const int w = v;
-    v = sum;
-    sum += w;
+  prefix_sums(&t->cost);
+}
+
+// Tap lists of the wide frame-pair form: per channel and block of row_block
+// window rows one contiguous piece (header, slices, 16-bit cells, entries;
+// every piece a multiple of 16 bytes), cells without taps included.
+struct WideTables {
+  std::vector<unsigned char> lists;
+  std::vector<int2> at;          // [C][nb_max] (offset, bytes) / 16
+  std::vector<int> row_cost, col_cost;
+  int nb_max = 0, max_lists = 0;
+};
+
+void build_wide_lists(const epic_plan_s* p, const std::vector<float>& wts, int gs, WideTables* t) {
+  const int rb = epic::wide_row_block(p->n), N = p->n;
+  t->nb_max = (p->rows_alloc + rb - 1) / rb;
+  t->at.assign(static_cast<size_t>(p->nc) * t->nb_max, make_int2(0, 0));
+  SliceLists l;
+  std::vector<std::vector<Tap>> taps;
+  std::vector<unsigned char> inside;
+  for (int c = 0; c < p->nc; ++c) {
+    const int R = p->rows[c];
+    block_taps(p, wts, c, gs, rb, &taps);
+    long long listed = 0;
+    for (size_t b = 0; b < taps.size(); ++b) {
+      const int rows = std::min(rb, R - static_cast<int>(b) * rb);
+      inside.assign(static_cast<size_t>(rb) * gs, 0);
+      for (int r = 0; r < rows; ++r) std::fill_n(inside.begin() + r * gs, p->cols[c], 1);
+      slice_lists(taps[b], rb * gs, &inside, p->na, &l);
+      const size_t ns = l.slice.size();
+      int hd[4] = {static_cast<int>(ns), 0, 0, 0};
+      hd[1] = static_cast<int>((sizeof hd + ns * sizeof(int2) + 15) & ~static_cast<size_t>(15));
+      hd[2] = hd[1] + static_cast<int>(ns * 64);
+      const size_t bytes = (hd[2] + l.ent.size() * sizeof(uint2) + 15) & ~static_cast<size_t>(15);
+      const size_t o = t->lists.size();
+      t->lists.resize(o + bytes, 0);
+      unsigned char* d = t->lists.data() + o;
+      std::memcpy(d, hd, sizeof hd);
+      std::memcpy(d + sizeof hd, l.slice.data(), ns * sizeof(int2));
+      for (size_t i = 0; i < ns * 32; ++i) {
+        const uint16_t v = l.cell[i] < 0 ? 0xffffu : static_cast<uint16_t>(l.cell[i]);
+        std::memcpy(d + hd[1] + 2 * i, &v, 2);
+      }
+      std::memcpy(d + hd[2], l.ent.data(), l.ent.size() * sizeof(uint2));
+      t->at[static_cast<size_t>(c) * t->nb_max + b] = make_int2(static_cast<int>(o / 16), static_cast<int>(bytes / 16));
+      t->max_lists = std::max(t->max_lists, static_cast<int>(bytes));
+      listed += static_cast<long long>(l.ent.size()) + 2 * static_cast<long long>(ns) * 32;
+    }
+    const long long rows = static_cast<long long>(R) * (N / 32) * task_cost(32, p->cols[c]) + 10 * listed + 20LL * p->na;
+    t->row_cost.push_back(static_cast<int>(std::max<long long>(1, rows / 256)));
+    t->col_cost.push_back(static_cast<int>(task_cost(32, R)));
   }
-  t->cost.push_back(sum);
+  t->max_lists = (t->max_lists + 127) & ~127;
+  prefix_sums(&t->row_cost);
+  prefix_sums(&t->col_cost);
 }
 
 // Arguments of one fused launch over a device batch.
@@ -630,8 +730,81 @@ epic_status image_cluster(epic_plan_t p, const void* d_volt, long long n_time, d
   return EPIC_OK;
 }
 
+// Arguments of the wide frame-pair form that belong to the plan.
+void wide_plan_args(const epic_plan_s* p, epic::WideArgs* w) {
+  w->u.grid_n = p->n;
+  w->u.n_chan = p->nc;
+  w->u.n_ant = p->na;
+  w->u.rs = p->rs;
+  w->win4 = p->d_win4.p;
+  w->lists = p->d_wlists.p;
+  w->lists_at = p->d_wat.p;
+  w->nb_max = p->w_nb_max;
+  w->max_lists = p->w_max_lists;
+  w->gs = p->w_gs;
+  w->row_cost = p->d_wrcost.p;
+  w->col_cost = p->d_wccost.p;
+  w->rows_ctas = p->w_rows_ctas;
+  w->cols_ctas = p->w_cols_ctas;
+}
+
+// Frame-pair form of the plain path: batches of up to kWideTime samples of a
+// group of channels through the device scratch.  Samples come first (an image
+// block is added to once per batch and share), channels as the budget allows.
+epic_status image_wide(epic_plan_t p, const void* d_volt, long long n_time, double* d_image) {
+  constexpr long long kWideTime = 256;
+  const int C = p->nc, N = p->n;
+  const size_t chan_t = static_cast<size_t>(N) * p->rs * sizeof(float2);   // one sample of one channel
+  long long nt = std::min<long long>((n_time + 1) / 2 * 2, kWideTime);
+  if (p->tune_nt > 0) nt = std::max<long long>(2, std::min<long long>(nt, p->tune_nt / 2 * 2));
+  nt = std::max<long long>(2, std::min<long long>(nt, static_cast<long long>(p->workspace_budget / chan_t) / 2 * 2));
+  const long long fit = std::max<long long>(1, static_cast<long long>(p->workspace_budget / (chan_t * static_cast<size_t>(nt))));
+  const int groups = static_cast<int>((C + std::min<long long>(fit, C) - 1) / std::min<long long>(fit, C));
+  const int nc = (C + groups - 1) / groups;
+  const size_t spec_n = static_cast<size_t>(nt) * nc * N * p->rs, need = spec_n + static_cast<size_t>(nt) * C;
+  if (p->d_ws.n < need) {
+    cudaError_t e = cudaStreamSynchronize(p->stream);
+    if (e != cudaSuccess) return cuda_fail(e, "stream sync before scratch growth");
+    if (p->d_ws.alloc(need) != cudaSuccess) return fail(EPIC_ERR_OOM, "unfused scratch allocation failed");
+  }
+  p->ws_time = static_cast<int>(std::max<long long>(1, nt * nc / C));   // samples of all channels the scratch holds
+  epic::WideArgs w{};
+  wide_plan_args(p, &w);
+  epic::UnfusedArgs& a = w.u;
+  a.volt = d_volt;
+  a.input_fmt = p->input;
+  a.cell0 = p->d_cell0.p;
+  a.wgain = p->d_wgain.p;
+  a.vscale = p->d_vscale.p;
+  a.twid = p->d_twid.p;
+  a.spec = p->d_ws.p;
+  a.pix = a.spec + spec_n;
+  a.pixph = p->d_pixph.p;
+  a.err = p->d_err.p;
+  a.sms = p->sms;
+  a.image = d_image;
+  a.img_scale = 1.0 / static_cast<double>(n_time);
+  a.do_cal = p->cal ? 1 : 0;
+  a.k0x = p->cal ? p->k0x : 0;
+  a.k0y = p->cal ? p->k0y : 0;
+  a.kacc = p->d_kacc.p;
+  a.pacc = p->d_pacc.p;
+  for (long long t0 = 0; t0 < n_time; t0 += nt) {
+    const int n = static_cast<int>(std::min<long long>(nt, n_time - t0));
+    for (int c0 = 0; c0 < C; c0 += nc) {
+      w.c0 = c0;
+      w.nc = std::min(nc, C - c0);
+      EPIC_CUDA(epic::launch_wide_batch(w, t0, n, p->stream));
+    }
+    if (p->cal) EPIC_CUDA(epic::launch_correlate(a, t0, n, p->stream));
+  }
+  if (p->cal) p->frames += n_time;
+  return EPIC_OK;
+}
+
 // Plain unfused path: batches of time samples through the device scratch.
 epic_status image_unfused(epic_plan_t p, const void* d_volt, long long n_time, double* d_image) {
+  if (p->wide) return image_wide(p, d_volt, n_time, d_image);
   const int C = p->nc, N = p->n;
   // per time sample: row spectra [C][N][rs] and the calibrator pixel [C]
   const size_t per_t = static_cast<size_t>(C) * (static_cast<size_t>(N) * p->rs + 1);
@@ -1003,7 +1176,7 @@ epic_status build_grid_tables(epic_plan_s* p, std::vector<int>& cell0, std::vect
 // placement (or the warp-specialised form), the cluster form when asked
 // for, else the plain unfused path; CTAs per launch.
 epic_status choose_path(epic_plan_s* p, const epic_plan_desc* d, bool fused_shape, bool unfused_ok,
-                        const std::vector<float>& wts, CellTables* cells) {
+                        const std::vector<float>& wts, CellTables* cells, WideTables* wide) {
   const int Na = p->na, N = p->n, KK = p->k * p->k;
   p->rs = epic::image_rs(p->rows_alloc);
   int dev = 0;
@@ -1129,6 +1302,25 @@ epic_status choose_path(epic_plan_s* p, const epic_plan_desc* d, bool fused_shap
     p->smem = 0;
     p->ctas = p->sms;
     p->path = EPIC_PATH_UNFUSED;
+    // frame pairs where a pair of one channel fits the scratch budget and the
+    // kernels' blocks fit shared memory; the persistent form keeps its own
+    const size_t pair_bytes = 2 * static_cast<size_t>(N) * p->rs * sizeof(float2);
+    if (p->precision == EPIC_PREC_FP32 && !p->persistent && epic::wide_supported(N) &&
+        pair_bytes <= p->workspace_budget) {
+      p->w_gs = ((*std::max_element(p->cols.begin(), p->cols.end()) + 3) & ~3) + 1;
+      build_wide_lists(p, wts, p->w_gs, wide);
+      p->w_nb_max = wide->nb_max;
+      p->w_max_lists = wide->max_lists;
+      epic::WideArgs w{};
+      wide_plan_args(p, &w);
+      int rows_per_sm = 0, cols_per_sm = 0;
+      e = epic::wide_prepare(w, p->input, &rows_per_sm, &cols_per_sm);
+      if (e != cudaSuccess) return cuda_fail(e, "wide kernel attributes");
+      p->wide = rows_per_sm > 0 && cols_per_sm > 0;
+      p->w_rows_ctas = rows_per_sm * p->sms;
+      p->w_cols_ctas = cols_per_sm * p->sms;
+      if (!p->wide) *wide = WideTables();
+    }
   }
 
   return EPIC_OK;
@@ -1217,7 +1409,8 @@ epic_status epic_plan_create(epic_plan_t* out, const epic_plan_desc* d) {
 
   // ---- launch shape ----
   CellTables cells;
-  if (epic_status st = choose_path(p, d, fused_shape, unfused_ok, wts, &cells)) {
+  WideTables wide;
+  if (epic_status st = choose_path(p, d, fused_shape, unfused_ok, wts, &cells, &wide)) {
     delete p;
     return st;
   }
@@ -1247,7 +1440,7 @@ epic_status epic_plan_create(epic_plan_t* out, const epic_plan_desc* d) {
   std::vector<int> gofs, gbase, ugofs, ugbase;
   std::vector<uint4> gcnt, ugcnt;
   std::vector<uint2> gent, ugent;
-  if ((p->path == EPIC_PATH_FUSED && !p->pair) || p->path == EPIC_PATH_UNFUSED) {
+  if ((p->path == EPIC_PATH_FUSED && !p->pair) || (p->path == EPIC_PATH_UNFUSED && !p->wide)) {
     const int n1 = p->path == EPIC_PATH_FUSED ? epic::image_fft_lanes(N) : epic::unfused_fft_lanes(N);
     if (epic_status st = build_gather(p, wts, n1, true, gofs, gcnt, gent, gbase)) {
       epic_plan_destroy(p);
@@ -1283,7 +1476,8 @@ epic_status epic_plan_create(epic_plan_t* out, const epic_plan_desc* d) {
                       up(p->d_ugofs, ugofs), up(p->d_ugcnt, ugcnt), up(p->d_ugent, ugent),
                       up(p->d_ugbase, ugbase), up(p->d_pcell, cells.cell), up(p->d_pslice, cells.slice),
                       up(p->d_pent, cells.ent), up(p->d_psbase, cells.sbase), up(p->d_pebase, cells.ebase),
-                      up(p->d_pcost, cells.cost)};
+                      up(p->d_pcost, cells.cost), up(p->d_wlists, wide.lists), up(p->d_wat, wide.at),
+                      up(p->d_wrcost, wide.row_cost), up(p->d_wccost, wide.col_cost)};
   for (cudaError_t x : es)
     if (x != cudaSuccess) {
       epic_plan_destroy(p);
@@ -1364,6 +1558,10 @@ epic_status epic_plan_destroy(epic_plan_t p) {
   p->d_psbase.release();
   p->d_pebase.release();
   p->d_pcost.release();
+  p->d_wlists.release();
+  p->d_wat.release();
+  p->d_wrcost.release();
+  p->d_wccost.release();
   p->d_uv.release();
   p->d_iters.release();
   if (p->graph_exec) cudaGraphExecDestroy(p->graph_exec);
@@ -2108,7 +2306,7 @@ epic_status epic_autotune(epic_plan_t p, const void* d_volt, long long n_time, d
     // one or two frames per step
     r.row_table = p->tune_row_table;
     r.row_frames = p->tune_row_frames;
-    if (p->precision == EPIC_PREC_FP32)
+    if (p->precision == EPIC_PREC_FP32 && !p->wide)
       for (int tb : {0, 1})
         for (int rf : {1, 2}) {
           if (st != EPIC_OK) break;
@@ -2127,7 +2325,7 @@ epic_status epic_autotune(epic_plan_t p, const void* d_volt, long long n_time, d
     p->tune_row_frames = r.row_frames;
     // then one persistent launch per call against the batched launches
     r.batch_persistent = p->persistent;
-    if (p->precision == EPIC_PREC_FP32 && epic::persistent_supported(p->n) && st == EPIC_OK) {
+    if (p->precision == EPIC_PREC_FP32 && !p->wide && epic::persistent_supported(p->n) && st == EPIC_OK) {
       const int def_pers = p->persistent;
       p->persistent = 1 - def_pers;
       double ms = 0;

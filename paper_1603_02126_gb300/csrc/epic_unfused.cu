@@ -21,6 +21,7 @@
 // pixph).  Every FFT therefore has at most NZ non-zero inputs per lane and
 // uses the pruned first-stage DFT.  The centring signs and 1/Na are folded
 // into the gridding weights.
+#include "epic_bulk.cuh"
 #include "epic_fft.cuh"
 #include "epic_internal.h"
 
@@ -50,10 +51,6 @@ __device__ __forceinline__ float2 load_volt_u(const void* volt, int fmt, size_t 
     return make_float2(static_cast<float>(re), static_cast<float>(im));
   }
   return __ldg(static_cast<const float2*>(volt) + idx);
-}
-
-__device__ __forceinline__ uint32_t smem_addr(const void* p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
 // Bytes of the row kernel's per-channel gather table in shared memory.
@@ -280,28 +277,6 @@ __global__ void __launch_bounds__(kUBT, (N <= 128 ? 3 : 2))
   extern __shared__ __align__(16) unsigned char rsm[];
   for (int i = threadIdx.x; i < N; i += kUBT) tw[i] = A.twid[(i % N1) * (i / N1)];
   rows_body<N, NZ, TS>(A, t0, nt, tw, zbuf, rsm, blockIdx.x, gridDim.x);   // its first step syncs
-}
-
-// Bounded wait of one thread on an mbarrier phase; false on timeout.
-__device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity) {
-  for (int i = 0; i < (1 << 22); ++i) {
-    uint32_t ok;
-    asm volatile(
-        "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    if (ok) return true;
-  }
-  return false;
-}
-
-__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-      ::"r"(dst), "l"(src), "r"(bytes), "r"(bar)
-      : "memory");
 }
 
 // ---- column FFTs + |E|^2: unit = (channel, block of GROUPS columns, time segment) ----
