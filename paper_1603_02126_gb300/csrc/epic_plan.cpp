@@ -748,20 +748,60 @@ void wide_plan_args(const epic_plan_s* p, epic::WideArgs* w) {
   w->cols_ctas = p->w_cols_ctas;
 }
 
-// Frame-pair form of the plain path: batches of up to kWideTime samples of a
-// group of channels through the device scratch.  Samples come first (an image
-// block is added to once per batch and share), channels as the budget allows.
-epic_status image_wide(epic_plan_t p, const void* d_volt, long long n_time, double* d_image) {
+// Batch of the wide frame-pair form: samples per batch and channels per
+// launch.  All samples that fit with every channel, or kWideTime of them with
+// fewer channels (an image block is added to once per batch and share).  The
+// whole scratch budget is used: a launch costs its start and its tail, and
+// batches that stay in L2 were slower (1024 antennas, 256 x 256: 48 MB 29.5,
+// 200 MB 20.7, 512 MB 17.9, 2 GB 16.6 ms).
+struct WideBatch {
+  long long nt = 0;
+  int nc = 0;
+  size_t spec_n = 0, need = 0;   // float2 of the spectra, of the whole scratch
+};
+
+WideBatch wide_batch(const epic_plan_s* p, long long n_time) {
   constexpr long long kWideTime = 256;
   const int C = p->nc, N = p->n;
   const size_t chan_t = static_cast<size_t>(N) * p->rs * sizeof(float2);   // one sample of one channel
-  long long nt = std::min<long long>((n_time + 1) / 2 * 2, kWideTime);
-  if (p->tune_nt > 0) nt = std::max<long long>(2, std::min<long long>(nt, p->tune_nt / 2 * 2));
-  nt = std::max<long long>(2, std::min<long long>(nt, static_cast<long long>(p->workspace_budget / chan_t) / 2 * 2));
-  const long long fit = std::max<long long>(1, static_cast<long long>(p->workspace_budget / (chan_t * static_cast<size_t>(nt))));
-  const int groups = static_cast<int>((C + std::min<long long>(fit, C) - 1) / std::min<long long>(fit, C));
-  const int nc = (C + groups - 1) / groups;
-  const size_t spec_n = static_cast<size_t>(nt) * nc * N * p->rs, need = spec_n + static_cast<size_t>(nt) * C;
+  const size_t budget = p->workspace_budget;
+  WideBatch b;
+  b.nt = std::min<long long>((n_time + 1) / 2 * 2,
+                             std::max<long long>(kWideTime, static_cast<long long>(budget / (chan_t * C))));
+  if (p->tune_nt > 0) b.nt = std::max<long long>(2, std::min<long long>(b.nt, p->tune_nt / 2 * 2));
+  b.nt = std::max<long long>(2, std::min<long long>(b.nt, static_cast<long long>(budget / chan_t) / 2 * 2));
+  const long long fit = static_cast<long long>(budget / (chan_t * static_cast<size_t>(b.nt)));
+  const int most = static_cast<int>(std::max<long long>(1, std::min<long long>(fit, C)));
+  const int groups = (C + most - 1) / most;
+  b.nc = (C + groups - 1) / groups;
+  b.spec_n = static_cast<size_t>(b.nt) * b.nc * N * p->rs;
+  b.need = b.spec_n + static_cast<size_t>(b.nt) * C;
+  return b;
+}
+
+// Whether a fused plan can take the wide form for this call: its scratch is
+// there, or can be allocated (not while the stream is being captured).
+bool wide_ready(epic_plan_t p, long long n_time) {
+  const size_t need = wide_batch(p, n_time).need;
+  if (p->d_ws.n >= need) return true;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(p->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return false;
+  }
+  if (cudaStreamSynchronize(p->stream) != cudaSuccess) return false;
+  if (p->d_ws.alloc(need) == cudaSuccess) return true;
+  cudaGetLastError();
+  return false;
+}
+
+// Frame-pair form of the plain path.
+epic_status image_wide(epic_plan_t p, const void* d_volt, long long n_time, double* d_image) {
+  const int C = p->nc;
+  const WideBatch wb = wide_batch(p, n_time);
+  const long long nt = wb.nt;
+  const int nc = wb.nc;
+  const size_t spec_n = wb.spec_n, need = wb.need;
   if (p->d_ws.n < need) {
     cudaError_t e = cudaStreamSynchronize(p->stream);
     if (e != cudaSuccess) return cuda_fail(e, "stream sync before scratch growth");
@@ -1171,6 +1211,30 @@ epic_status build_grid_tables(epic_plan_s* p, std::vector<int>& cell0, std::vect
   return EPIC_OK;
 }
 
+// Tables and launch shape of the wide frame-pair form where a pair of one
+// channel fits the scratch budget and the kernels' blocks fit shared memory;
+// the persistent form keeps its own kernel.
+epic_status plan_wide(epic_plan_s* p, const std::vector<float>& wts, WideTables* wide) {
+  const int N = p->n;
+  const size_t pair_bytes = 2 * static_cast<size_t>(N) * p->rs * sizeof(float2);
+  if (p->precision != EPIC_PREC_FP32 || p->persistent || !epic::wide_supported(N) || pair_bytes > p->workspace_budget)
+    return EPIC_OK;
+  p->w_gs = ((*std::max_element(p->cols.begin(), p->cols.end()) + 3) & ~3) + 1;
+  build_wide_lists(p, wts, p->w_gs, wide);
+  p->w_nb_max = wide->nb_max;
+  p->w_max_lists = wide->max_lists;
+  epic::WideArgs w{};
+  wide_plan_args(p, &w);
+  int rows_per_sm = 0, cols_per_sm = 0;
+  cudaError_t e = epic::wide_prepare(w, p->input, &rows_per_sm, &cols_per_sm);
+  if (e != cudaSuccess) return cuda_fail(e, "wide kernel attributes");
+  p->wide = rows_per_sm > 0 && cols_per_sm > 0;
+  p->w_rows_ctas = rows_per_sm * p->sms;
+  p->w_cols_ctas = cols_per_sm * p->sms;
+  if (!p->wide) *wide = WideTables();
+  return EPIC_OK;
+}
+
 // Launch shape and path of the plan: the tensor-core form's K extent for
 // FP16/BF16, else the fused kernel's frames per step and gather-table
 // placement (or the warp-specialised form), the cluster form when asked
@@ -1298,29 +1362,17 @@ epic_status choose_path(epic_plan_s* p, const epic_plan_desc* d, bool fused_shap
                               : fail(EPIC_ERR_UNSUPPORTED, "image kernel cannot be resident");
     p->ctas = per_sm * p->sms;
     p->path = EPIC_PATH_FUSED;
+    // footprints that leave no room for two frames on one SM: the spectra of
+    // a pair through HBM (N = 128); multiple-pixel EPICal and calls that may
+    // not allocate stay with the one-frame kernel
+    if (!p->pair && !p->piped)
+      if (epic_status st = plan_wide(p, wts, wide)) return st;
   } else {
     p->smem = 0;
     p->ctas = p->sms;
     p->path = EPIC_PATH_UNFUSED;
-    // frame pairs where a pair of one channel fits the scratch budget and the
-    // kernels' blocks fit shared memory; the persistent form keeps its own
-    const size_t pair_bytes = 2 * static_cast<size_t>(N) * p->rs * sizeof(float2);
-    if (p->precision == EPIC_PREC_FP32 && !p->persistent && epic::wide_supported(N) &&
-        pair_bytes <= p->workspace_budget) {
-      p->w_gs = ((*std::max_element(p->cols.begin(), p->cols.end()) + 3) & ~3) + 1;
-      build_wide_lists(p, wts, p->w_gs, wide);
-      p->w_nb_max = wide->nb_max;
-      p->w_max_lists = wide->max_lists;
-      epic::WideArgs w{};
-      wide_plan_args(p, &w);
-      int rows_per_sm = 0, cols_per_sm = 0;
-      e = epic::wide_prepare(w, p->input, &rows_per_sm, &cols_per_sm);
-      if (e != cudaSuccess) return cuda_fail(e, "wide kernel attributes");
-      p->wide = rows_per_sm > 0 && cols_per_sm > 0;
-      p->w_rows_ctas = rows_per_sm * p->sms;
-      p->w_cols_ctas = cols_per_sm * p->sms;
-      if (!p->wide) *wide = WideTables();
-    }
+    if (N > 128)
+      if (epic_status st = plan_wide(p, wts, wide)) return st;
   }
 
   return EPIC_OK;
@@ -1440,7 +1492,7 @@ epic_status epic_plan_create(epic_plan_t* out, const epic_plan_desc* d) {
   std::vector<int> gofs, gbase, ugofs, ugbase;
   std::vector<uint4> gcnt, ugcnt;
   std::vector<uint2> gent, ugent;
-  if ((p->path == EPIC_PATH_FUSED && !p->pair) || (p->path == EPIC_PATH_UNFUSED && !p->wide)) {
+  if (p->path == EPIC_PATH_FUSED ? !p->pair : (p->path == EPIC_PATH_UNFUSED && !p->wide)) {
     const int n1 = p->path == EPIC_PATH_FUSED ? epic::image_fft_lanes(N) : epic::unfused_fft_lanes(N);
     if (epic_status st = build_gather(p, wts, n1, true, gofs, gcnt, gent, gbase)) {
       epic_plan_destroy(p);
@@ -1628,6 +1680,7 @@ epic_status epic_image(epic_plan_t p, const void* d_volt, long long n_time, doub
   if (p->precision != EPIC_PREC_FP32) return image_tc(p, d_volt, n_time, d_image);
   if (p->path == EPIC_PATH_CLUSTER) return image_cluster(p, d_volt, n_time, d_image);
   if (p->path == EPIC_PATH_UNFUSED) return image_unfused(p, d_volt, n_time, d_image);
+  if (p->wide && !(p->cal && p->npix > 0) && wide_ready(p, n_time)) return image_wide(p, d_volt, n_time, d_image);
   epic::ImageArgs a = fused_args(p, d_volt, n_time, d_image, 1.0 / static_cast<double>(n_time));
   if (p->cal && p->npix > 0) {
     if (epic_status st = ensure_ptap(p, n_time)) return st;
@@ -2354,7 +2407,7 @@ epic_status epic_graph_capture(epic_plan_t p, const void* d_volt, long long n_ti
   if (p->cal && p->frames != 0)
     return fail(EPIC_ERR_STATE, "update EPICal before capturing (frames are pending)");
   if (epic_status st = ensure_ptap(p, n_time)) return st;    // multiple-pixel taps
-  if (p->path == EPIC_PATH_UNFUSED) {
+  if (p->path == EPIC_PATH_UNFUSED || p->wide) {
     // allocate the batch scratch outside the capture
     const bool cal = p->cal;
     const long long frames = p->frames;

@@ -1,5 +1,6 @@
-// Frame-pair form of the plain FP32 path for N = 256 and 512 (sm_103a): the
-// row spectra of a batch of frames go through HBM, two frames per FP32 pair.
+// Frame-pair form of the plain FP32 path for N = 256 and 512, and of N = 128
+// where the footprint does not fit one SM (sm_103a): the row spectra of a
+// batch of frames go through HBM, two frames per FP32 pair.
 //
 //   wide_rows    per (channel, frame pair): E' = E / g (Eq. 8) of every
 //                antenna into shared memory, then by blocks of RB grid rows
@@ -11,6 +12,18 @@
 //                one is transformed (Eq. 10); |E|^2 stays in registers, the
 //                calibrator pixel is stored per frame.
 // The correlation kernel of the plain path follows.
+//
+// What bounds it: latency with the 8 warps per SM that 32-output tasks leave
+// (255 registers), the FP32 pipe at 65 % in the column kernel (packed
+// instructions take two cycles, three with distinct operands), at 27 % in the
+// row kernel, whose loads and gridding share the shared-memory pipe (51 %).
+// 8192 frames of 1024 antennas, 256 x 256: rows 0.47, columns 0.55 ms, HBM 2.7
+// and 2.6 TB/s.  16-output tasks would need twice the loads; three CTAs per SM
+// (168 registers) were slower in the row kernel (17.0 against 16.6 ms).  4096
+// samples of 32 channels: 16.6 ms against 38.1 for the one-frame kernels; 2048
+// antennas, 512 x 512, 128 complex64 samples of 256 channels 23.5 against 53.4;
+// 200 antennas on 76 of 128 grid rows, 16 channels, 2000 samples 1.34 against
+// 1.57 for the one-frame fused kernel.
 //
 // Gridding: one lane per grid cell; the cells of a row block sorted by their
 // number of taps in slices of 32 (empty cells last, stored as zeros, since
@@ -33,7 +46,7 @@ using fft::f2_pack;
 using fft::f2_splat;
 using fft::f32x2;
 
-constexpr int kWBT = 128;          // threads; two CTAs per SM (255 registers each)
+constexpr int kWBT = 128;          // threads of the row kernel; two CTAs per SM (255 registers each)
 constexpr int kWP = 32;            // outputs per task
 // Frame pairs per FP32 partial image (FP64 across), as in the fused form.
 constexpr int kWideRun = 128;
@@ -42,7 +55,8 @@ template <int N>
 struct WGeo {
   static constexpr int NR = N / kWP;                 // residues
   static constexpr int RB = kWBT / NR;               // grid rows per block
-  static constexpr int NCOL = kWBT / NR;             // columns per block
+  static constexpr int CT = N == 128 ? 64 : 128;     // threads of the column kernel, 256 per SM
+  static constexpr int NCOL = CT / NR;               // columns per block
   static constexpr int CB = N / NCOL;                // column blocks
 };
 
@@ -221,7 +235,7 @@ __global__ void __launch_bounds__(kWBT, 2) wide_rows_kernel(const WideArgs W, lo
 }
 
 template <int N>
-__global__ void __launch_bounds__(kWBT, 2) wide_cols_kernel(const WideArgs W, int nt) {
+__global__ void __launch_bounds__(WGeo<N>::CT, 256 / WGeo<N>::CT) wide_cols_kernel(const WideArgs W, int nt) {
   using G = WGeo<N>;
   constexpr int NR = G::NR, NCOL = G::NCOL, CB = G::CB;
   const UnfusedArgs& A = W.u;
@@ -232,7 +246,7 @@ __global__ void __launch_bounds__(kWBT, 2) wide_cols_kernel(const WideArgs W, in
   float2* wq = tw + N;                                       // [NR][NR]
   __shared__ uint64_t bars[2];
   __shared__ int abort_flag;
-  residue_tables<N, NR>(A.twid, tw, wq, kWBT);
+  residue_tables<N, NR>(A.twid, tw, wq, G::CT);
   if (tid == 0) {
     mbar_init_one(bars, 2);
     abort_flag = 0;
@@ -319,7 +333,8 @@ cudaError_t prepare_n(const WideArgs& w, int fmt, int* rows_per_sm, int* cols_pe
   if (e == cudaSuccess) e = cudaFuncSetAttribute(wide_cols_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, room);
   if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(rows_per_sm, rk, kWBT, rows_smem<N>(w));
   if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(cols_per_sm, wide_cols_kernel<N>, kWBT, cols_smem<N>(w));
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(cols_per_sm, wide_cols_kernel<N>,
+                                                      WGeo<N>::CT, cols_smem<N>(w));
   return e;
 }
 
@@ -333,18 +348,19 @@ cudaError_t launch_n(const WideArgs& w, long long t0, int nt, cudaStream_t s) {
   if (e != cudaSuccess) return e;
   const long long cu = pairs * WGeo<N>::CB;
   const long long cg = cu < w.cols_ctas ? cu : w.cols_ctas;
-  wide_cols_kernel<N><<<static_cast<unsigned>(cg), kWBT, cols_smem<N>(w), s>>>(w, nt);
+  wide_cols_kernel<N><<<static_cast<unsigned>(cg), WGeo<N>::CT, cols_smem<N>(w), s>>>(w, nt);
   return cudaGetLastError();
 }
 
 }  // namespace
 
-bool wide_supported(int n) { return n == 256 || n == 512; }
+bool wide_supported(int n) { return n == 128 || n == 256 || n == 512; }
 
-int wide_row_block(int n) { return n == 256 ? WGeo<256>::RB : n == 512 ? WGeo<512>::RB : 0; }
+int wide_row_block(int n) { return n == 128 ? WGeo<128>::RB : n == 256 ? WGeo<256>::RB : n == 512 ? WGeo<512>::RB : 0; }
 
 cudaError_t wide_prepare(const WideArgs& w, int fmt, int* rows_per_sm, int* cols_per_sm) {
   switch (w.u.grid_n) {
+    case 128: return prepare_n<128>(w, fmt, rows_per_sm, cols_per_sm);
     case 256: return prepare_n<256>(w, fmt, rows_per_sm, cols_per_sm);
     case 512: return prepare_n<512>(w, fmt, rows_per_sm, cols_per_sm);
     default: return cudaErrorInvalidValue;
@@ -353,6 +369,7 @@ cudaError_t wide_prepare(const WideArgs& w, int fmt, int* rows_per_sm, int* cols
 
 cudaError_t launch_wide_batch(const WideArgs& w, long long t0, int nt, cudaStream_t s) {
   switch (w.u.grid_n) {
+    case 128: return launch_n<128>(w, t0, nt, s);
     case 256: return launch_n<256>(w, t0, nt, s);
     case 512: return launch_n<512>(w, t0, nt, s);
     default: return cudaErrorInvalidValue;

@@ -1,4 +1,5 @@
-"""Frame-pair form of the plain path (N = 256, 512) against the FP64 oracle at
+"""Frame-pair form through HBM (N = 256, 512, and N = 128 with a footprint
+too large for one SM) against the FP64 oracle at
 the edges of its tiles: sample counts around a pair and a batch, footprints
 around the 4-row, row-block and 32-entry edges, one channel and several,
 scratch budgets of one pair and of part of the channels, both voltage
@@ -25,7 +26,8 @@ def _built():
     (256, 40, 17, 33, 1, 1, "ci4", 3, 0), (256, 300, 96, 129, 5, 3, "c64", 5, 1 << 21),
     (256, 700, 250, 61, 4, 2, "ci4", 3, 1), (256, 90, 32, 32, 260, 1, "c64", 1, 0),
     (512, 60, 8, 40, 3, 2, "ci4", 3, 0), (512, 500, 261, 257, 2, 2, "c64", 3, 3 << 20),
-    (512, 200, 505, 500, 2, 1, "ci4", 3, 0),
+    (512, 200, 505, 500, 2, 1, "ci4", 3, 0), (128, 90, 97, 101, 67, 3, "ci4", 3, 0),
+    (128, 200, 127, 90, 9, 2, "c64", 5, 0), (128, 700, 70, 127, 3, 2, "ci4", 3, 1 << 20),
 ])
 def test_wide_interval(n, na, rows, cols, T, C, fmt, support, budget):
     from paper_1603_02126_gb300 import Plan
@@ -46,8 +48,8 @@ def test_wide_interval(n, na, rows, cols, T, C, fmt, support, budget):
     else:
         E = E.astype(np.complex64).astype(np.complex128)
         dev = torch.from_numpy(E.astype(np.complex64)).cuda()
-    p = Plan(ant, freqs, n, 0.5, support=support, input=fmt, voltage_scale=lsb, path="unfused",
-             workspace_bytes=budget)
+    p = Plan(ant, freqs, n, 0.5, support=support, input=fmt, voltage_scale=lsb,
+             path="fused" if n == 128 else "unfused", workspace_bytes=budget)
     g0 = synth.true_gains(C, na, rng)
     p.configure((0.0, 0.0), sky, 0.5, g0=g0)
     img = p.image(dev).cpu().numpy()
