@@ -529,33 +529,71 @@ constexpr uint32_t kXeStageBytes = kChunkBytes + kXeN * 128;
 
 size_t xe_smem_bytes() { return 1024 + kXeStages * kXeStageBytes + 256; }
 
-// volt [T][C][Na] 4-bit -> Z [C][2 Na_p][Tp] FP16; block = (channel, 32
-// antennas, 64 samples); thread = (row r of the 64, 16 samples).
-__global__ void __launch_bounds__(256) xe_pack_kernel(const unsigned char* __restrict__ volt, long long t0,
-                                                      int nt, int n_chan, int n_ant, int na_p, int tp,
+// volt [T][C][Na] 4-bit -> Z [C][2 Na_p][Tp] FP16.  A warp takes 32 antennas
+// x 32 samples: a lane loads the bytes of 4 antennas (one word where rows are
+// word-aligned: ALIGNED) at 8 samples, transposes them in registers and
+// stores 8 samples of each of its 8 rows as 16 bytes, four lanes a 64-byte
+// run.  A nibble n becomes the half 1024 + (n ^ 8) by its bits, minus 1032.
+//
+// Bound by HBM (1 byte read, 4 written per sample): 64 channels x 256
+// antennas x 4254 samples 51 us, 6.9 TB/s (155 us with bytes through shared
+// memory).
+template <bool ALIGNED>
+__global__ void __launch_bounds__(256) xe_pack_kernel(const unsigned char* __restrict__ volt, long long t0, int nt,
+                                                      int n_chan, int n_ant, int na_p, int tp,
                                                       __half* __restrict__ z) {
-  __shared__ unsigned char tile[64][33];
-  const int c = blockIdx.x, ab = blockIdx.y * 32, tb = blockIdx.z * 64;
-  for (int i = threadIdx.x; i < 64 * 32; i += 256) {
-    const int tt = i / 32, k = i % 32;
-    const int t = tb + tt, a = ab + k;
-    tile[tt][k] = (t < nt && a < n_ant)
-                      ? __ldg(volt + (static_cast<size_t>(t0 + t) * n_chan + c) * n_ant + a)
-                      : static_cast<unsigned char>(0);
-  }
-  __syncthreads();
-  const int r = threadIdx.x / 4, q = threadIdx.x % 4;     // row 2k + s of the block, 16-sample quarter
-  const int k = r >> 1, sgn = r & 1;
-  __align__(16) __half v[16];
+  const int lane = threadIdx.x & 31;
+  const int tb_n = tp / 32, per = (na_p / 32 * tb_n + 7) / 8;   // blocks per channel
+  const int c = blockIdx.x / per, warp = (blockIdx.x - c * per) * 8 + (threadIdx.x >> 5);
+  const int ab = warp / tb_n, tb = warp - ab * tb_n;         // blocks of 32 antennas, of 32 samples
+  if (ab * 32 >= na_p) return;
+  const int a = ab * 32 + (lane >> 2) * 4, t = tb * 32 + (lane & 3) * 8;
+  unsigned w[8];
 #pragma unroll
-  for (int j = 0; j < 16; ++j) {
-    const unsigned b = tile[q * 16 + j][k];
-    const int x = sgn ? static_cast<int>(b << 28) >> 28 : static_cast<int>(b << 24) >> 28;
-    v[j] = __int2half_rn(x);
+  for (int i = 0; i < 8; ++i) {
+    w[i] = 0;
+    if (t + i < nt) {
+      const unsigned char* src = volt + (static_cast<size_t>(t0 + t + i) * n_chan + c) * n_ant + a;
+      if (ALIGNED) {
+        if (a < n_ant) w[i] = __ldg(reinterpret_cast<const unsigned*>(src));
+      } else {
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (a + k < n_ant) w[i] |= static_cast<unsigned>(__ldg(src + k)) << (8 * k);
+      }
+    }
   }
-  __half* dst = z + (static_cast<size_t>(c) * 2 * na_p + 2 * ab + r) * tp + tb + q * 16;
-  reinterpret_cast<uint4*>(dst)[0] = reinterpret_cast<const uint4*>(v)[0];
-  reinterpret_cast<uint4*>(dst)[1] = reinterpret_cast<const uint4*>(v)[1];
+  // bytes [sample][antenna] -> [antenna][sample], 4 x 4 at a time
+  unsigned x[4][2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const unsigned p0 = __byte_perm(w[4 * h], w[4 * h + 1], 0x5140), p1 = __byte_perm(w[4 * h + 2], w[4 * h + 3], 0x5140);
+    const unsigned q0 = __byte_perm(w[4 * h], w[4 * h + 1], 0x7362), q1 = __byte_perm(w[4 * h + 2], w[4 * h + 3], 0x7362);
+    x[0][h] = __byte_perm(p0, p1, 0x5410);
+    x[1][h] = __byte_perm(p0, p1, 0x7632);
+    x[2][h] = __byte_perm(q0, q1, 0x5410);
+    x[3][h] = __byte_perm(q0, q1, 0x7632);
+  }
+  const __half2 off = __floats2half2_rn(1032.f, 1032.f);
+  __half* dst = z + (static_cast<size_t>(c) * 2 * na_p + 2 * a) * tp + t;
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {                            // Re: high nibble, Im: low nibble
+      uint4 o;
+      unsigned* v = &o.x;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const unsigned n = ((s ? x[k][h] : x[k][h] >> 4) & 0x0f0f0f0fu) ^ 0x08080808u;
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const unsigned m = __byte_perm(n, 0x64u, e ? 0x4342 : 0x4140);
+          const __half2 r = __hsub2(*reinterpret_cast<const __half2*>(&m), off);
+          v[2 * h + e] = *reinterpret_cast<const unsigned*>(&r);
+        }
+      }
+      *reinterpret_cast<uint4*>(dst + static_cast<size_t>(2 * k + s) * tp) = o;
+    }
 }
 
 __global__ void __launch_bounds__(kXeThreads, 1)
@@ -1044,9 +1082,12 @@ bool xe_make_map(void* z, int n_chan, int na_p, int tp, void* tm) {
 
 cudaError_t launch_xengine_tc(const XeTcArgs& a, const void* volt, long long t0, int nt, void* z, const void* tm,
                               int sms, cudaStream_t s) {
-  dim3 pg(static_cast<unsigned>(a.n_chan), static_cast<unsigned>(a.na_p / 32), static_cast<unsigned>(a.tp / 64));
-  xe_pack_kernel<<<pg, 256, 0, s>>>(static_cast<const unsigned char*>(volt), t0, nt, a.n_chan, a.n_ant, a.na_p,
-                                    a.tp, static_cast<__half*>(z));
+  const int warps = a.na_p / 32 * (a.tp / 32);
+  const unsigned pg = static_cast<unsigned>((warps + 7) / 8) * static_cast<unsigned>(a.n_chan);
+  const unsigned char* v = static_cast<const unsigned char*>(volt);
+  const bool aligned = a.n_ant % 4 == 0 && reinterpret_cast<uintptr_t>(volt) % 4 == 0;
+  if (aligned) xe_pack_kernel<true><<<pg, 256, 0, s>>>(v, t0, nt, a.n_chan, a.n_ant, a.na_p, a.tp, static_cast<__half*>(z));
+  else xe_pack_kernel<false><<<pg, 256, 0, s>>>(v, t0, nt, a.n_chan, a.n_ant, a.na_p, a.tp, static_cast<__half*>(z));
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const int nb = 2 * a.na_p / kTile, nbp = (nb + 1) / 2;
