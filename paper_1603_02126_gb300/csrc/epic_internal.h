@@ -146,7 +146,9 @@ cudaError_t launch_model_vis(int n_chan, int n_ant, int n_src, const double2* ph
                              float2* vm, cudaStream_t s);
 struct StefcalArgs {
   int n_chan, n_ant;
-  float2* vis32;           // [C][Na][Na] scratch: the visibilities rounded to FP32
+  float2* w;               // [C][Na][ld] scratch: pair terms V conj(V^M) in FP32
+  float* m2;               // [C][Na][ld] scratch: |V^M|^2
+  int ld, rows;            // row stride of both; antennas per CTA (set by the launch)
   const float2* vm;        // [C][Na][Na] model visibilities (FP32)
   const double2* uv;       // [C][Na] antenna positions in wavelengths
   const unsigned char* flags;
@@ -156,8 +158,9 @@ struct StefcalArgs {
   double2* gains;          // [C][Na] in: start, out: solution
   int* iters;              // [C] iterations used, or nullptr
 };
-// Rounds vis64 into a.vis32, then solves.
-cudaError_t launch_stefcal(const StefcalArgs& a, const double2* vis64, cudaStream_t s);
+// Forms the pair terms of vis64, then solves.
+int stefcal_ld(int n_ant);
+cudaError_t launch_stefcal(const StefcalArgs& a, const double2* vis64, int sms, cudaStream_t s);
 int image_rs(int rows_alloc);
 int image_rs_fused(int rows_alloc);
 

@@ -11,10 +11,10 @@
 //   model_vis    V^M[c][a][b] = sum_s S_s e_a(s) conj(e_b(s)), e_a(s) =
 //                e^{-2 pi i u_a . s}, FP64 from host phasors, kept in FP32.
 //   stefcal      Eq. 21 by alternating least squares with every other iterate
-//                averaged (StEFCal): one CTA per channel, one warp per antenna
-//                row at a time, FP32 products with FP64 reductions and
-//                update, iterated in the kernel until
-//                max_a |g_new - g| <= tol max_a |g_new| or max_iter.
+//                averaged (StEFCal): a cluster of CTAs per channel, iterated
+//                in the kernel until max_a |g_new - g| <= tol max_a |g_new| or
+//                max_iter.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -137,117 +137,205 @@ __global__ void model_vis_kernel(int n_chan, int n_ant, int n_src, const double2
   vm[i] = make_float2(static_cast<float>(re), static_cast<float>(im));
 }
 
-__global__ void to_f32_kernel(long long n, const double2* __restrict__ in, float2* __restrict__ out) {
-  const long long stride = static_cast<long long>(gridDim.x) * blockDim.x;
-  for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < n; i += stride) {
-    const double2 v = in[i];
-    out[i] = make_float2(static_cast<float>(v.x), static_cast<float>(v.y));
-  }
-}
-
 constexpr int kSThreads = 1024;
 constexpr double kStefcalMinTol = 1e-6;   // smallest stopping tolerance with FP32 pair products
 
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
+// Pair terms of the solve, once per call: W_ab = V_ab conj(V^M_ab) and
+// |V^M_ab|^2 in FP32, zero for the pairs that are left out (autos, flagged
+// antennas, baselines below the cut) and in the padding of a row.
+__global__ void __launch_bounds__(128) pair_terms_kernel(const StefcalArgs A, const double2* __restrict__ vis) {
+  const int Na = A.n_ant, ld = A.ld;
+  const long long row = blockIdx.x;                          // channel * Na + antenna
+  const int c = static_cast<int>(row / Na), a = static_cast<int>(row - static_cast<long long>(c) * Na);
+  const double mb2 = A.min_baseline * A.min_baseline;
+  const bool live = !A.flags[a];
+  for (int b = threadIdx.x; b < ld; b += 128) {
+    float2 w = make_float2(0.f, 0.f);
+    float m2 = 0.f;
+    bool use = live && b < Na && b != a && !A.flags[b];
+    if (use && mb2 > 0.0) {
+      const double2 ua = A.uv[row], ub = A.uv[static_cast<size_t>(c) * Na + b];
+      const double dx = ua.x - ub.x, dy = ua.y - ub.y;
+      use = !(dx * dx + dy * dy < mb2);
+    }
+    if (use) {
+      const float2 m = A.vm[row * Na + b];
+      const double2 v = vis[row * Na + b];
+      const float vr = static_cast<float>(v.x), vi = static_cast<float>(v.y);
+      w = make_float2(fmaf(vr, m.x, vi * m.y), fmaf(vi, m.x, -vr * m.y));
+      m2 = fmaf(m.x, m.x, m.y * m.y);
+    }
+    A.w[row * ld + b] = w;
+    A.m2[row * ld + b] = m2;
+  }
 }
 
-// One CTA per channel.  The per-pair products run in FP32 (V and V^M
-// rounded to FP32, this GPU's FP64 rate being a small fraction of its FP32
-// rate); each lane's partial sums go to FP64 for the warp reduction, the
-// division, the averaging and the convergence test.  Shared memory: g (FP64)
-// and gn [Na], g as FP32 [Na].
-__global__ void __launch_bounds__(kSThreads) stefcal_kernel(const StefcalArgs A) {
-  extern __shared__ __align__(16) double2 sg[];
-  double2* g = sg;
-  double2* gn = sg + A.n_ant;
-  float2* gf = reinterpret_cast<float2*>(sg + 2 * A.n_ant);
-  __shared__ double red_d[kSThreads / 32], red_m[kSThreads / 32];
-  __shared__ int done;
-  const int c = blockIdx.x, Na = A.n_ant;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = kSThreads / 32;
-  const float2* V = A.vis32 + static_cast<size_t>(c) * Na * Na;
-  const float2* VM = A.vm + static_cast<size_t>(c) * Na * Na;
-  const double2* uv = A.uv + static_cast<size_t>(c) * Na;
-  const double mb2 = A.min_baseline * A.min_baseline;
-  double2* gio = A.gains + static_cast<size_t>(c) * Na;
-  for (int a = threadIdx.x; a < Na; a += kSThreads) {
-    g[a] = gio[a];
-    gf[a] = make_float2(static_cast<float>(g[a].x), static_cast<float>(g[a].y));
+// A sum as hi + lo (FP32 each, error-free two-sum: about 48 bits).
+struct Sum2 {
+  float hi, lo;
+  __device__ __forceinline__ void add(float h, float l) {
+    const float s = hi + h, t = s - hi;
+    lo += l + ((hi - (s - t)) + (h - t));
+    hi = s;
   }
-  if (threadIdx.x == 0) done = 0;
-  __syncthreads();
-  int it = 0;
-  for (; it < A.max_iter; ++it) {
-    for (int a = warp; a < Na; a += nw) {
-      float nr = 0.f, ni = 0.f, den = 0.f;
-      if (!A.flags[a]) {
-        const double2 ua = uv[a];
-        for (int b = lane; b < Na; b += 32) {
-          if (b == a || A.flags[b]) continue;
-          if (mb2 > 0.0) {
-            const double2 ub = uv[b];
-            const double dx = ua.x - ub.x, dy = ua.y - ub.y;
-            if (dx * dx + dy * dy < mb2) continue;
-          }
-          const float2 gb = gf[b];
-          const float2 m = VM[static_cast<size_t>(a) * Na + b];
-          const float2 v = V[static_cast<size_t>(a) * Na + b];
-          // z = g_b conj(VM_ab)
-          const float zr = fmaf(gb.x, m.x, gb.y * m.y), zi = fmaf(gb.y, m.x, -gb.x * m.y);
-          nr = fmaf(v.x, zr, fmaf(-v.y, zi, nr));
-          ni = fmaf(v.x, zi, fmaf(v.y, zr, ni));
-          den = fmaf(zr, zr, fmaf(zi, zi, den));
-        }
-      }
-      const double snr = warp_sum(static_cast<double>(nr));
-      const double sni = warp_sum(static_cast<double>(ni));
-      const double sden = warp_sum(static_cast<double>(den));
-      if (lane == 0) gn[a] = sden > 0.0 ? make_double2(snr / sden, sni / sden) : g[a];
-    }
-    __syncthreads();
-    double dmax = 0.0, gmax = 0.0;
-    for (int a = threadIdx.x; a < Na; a += kSThreads) {
-      double2 x = gn[a];
-      const double2 o = g[a];
-      if (it & 1) x = make_double2(0.5 * (x.x + o.x), 0.5 * (x.y + o.y));
-      gn[a] = x;
-      dmax = fmax(dmax, hypot(x.x - o.x, x.y - o.y));
-      gmax = fmax(gmax, hypot(x.x, x.y));
+};
+
+// Sums over the warp of three values of four rows: lane 8 j ends with row j's.
+__device__ __forceinline__ void sum_rows(const float (&v)[4][3], Sum2 (&out)[3]) {
+  const int lane = threadIdx.x & 31;
+  Sum2 h[2][3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const float keep = lane & 16 ? v[2 + i][k] : v[i][k], send = lane & 16 ? v[i][k] : v[2 + i][k];
+      h[i][k] = Sum2{keep, 0.f};
+      h[i][k].add(__shfl_xor_sync(0xffffffffu, send, 16), 0.f);
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      dmax = fmax(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
-      gmax = fmax(gmax, __shfl_xor_sync(0xffffffffu, gmax, o));
-    }
-    if (lane == 0) {
-      red_d[warp] = dmax;
-      red_m[warp] = gmax;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double d = 0.0, m = 0.0;
-      for (int w = 0; w < nw; ++w) {
-        d = fmax(d, red_d[w]);
-        m = fmax(m, red_m[w]);
-      }
-      // FP32 pair products: changes below ~1e-6 are rounding, not progress
-      done = (d <= fmax(A.tol, kStefcalMinTol) * m) ? 1 : 0;
-    }
-    for (int a = threadIdx.x; a < Na; a += kSThreads) {
-      g[a] = gn[a];
-      gf[a] = make_float2(static_cast<float>(gn[a].x), static_cast<float>(gn[a].y));
-    }
-    __syncthreads();
-    if (done) {
-      ++it;
-      break;
-    }
+  for (int k = 0; k < 3; ++k) {
+    const Sum2 keep = lane & 8 ? h[1][k] : h[0][k], send = lane & 8 ? h[0][k] : h[1][k];
+    out[k] = keep;
+    out[k].add(__shfl_xor_sync(0xffffffffu, send.hi, 8), __shfl_xor_sync(0xffffffffu, send.lo, 8));
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1)
+      out[k].add(__shfl_xor_sync(0xffffffffu, out[k].hi, o), __shfl_xor_sync(0xffffffffu, out[k].lo, o));
   }
-  for (int a = threadIdx.x; a < Na; a += kSThreads) gio[a] = g[a];
-  if (threadIdx.x == 0 && A.iters) A.iters[c] = it;
+}
+
+// Eq. 21 by alternating least squares: g_a <- sum_b W_ab g_b / sum_b |V^M_ab|^2
+// |g_b|^2, every other iterate averaged.  A cluster of CTAs per channel, each
+// with a block of antenna rows; a warp sums four rows at a time (FP32
+// products, two-float sums across the lanes: this GPU's FP64 rate is 1/73 of
+// its FP32 rate, and the FP64 lane reductions took a third of an iteration),
+// one thread per antenna divides, averages and tests in FP64 and writes the
+// new gain, rounded to FP32, into every CTA's shared memory; one cluster
+// barrier per iteration.
+//
+// What bounds it: W and |V^M|^2 (12 bytes a pair) come through L2 once per
+// iteration, the division and a cluster barrier follow in series.
+__global__ void __launch_bounds__(kSThreads) stefcal_kernel(const StefcalArgs A) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  extern __shared__ __align__(16) unsigned char ssm[];
+  const int Na = A.n_ant, ld = A.ld, rows = A.rows;
+  float2* gf = reinterpret_cast<float2*>(ssm);               // [2][ld] gains as FP32 (flagged and padding: 0)
+  float* g2 = reinterpret_cast<float*>(gf + 2 * ld);         // [2][ld] |g|^2
+  double2* g = reinterpret_cast<double2*>(g2 + 2 * ld);      // [rows] own gains
+  float* sums = reinterpret_cast<float*>(g + rows);          // [rows][6] (hi, lo) of Re, Im, denominator
+  __shared__ unsigned long long most[2][2];                  // by parity: largest |change|^2, |g|^2 of this CTA
+  __shared__ unsigned long long all[2][2][8];                // the same of every CTA of the cluster
+  const int cl = static_cast<int>(cluster.num_blocks()), q = static_cast<int>(cluster.block_rank());
+  const int c = blockIdx.x / cl;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int a0 = q * rows, na = Na - a0 < rows ? (Na - a0 > 0 ? Na - a0 : 0) : rows;   // own antennas
+  const float2* W = A.w + static_cast<size_t>(c) * Na * ld;
+  const float* M = A.m2 + static_cast<size_t>(c) * Na * ld;
+  double2* gio = A.gains + static_cast<size_t>(c) * Na;
+  for (int a = threadIdx.x; a < ld; a += kSThreads) {
+    const double2 v = a < Na ? gio[a] : make_double2(0.0, 0.0);
+    const bool live = a < Na && !A.flags[a];
+    const float2 f = live ? make_float2(static_cast<float>(v.x), static_cast<float>(v.y)) : make_float2(0.f, 0.f);
+    gf[a] = f;
+    gf[ld + a] = make_float2(0.f, 0.f);
+    g2[a] = fmaf(f.x, f.x, f.y * f.y);
+    g2[ld + a] = 0.f;
+    if (a >= a0 && a < a0 + na) g[a - a0] = v;
+  }
+  if (threadIdx.x < 4) most[threadIdx.x >> 1][threadIdx.x & 1] = 0ull;
+  cluster.sync();                                            // every CTA is resident and has read the gains
+  const double tol = fmax(A.tol, kStefcalMinTol), tol2 = tol * tol;
+  int it = 0;
+  for (; it < A.max_iter;) {
+    const int cur = it & 1, nxt = cur ^ 1;
+    const float4* gp = reinterpret_cast<const float4*>(gf + cur * ld);
+    const float4* hp = reinterpret_cast<const float4*>(g2 + cur * ld);
+    for (int r = 4 * warp; r < na; r += 4 * (kSThreads / 32)) {
+      float v[4][3];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) v[i][0] = v[i][1] = v[i][2] = 0.f;
+      for (int b = lane; 4 * b < ld; b += 32) {              // antennas 4 b .. 4 b + 3
+        const float4 x0 = gp[2 * b], x1 = gp[2 * b + 1], y = hp[b];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int row = a0 + (r + i < na ? r + i : r);
+          const float4* wp = reinterpret_cast<const float4*>(W + static_cast<size_t>(row) * ld);
+          const float4 w0 = __ldg(wp + 2 * b), w1 = __ldg(wp + 2 * b + 1);
+          const float4 m = __ldg(reinterpret_cast<const float4*>(M + static_cast<size_t>(row) * ld) + b);
+          v[i][0] = fmaf(w0.x, x0.x, fmaf(-w0.y, x0.y, v[i][0]));
+          v[i][1] = fmaf(w0.x, x0.y, fmaf(w0.y, x0.x, v[i][1]));
+          v[i][0] = fmaf(w0.z, x0.z, fmaf(-w0.w, x0.w, v[i][0]));
+          v[i][1] = fmaf(w0.z, x0.w, fmaf(w0.w, x0.z, v[i][1]));
+          v[i][0] = fmaf(w1.x, x1.x, fmaf(-w1.y, x1.y, v[i][0]));
+          v[i][1] = fmaf(w1.x, x1.y, fmaf(w1.y, x1.x, v[i][1]));
+          v[i][0] = fmaf(w1.z, x1.z, fmaf(-w1.w, x1.w, v[i][0]));
+          v[i][1] = fmaf(w1.z, x1.w, fmaf(w1.w, x1.z, v[i][1]));
+          v[i][2] = fmaf(m.x, y.x, fmaf(m.y, y.y, fmaf(m.z, y.z, fmaf(m.w, y.w, v[i][2]))));
+        }
+      }
+      Sum2 t[3];
+      sum_rows(v, t);
+      const int row = r + (lane >> 3);
+      if ((lane & 7) == 0 && row < na) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          sums[row * 6 + 2 * k] = t[k].hi;
+          sums[row * 6 + 2 * k + 1] = t[k].lo;
+        }
+      }
+    }
+    __syncthreads();
+    for (int r = threadIdx.x; r < na; r += kSThreads) {
+      const float* s = sums + 6 * r;
+      const double den = static_cast<double>(s[4]) + static_cast<double>(s[5]);
+      const double2 o = g[r];
+      double2 x = o;
+      if (den > 0.0) {
+        x.x = (static_cast<double>(s[0]) + static_cast<double>(s[1])) / den;
+        x.y = (static_cast<double>(s[2]) + static_cast<double>(s[3])) / den;
+      }
+      if (it & 1) x = make_double2(0.5 * (x.x + o.x), 0.5 * (x.y + o.y));
+      const double dx = x.x - o.x, dy = x.y - o.y;
+      g[r] = x;
+      // non-negative doubles order as their bits; NaN is passed over
+      const double d2 = dx * dx + dy * dy, x2 = x.x * x.x + x.y * x.y;
+      if (d2 >= 0.0) atomicMax(&most[cur][0], static_cast<unsigned long long>(__double_as_longlong(d2)));
+      if (x2 >= 0.0) atomicMax(&most[cur][1], static_cast<unsigned long long>(__double_as_longlong(x2)));
+      if (!A.flags[a0 + r]) {
+        const float2 f = make_float2(static_cast<float>(x.x), static_cast<float>(x.y));
+        const float h = fmaf(f.x, f.x, f.y * f.y);
+        for (int d = 0; d < cl; ++d) {
+          cluster.map_shared_rank(gf, d)[nxt * ld + a0 + r] = f;
+          cluster.map_shared_rank(g2, d)[nxt * ld + a0 + r] = h;
+        }
+      }
+    }
+    __syncthreads();
+    if (threadIdx.x < cl) {
+      unsigned long long(*dst)[2][8] = cluster.map_shared_rank(all, static_cast<int>(threadIdx.x));
+      dst[cur][0][q] = most[cur][0];
+      dst[cur][1][q] = most[cur][1];
+    }
+    if (threadIdx.x < 2) most[nxt][threadIdx.x] = 0ull;
+    cluster.sync();
+    ++it;
+    unsigned long long d = 0, m = 0;
+    for (int k = 0; k < cl; ++k) {
+      d = all[cur][0][k] > d ? all[cur][0][k] : d;
+      m = all[cur][1][k] > m ? all[cur][1][k] : m;
+    }
+    // FP32 pair products: changes below ~1e-6 are rounding, not progress
+    if (__longlong_as_double(static_cast<long long>(d)) <= tol2 * __longlong_as_double(static_cast<long long>(m))) break;
+  }
+  for (int r = threadIdx.x; r < na; r += kSThreads) gio[a0 + r] = g[r];
+  if (threadIdx.x == 0 && q == 0 && A.iters) A.iters[c] = it;
+}
+
+// CTAs per channel: as many as fill the GPU, up to 8 (a portable cluster),
+// and as many as the gains' shared memory needs; rows per CTA a multiple of 4.
+size_t stefcal_smem(int ld, int rows) {
+  return static_cast<size_t>(2 * ld) * (sizeof(float2) + sizeof(float)) +
+         static_cast<size_t>(rows) * (sizeof(double2) + 6 * sizeof(float));
 }
 
 }  // namespace
@@ -268,16 +356,38 @@ cudaError_t launch_model_vis(int n_chan, int n_ant, int n_src, const double2* ph
   return cudaGetLastError();
 }
 
-cudaError_t launch_stefcal(const StefcalArgs& a, const double2* vis64, cudaStream_t s) {
-  const long long nv = static_cast<long long>(a.n_chan) * a.n_ant * a.n_ant;
-  to_f32_kernel<<<static_cast<unsigned>(std::min<long long>((nv + 255) / 256, 152 * 16)), 256, 0, s>>>(
-      nv, vis64, a.vis32);
-  const size_t smem = static_cast<size_t>(a.n_ant) * (2 * sizeof(double2) + sizeof(float2));
-  cudaError_t e = cudaFuncSetAttribute(stefcal_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
+int stefcal_ld(int n_ant) { return (n_ant + 3) & ~3; }
+
+// 64 channels x 256 antennas, 50 sources: 0.118 ms and 0.030 for the pair
+// terms (two CTAs a channel), 1.2 ms with one CTA a channel and FP64 lane
+// reductions.
+cudaError_t launch_stefcal(const StefcalArgs& args, const double2* vis64, int sms, cudaStream_t s) {
+  StefcalArgs a = args;
+  a.ld = stefcal_ld(a.n_ant);
+  int cl = 1;
+  while (cl < 8 && (a.n_chan * 2 * cl <= sms && a.n_ant > 32 * cl)) cl *= 2;
+  auto rows_of = [&](int k) { return ((a.n_ant + k - 1) / k + 3) & ~3; };
+  while (cl < 8 && stefcal_smem(a.ld, rows_of(cl)) > 220 * 1024) cl *= 2;
+  a.rows = rows_of(cl);
+  const size_t smem = stefcal_smem(a.ld, a.rows);
+  pair_terms_kernel<<<static_cast<unsigned>(a.n_chan * a.n_ant), 128, 0, s>>>(a, vis64);
+  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  stefcal_kernel<<<a.n_chan, kSThreads, smem, s>>>(a);
-  return cudaGetLastError();
+  e = cudaFuncSetAttribute(stefcal_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(a.n_chan * cl));
+  cfg.blockDim = dim3(kSThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = static_cast<unsigned>(cl);
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, stefcal_kernel, a);
 }
 
 }  // namespace epic
