@@ -376,7 +376,16 @@ struct TcArgs {
   const int4* win4;        // [C] (y0, rows, x0, cols)
   const void* tm_gh;       // host CUtensorMap over gh
   const void* tm_fr;       // host CUtensorMap over the row DFT matrix [2N][kr]
+  // gridding lists by blocks of rb rows, places in a [rb][kr / 2] block
+  const unsigned char* lists;
+  const int2* lists_at;    // [C][nb_max] (offset, bytes) / 16 of each block's lists
+  int nb_max, max_lists, rb;
+  int lists_smem;          // 1: two blocks' lists fit in shared memory
+  const int* row_cost;     // [C + 1] prefix sums of a frame pair's cost
+  const float2* pixel;     // [C][Na] response of the calibrator pixel without phasing
 };
+// Dynamic shared memory of the gridding kernel (max_lists 0: lists through L1).
+size_t tc_grid_smem(int n_ant, int rb, int kr, int max_lists);
 bool tc_make_row_maps(void* gh, void* dftr, long long rows_cap, int n, int kr, bool bf16, void* tm_gh,
                       void* tm_fr);
 bool tc_supported(int n, int rows_alloc);

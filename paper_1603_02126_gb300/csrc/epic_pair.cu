@@ -26,6 +26,7 @@
 // 2000 samples 37.6 against 53.9 us (with the update).
 #include "epic_fft.cuh"
 #include "epic_internal.h"
+#include "epic_lists.cuh"
 #include "epic_residue.cuh"
 
 #include <cstdint>
@@ -35,10 +36,7 @@ namespace {
 
 using fft::Cf2;
 using fft::cmul;
-using fft::f2_fma;
 using fft::f2_pack;
-using fft::f2_splat;
-using fft::f32x2;
 
 // Frame pairs per FP32 partial image (FP64 across): 128 roundings of a running
 // sum, image error 0.9e-7 against 64 bits over 10^4 samples (1.4e-7 at 256).
@@ -48,20 +46,13 @@ constexpr int kPairRun = 128;
 template <int BT>
 __device__ __forceinline__ void grid_pair(const int* __restrict__ cell, const int2* __restrict__ slice,
                                           const uint2* __restrict__ ent, int nslice, const Cf2* Es, Cf2* grid) {
-  const int lane = threadIdx.x & 31;
-  for (int sl = threadIdx.x >> 5; sl < nslice; sl += BT / 32) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int k = 0; k * (BT / 32) < nslice; ++k) {
+    const int sl = slice_of(k, warp, BT / 32);
+    if (sl >= nslice) break;
     const int2 s = slice[sl];
     const int at = cell[sl * 32 + lane];
-    const uint2* e = ent + s.x + lane;
-    Cf2 sum{0ull, 0ull};
-#pragma unroll 2
-    for (int k = 0; k < s.y; ++k) {
-      const uint2 en = e[k * 32];
-      const Cf2 x = *reinterpret_cast<const Cf2*>(reinterpret_cast<const unsigned char*>(Es) + en.x);
-      const f32x2 w = f2_splat(__uint_as_float(en.y));
-      sum.re = f2_fma(w, x.re, sum.re);
-      sum.im = f2_fma(w, x.im, sum.im);
-    }
+    const Cf2 sum = sum_taps(ent + s.x + lane, s.y, Es);
     if (at >= 0) grid[at] = sum;
   }
 }

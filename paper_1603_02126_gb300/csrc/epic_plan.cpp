@@ -203,6 +203,8 @@ struct epic_plan_s {
   alignas(64) unsigned char tm_dft[128];
   alignas(64) unsigned char tm_data[128];
   int kr = 0;                   // K extent of the row DFT (2 x window columns, padded to 64)
+  int tc_rb = 0, tc_lists_smem = 0;   // gridding: rows per block of lists, lists in shared memory
+  DevBuf<float2> d_tc_pixel;    // [C][Na] response of the calibrator pixel without phasing
   DevBuf<uint16_t> d_tc_gh;     // [tc_time*C*rows_alloc][kr] scaled window grid
   DevBuf<uint16_t> d_tc_dftr;   // [2N][kr] row DFT over window columns
   alignas(64) unsigned char tm_gh[128];
@@ -332,6 +334,28 @@ bool nearest_pixel(epic_plan_t p, double l, double m, int* kx, int* ky) {
   *kx = static_cast<int>(kxd);
   *ky = static_cast<int>(kyd);
   return true;
+}
+
+// Response of pixel (kx, ky) to the phased voltages E' of the reduced-precision
+// form, FP32 on the device (the phasing is in E').
+epic_status set_tc_pixel(epic_plan_t p, int kx, int ky) {
+  if (p->precision == EPIC_PREC_FP32) return EPIC_OK;
+  const size_t n = static_cast<size_t>(p->nc) * p->na;
+  std::vector<float2> r(n);
+  std::vector<std::complex<double>> A;
+  for (int c = 0; c < p->nc; ++c) {
+    pixel_response(p, c, kx, ky, A);
+    for (int a = 0; a < p->na; ++a) {
+      const size_t i = static_cast<size_t>(c) * p->na + a;
+      std::complex<double> v = A[a];
+      if (!p->phase.empty()) v *= std::conj(std::complex<double>(p->phase[i].x, p->phase[i].y));
+      r[i] = make_float2(static_cast<float>(v.real()), static_cast<float>(v.imag()));
+    }
+  }
+  if (!p->d_tc_pixel.p && p->d_tc_pixel.alloc(n) != cudaSuccess) return fail(EPIC_ERR_OOM, "EPICal allocation failed");
+  EPIC_CUDA(cudaMemcpyAsync(p->d_tc_pixel.p, r.data(), n * sizeof(float2), cudaMemcpyHostToDevice, p->stream));
+  EPIC_CUDA(cudaStreamSynchronize(p->stream));
+  return EPIC_OK;
 }
 
 // Window-coordinate phase of pixel (kx, ky) in channel c:
@@ -578,8 +602,8 @@ void build_cells(const epic_plan_s* p, const std::vector<float>& wts, int gs, Ce
   prefix_sums(&t->cost);
 }
 
-// Tap lists of the wide frame-pair form: per channel and block of row_block
-// window rows one contiguous piece (header, slices, 16-bit cells, entries;
+// Tap lists of the frame-pair forms that grid by blocks of rb window rows: per
+// channel and block one contiguous piece (header, slices, 16-bit cells, entries;
 // every piece a multiple of 16 bytes), cells without taps included.
 struct WideTables {
   std::vector<unsigned char> lists;
@@ -588,8 +612,9 @@ struct WideTables {
   int nb_max = 0, max_lists = 0;
 };
 
-void build_wide_lists(const epic_plan_s* p, const std::vector<float>& wts, int gs, WideTables* t) {
-  const int rb = epic::wide_row_block(p->n), N = p->n;
+epic_status build_wide_lists(const epic_plan_s* p, const std::vector<float>& wts, int gs, int rb, WideTables* t) {
+  const int N = p->n;
+  *t = WideTables();
   t->nb_max = (p->rows_alloc + rb - 1) / rb;
   t->at.assign(static_cast<size_t>(p->nc) * t->nb_max, make_int2(0, 0));
   SliceLists l;
@@ -605,6 +630,7 @@ void build_wide_lists(const epic_plan_s* p, const std::vector<float>& wts, int g
       for (int r = 0; r < rows; ++r) std::fill_n(inside.begin() + r * gs, p->cols[c], 1);
       slice_lists(taps[b], rb * gs, &inside, p->na, &l);
       const size_t ns = l.slice.size();
+      if (ns && l.slice[0].y > 255) return fail(EPIC_ERR_UNSUPPORTED, "more than 255 gridding taps on one grid cell");
       int hd[4] = {static_cast<int>(ns), 0, 0, 0};
       hd[1] = static_cast<int>((sizeof hd + ns * sizeof(int2) + 15) & ~static_cast<size_t>(15));
       hd[2] = hd[1] + static_cast<int>(ns * 64);
@@ -623,13 +649,16 @@ void build_wide_lists(const epic_plan_s* p, const std::vector<float>& wts, int g
       t->max_lists = std::max(t->max_lists, static_cast<int>(bytes));
       listed += static_cast<long long>(l.ent.size()) + 2 * static_cast<long long>(ns) * 32;
     }
-    const long long rows = static_cast<long long>(R) * (N / 32) * task_cost(32, p->cols[c]) + 10 * listed + 20LL * p->na;
+    // gridding, and the row transforms where the same kernel runs them
+    long long rows = 10 * listed + 20LL * p->na;
+    if (p->precision == EPIC_PREC_FP32) rows += static_cast<long long>(R) * (N / 32) * task_cost(32, p->cols[c]);
     t->row_cost.push_back(static_cast<int>(std::max<long long>(1, rows / 256)));
     t->col_cost.push_back(static_cast<int>(task_cost(32, R)));
   }
   t->max_lists = (t->max_lists + 127) & ~127;
   prefix_sums(&t->row_cost);
   prefix_sums(&t->col_cost);
+  return EPIC_OK;
 }
 
 // Arguments of one fused launch over a device batch.
@@ -954,7 +983,6 @@ uint16_t to_bf16_bits(float f) {
 epic_status image_tc(epic_plan_t p, const void* d_volt, long long n_time, double* d_image) {
   const int C = p->nc, N = p->n;
   if (p->tc_time == 0) {
-    p->kr = ((2 * *std::max_element(p->cols.begin(), p->cols.end()) + 63) / 64) * 64;
     const size_t per_t = static_cast<size_t>(C) *
                          (static_cast<size_t>(N) * p->kp * 2 + static_cast<size_t>(p->rows_alloc) * p->kr * 2 +
                           2 * sizeof(float) + sizeof(float2));
@@ -1026,10 +1054,6 @@ epic_status image_tc(epic_plan_t p, const void* d_volt, long long n_time, double
   u.win = p->d_win.p;
   u.twid = p->d_twid.p;
   u.spec = nullptr;
-  u.gofs = p->d_gofs.p;                    // window-column gather tables
-  u.gcnt = p->d_gcnt.p;
-  u.gent = p->d_gent.p;
-  u.gbase = p->d_gbase.p;
   u.pix = p->d_tc_pix.p;
   u.rows_alloc = p->rows_alloc;
   u.rs = p->rs;
@@ -1049,6 +1073,14 @@ epic_status image_tc(epic_plan_t p, const void* d_volt, long long n_time, double
   a.kp = p->kp;
   a.bf16 = p->precision == EPIC_PREC_BF16 ? 1 : 0;
   a.err = p->d_err.p;
+  a.lists = p->d_wlists.p;
+  a.lists_at = p->d_wat.p;
+  a.nb_max = p->w_nb_max;
+  a.max_lists = p->w_max_lists;
+  a.rb = p->tc_rb;
+  a.lists_smem = p->tc_lists_smem;
+  a.row_cost = p->d_wrcost.p;
+  a.pixel = p->d_tc_pixel.p;
   a.gh = p->d_tc_gh.p;
   a.kr = p->kr;
   a.r_alloc = p->rows_alloc;
@@ -1221,7 +1253,7 @@ epic_status plan_wide(epic_plan_s* p, const std::vector<float>& wts, WideTables*
   if (p->precision != EPIC_PREC_FP32 || p->persistent || !epic::wide_supported(N) || pair_bytes > p->workspace_budget)
     return EPIC_OK;
   p->w_gs = ((*std::max_element(p->cols.begin(), p->cols.end()) + 3) & ~3) + 1;
-  build_wide_lists(p, wts, p->w_gs, wide);
+  if (epic_status st = build_wide_lists(p, wts, p->w_gs, epic::wide_row_block(N), wide)) return st;
   p->w_nb_max = wide->nb_max;
   p->w_max_lists = wide->max_lists;
   epic::WideArgs w{};
@@ -1260,6 +1292,17 @@ epic_status choose_path(epic_plan_s* p, const epic_plan_desc* d, bool fused_shap
     p->kp = epic::tc_kp(p->rows_alloc);
     e = epic::tc_prepare(p->precision == EPIC_PREC_BF16, epic::tc_smem(p->kp));
     if (e != cudaSuccess) return cuda_fail(e, "tensor-core kernel attributes");
+    // gridding lists by blocks of rows small enough for four CTAs per SM;
+    // through L1 where two blocks' lists of 4 rows are still too large
+    p->kr = ((2 * *std::max_element(p->cols.begin(), p->cols.end()) + 63) / 64) * 64;
+    for (p->tc_rb = N == 128 ? 16 : 8;; p->tc_rb /= 2) {
+      if (epic_status st = build_wide_lists(p, wts, p->kr / 2, p->tc_rb, wide)) return st;
+      const size_t need = epic::tc_grid_smem(Na, p->tc_rb, p->kr, wide->max_lists) + 2048;
+      p->tc_lists_smem = (p->tc_rb > 4 ? 4 : 1) * need <= static_cast<size_t>(smem_optin);
+      if (p->tc_lists_smem || p->tc_rb <= 4) break;
+    }
+    p->w_nb_max = wide->nb_max;
+    p->w_max_lists = wide->max_lists;
   }
   p->rs_fused = epic::image_rs_fused(p->rows_alloc);
   if (fused && d->path == EPIC_PATH_PIPED && epic::piped_supported(N, Na)) {
@@ -1493,7 +1536,8 @@ epic_status epic_plan_create(epic_plan_t* out, const epic_plan_desc* d) {
   std::vector<int> gofs, gbase, ugofs, ugbase;
   std::vector<uint4> gcnt, ugcnt;
   std::vector<uint2> gent, ugent;
-  if (p->path == EPIC_PATH_FUSED ? !p->pair : (p->path == EPIC_PATH_UNFUSED && !p->wide)) {
+  if (p->path == EPIC_PATH_FUSED ? !p->pair
+                                 : (p->path == EPIC_PATH_UNFUSED && !p->wide && p->precision == EPIC_PREC_FP32)) {
     const int n1 = p->path == EPIC_PATH_FUSED ? epic::image_fft_lanes(N) : epic::unfused_fft_lanes(N);
     if (epic_status st = build_gather(p, wts, n1, true, gofs, gcnt, gent, gbase)) {
       epic_plan_destroy(p);
@@ -1616,6 +1660,7 @@ epic_status epic_plan_destroy(epic_plan_t p) {
   p->d_wat.release();
   p->d_wrcost.release();
   p->d_wccost.release();
+  p->d_tc_pixel.release();
   p->d_uv.release();
   p->d_iters.release();
   if (p->graph_exec) cudaGraphExecDestroy(p->graph_exec);
@@ -1796,6 +1841,7 @@ epic_status epical_configure(epic_plan_t p, double cal_l, double cal_m, int n_sr
   EPIC_CUDA(cudaMemsetAsync(p->d_kacc.p, 0, n * sizeof(double2), p->stream));
   EPIC_CUDA(cudaMemsetAsync(p->d_pacc.p, 0, n * sizeof(double), p->stream));
   EPIC_CUDA(cudaStreamSynchronize(p->stream));
+  if (epic_status st = set_tc_pixel(p, k0x, k0y)) return st;
   p->k0x = k0x;
   p->k0y = k0y;
   p->gamma = gamma;
@@ -2262,6 +2308,8 @@ epic_status epical_set_state(epic_plan_t p, const void* buf, size_t bytes) {
   EPIC_CUDA(cudaMemcpyAsync(p->d_pacc.p, i + 2 * n * sizeof(double2), n * sizeof(double),
                             cudaMemcpyHostToDevice, p->stream));
   EPIC_CUDA(cudaStreamSynchronize(p->stream));
+  if (hd.k0x != p->k0x || hd.k0y != p->k0y)
+    if (epic_status st = set_tc_pixel(p, hd.k0x, hd.k0y)) return st;
   p->k0x = hd.k0x;
   p->k0y = hd.k0y;
   p->gamma = hd.gamma;

@@ -2,14 +2,13 @@
 // tensor-core GEMMs (tcgen05, FP16 or BF16 operands, FP32 accumulation).
 //
 // Per batch of frames (frame f = t_local * C + c):
-//   grid_lp      per frame, E' = E / g (Eq. 8) into shared memory and
+//   grid_lp      per frame pair, E' = E / g (Eq. 8) into shared memory and
 //                S_f = sum_a |E'_a| / Na, an upper bound of every grid cell
 //                and row-spectrum value (s_f = largest power of two with
-//                s_f S_f < 1); FP32
-//                gridding (Eq. 9) as a gather into the window grid (the
-//                plain path's window-column lists), scaled by s_f and stored
-//                FP16/BF16 as Gh[f R + jw][2 x + (re, im)]; the calibrator
-//                pixel is summed in FP32 from the same cells;
+//                s_f S_f < 1); FP32 gridding (Eq. 9) by per-cell tap lists,
+//                scaled by s_f and stored FP16/BF16 as Gh[f R + jw][2 x +
+//                (re, im)]; the calibrator pixel is summed in FP32 over the
+//                antennas' responses;
 //   tc_rows      H = Gh F_r^T with the real-expanded DFT over window columns
 //                (outputs 2 kx + (re, im)); the epilogue writes each row's
 //                spectrum K-major as Hh[c][kx][t][2 jw + (re, im)];
@@ -40,17 +39,18 @@
 #include <cstdint>
 #include <type_traits>
 
+#include "epic_bulk.cuh"
 #include "epic_fft.cuh"
 #include "epic_internal.h"
+#include "epic_lists.cuh"
+#include "epic_residue.cuh"
 
 namespace epic {
 namespace {
 
-template <int N> struct LCfg;
-template <> struct LCfg<128> { static constexpr int N1 = 8,  N2 = 16; };
-template <> struct LCfg<256> { static constexpr int N1 = 16, N2 = 16; };
+using fft::Cf2;
 
-constexpr int kLBT = 256;
+constexpr int kLBT = 256;          // threads of the gridding kernel
 
 // Exponent k of the largest power of two s = 2^k with s * S < 1 (S > 0),
 // from the float's exponent field, clamped to [-60, 60] so that s and 1/s^2
@@ -65,16 +65,6 @@ __device__ __forceinline__ float exp2i(int k) {   // 2^k for k in [-126, 127]
   return __uint_as_float(static_cast<unsigned>(k + 127) << 23);
 }
 
-__device__ __forceinline__ float2 load_volt_tc(const void* volt, int fmt, size_t idx) {
-  if (fmt == 0) {
-    const unsigned b = __ldg(static_cast<const unsigned char*>(volt) + idx);
-    const int re = static_cast<int>(b << 24) >> 28;
-    const int im = static_cast<int>(b << 28) >> 28;
-    return make_float2(static_cast<float>(re), static_cast<float>(im));
-  }
-  return __ldg(static_cast<const float2*>(volt) + idx);
-}
-
 // (re, im) rounded to the storage type, as one 4-byte store.
 __device__ __forceinline__ void store_lp(__half* dst, float re, float im) {
   *reinterpret_cast<__half2*>(dst) = __floats2half2_rn(re, im);
@@ -84,108 +74,171 @@ __device__ __forceinline__ void store_lp(__nv_bfloat16* dst, float re, float im)
 }
 
 // ---- gridding into the low-precision window grid, FP32 calibrator pixel ----
-// One frame at a time per CTA: E' = E / g (Eq. 8) into shared memory, then
-// every lane (window row jw, n1) gathers the taps of its window columns
-// x = n1 + N1 j (Eq. 9, the plan's window-column lists), scales by s_f and
-// stores the cell rounded to FP16/BF16 into Gh[f R_alloc + jw][2x + re/im]
-// (columns without taps get zeros).  The calibrator pixel, the Eq. 10 sum
-// at k0, is accumulated from the FP32 cells with their absolute phases.
-template <int N, typename T>
+// Two frames of one channel at a time per CTA (FP32 pairs): E' = E / g (Eq. 8)
+// into shared memory with S_f and the calibrator pixel P_f = sum_a r_a E'_a
+// (r_a: the response of pixel k0 through antenna a's taps, without the
+// phasing that E' carries), then by blocks of rb grid rows every lane sums
+// one grid cell's taps (Eq. 9; lists sorted by length, cells without taps
+// last), scales it by s_f and rounds it into the block's FP16/BF16 tile of
+// both frames, which one bulk copy per frame takes to Gh[f R_alloc + jw][2x +
+// re/im] while the next block is gridded.  The lists of a block are copied
+// to shared memory a block ahead (TS), or read through L1 where two blocks'
+// do not fit.
+//
+// What bounds it: instruction issue (49 %) and the shared-memory pipe (46 %:
+// list entries and E' of a tap, 4-byte tile stores), and the barrier per
+// block, whose slices do not divide evenly over 8 warps.  8192 frames of 256
+// antennas at N = 128: 51 us (one frame at a time through 256-entry lane lists
+// 124 us); 4096 frames of 1024 antennas at N = 256: 111 us (209 us).  Blocks
+// of 16 (N = 128) and 8 rows leave four CTAs per SM; 32 and 16 rows with two:
+// 66 and 111 us.
+template <int FMT, typename T, bool TS>
 __global__ void __launch_bounds__(kLBT) grid_lp_kernel(const TcArgs A, long long t0, int nt) {
-  constexpr int N1 = LCfg<N>::N1, N2 = LCfg<N>::N2;
-  constexpr int GROUPS = kLBT / N1;
-  constexpr int CW = (N2 + 15) / 16;
-  extern __shared__ float2 Es[];                   // [Na] E / g of the current frame
-  __shared__ float red[kLBT / 32];
-  const int g = threadIdx.x / N1, n1 = threadIdx.x % N1;
-  const int lane = threadIdx.x & 31;
-  const int C = A.u.n_chan, Na = A.u.n_ant;
-  const int nj = A.kr / (2 * N1);                  // column blocks held in Gh
+  using T2 = typename std::conditional<std::is_same<T, __half>::value, __half2, __nv_bfloat162>::type;
+  extern __shared__ __align__(128) unsigned char glp_smem[];
+  const int C = A.u.n_chan, Na = A.u.n_ant, rb = A.rb, kc = A.kr / 2, tid = threadIdx.x;
+  const int lane = tid & 31, warp = tid >> 5;
+  T2* tile = reinterpret_cast<T2*>(glp_smem);                // [2 slots][2 frames][rb][kc]
+  unsigned char* slists = glp_smem + static_cast<size_t>(4) * rb * kc * sizeof(T2);   // [2][max_lists] (TS)
+  Cf2* Es = reinterpret_cast<Cf2*>(slists + (TS ? 2 * static_cast<size_t>(A.max_lists) : 0));   // [Na + 1], entry Na zero
+  __shared__ uint64_t bars[2];
+  __shared__ int abort_flag;
+  __shared__ float red[kLBT / 32][6];
+  if (tid == 0) {
+    Es[Na] = Cf2{0ull, 0ull};
+    mbar_init_one(bars, 2);
+    abort_flag = 0;
+  }
   T* gh = static_cast<T*>(A.gh);
-  const long long frames = static_cast<long long>(nt) * C;
-  for (long long it = blockIdx.x; it < frames; it += gridDim.x) {
-    const int c = static_cast<int>(it / nt);
-    const int tl = static_cast<int>(it - static_cast<long long>(c) * nt);
-    const size_t f = static_cast<size_t>(tl) * C + c;
+  const long long P = (nt + 1) / 2;
+  const Share share(A.row_cost, C, 1, P);
+  auto load_lists = [&](int c, int b, int slot) {
+    const int2 at = __ldg(A.lists_at + c * A.nb_max + b);    // (offset, bytes) / 16
+    bulk_load(smem_addr(slists + static_cast<size_t>(slot) * A.max_lists), A.lists + static_cast<size_t>(at.x) * 16,
+              static_cast<uint32_t>(at.y) * 16u, smem_addr(bars + slot));
+  };
+  unsigned it = 0;                                           // row blocks so far: lists and tile slot it & 1
+  bool first = true;
+  for (int c = share.first(C); c < C && share.before(c) < share.hi; ++c) {
+    const long long p_lo = share.pair_at(share.lo, c), p_hi = share.pair_at(share.hi, c);
+    if (p_lo >= p_hi) continue;
+    const int R = __ldg(A.win4 + c).y, nb = (R + rb - 1) / rb;
+    const bool more = c + 1 < C && share.pair_at(share.hi, c + 1) > 0;
     const float vs = A.u.vscale ? __ldg(A.u.vscale + c) : 1.0f;
+    // columns past this channel's window are zero in both tile slots
+    if (tid == 0) bulk_store_wait_read();
     __syncthreads();
-    // E' and S_f = sum_a |E'_a| / Na over unflagged antennas: an upper bound
-    // of every grid cell and row-spectrum value (normalised taps, 1/Na folded)
-    float sa = 0.f;
-    for (int a = threadIdx.x; a < Na; a += kLBT) {
-      const float2 e = load_volt_tc(A.u.volt, A.u.input_fmt, (static_cast<size_t>(t0 + tl) * C + c) * Na + a);
-      const float2 ec = fft::cmul(make_float2(e.x * vs, e.y * vs), __ldg(A.u.wgain + static_cast<size_t>(c) * Na + a));
-      Es[a] = ec;
-      if (__ldg(A.u.cell0 + static_cast<size_t>(c) * Na + a) >= 0) sa += sqrtf(ec.x * ec.x + ec.y * ec.y);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) sa += __shfl_xor_sync(fft::kFull, sa, o);
-    if (lane == 0) red[threadIdx.x >> 5] = sa;
-    __syncthreads();
-    float S = 0.f;
-#pragma unroll
-    for (int w = 0; w < kLBT / 32; ++w) S += red[w];
-    const int ke = pow2_exp_below_inverse(S / static_cast<float>(Na));
-    const float sf = exp2i(ke);                    // s_f multiplies the cells
-    if (threadIdx.x == 0) {
-      A.fscale[f] = sf;
-      A.finv2[f] = exp2i(-2 * ke);                 // 1 / s_f^2 multiplies |D|^2
-    }
-    const int4 wn = __ldg(A.win4 + c);             // (y0, rows, x0, cols)
-    const int R = wn.y;
-    const int nl = A.u.rows_alloc * N1;
-    const int* gofs = A.u.gofs + static_cast<size_t>(c) * nl;
-    const uint4* gcnt = A.u.gcnt + static_cast<size_t>(c) * nl * CW;
-    const uint2* gent = A.u.gent + __ldg(A.u.gbase + c);
-    float2 pix = make_float2(0.f, 0.f);
-    for (int row = g; row < R; row += GROUPS) {
-      const int li = row * N1 + n1;
-      int e = __ldg(gofs + li);
-      unsigned cv[4 * CW];
-#pragma unroll
-      for (int w = 0; w < CW; ++w) {
-        const uint4 q = __ldg(gcnt + static_cast<size_t>(li) * CW + w);
-        cv[4 * w] = q.x;
-        cv[4 * w + 1] = q.y;
-        cv[4 * w + 2] = q.z;
-        cv[4 * w + 3] = q.w;
-      }
-      T* dst = gh + (f * A.r_alloc + row) * static_cast<size_t>(A.kr);
-#pragma unroll
-      for (int j = 0; j < N2; ++j) {
-        if (j >= nj) break;
-        const int cj = static_cast<int>((cv[j >> 2] >> (8 * (j & 3))) & 255u);
-        float2 sum = make_float2(0.f, 0.f);
-        for (int k = 0; k < cj; ++k) {
-          const uint2 en = __ldg(gent + e + k);
-          const float2 x = Es[en.x];
-          const float w = __uint_as_float(en.y);
-          sum.x = fmaf(w, x.x, sum.x);
-          sum.y = fmaf(w, x.y, sum.y);
-        }
-        e += cj;
-        const int x = n1 + N1 * j;
-        store_lp(dst + 2 * x, sum.x * sf, sum.y * sf);
-        if (A.u.do_cal && cj > 0) {
-          const int m = ((wn.z + x) * A.u.k0x + (wn.x + row) * A.u.k0y) & (N - 1);
-          const float2 t = __ldg(A.u.twid + m);
-          pix.x += sum.x * t.x - sum.y * t.y;
-          pix.y += sum.x * t.y + sum.y * t.x;
+    for (int i = tid; i < 2 * rb * kc * 2; i += kLBT) reinterpret_cast<unsigned*>(tile)[i] = 0u;
+    if (first && tid == 0 && TS) load_lists(c, 0, 0);
+    first = false;
+    for (long long p = p_lo; p < p_hi; ++p) {
+      const bool two = 2 * p + 1 < nt;
+      // E', and over unflagged antennas S_f = sum_a |E'_a| / Na, an upper bound
+      // of every grid cell and row-spectrum value (normalised taps, 1/Na
+      // folded), and the calibrator pixel
+      float v[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+      const size_t i0 = (static_cast<size_t>(t0 + 2 * p) * C + c) * Na, ic = static_cast<size_t>(c) * Na;
+#pragma unroll 4
+      for (int a = tid; a < Na; a += kLBT) {
+        const float2 w = __ldg(A.u.wgain + ic + a);
+        const float2 e0 = fft::cmul(pair_volt<FMT>(A.u.volt, i0 + a, vs), w);
+        float2 e1 = make_float2(0.f, 0.f);
+        if (two) e1 = fft::cmul(pair_volt<FMT>(A.u.volt, i0 + static_cast<size_t>(C) * Na + a, vs), w);
+        Es[a] = Cf2{fft::f2_pack(e0.x, e1.x), fft::f2_pack(e0.y, e1.y)};
+        if (__ldg(A.u.cell0 + ic + a) >= 0) {
+          v[0] += sqrtf(e0.x * e0.x + e0.y * e0.y);
+          v[1] += sqrtf(e1.x * e1.x + e1.y * e1.y);
+          if (A.u.do_cal) {
+            const float2 r = __ldg(A.pixel + ic + a);
+            v[2] = fmaf(r.x, e0.x, fmaf(-r.y, e0.y, v[2]));
+            v[3] = fmaf(r.x, e0.y, fmaf(r.y, e0.x, v[3]));
+            v[4] = fmaf(r.x, e1.x, fmaf(-r.y, e1.y, v[4]));
+            v[5] = fmaf(r.x, e1.y, fmaf(r.y, e1.x, v[5]));
+          }
         }
       }
-    }
-    if (A.u.do_cal) {
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        pix.x += __shfl_xor_sync(fft::kFull, pix.x, o);
-        pix.y += __shfl_xor_sync(fft::kFull, pix.y, o);
+      for (int j = 0; j < 6; ++j) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v[j] += __shfl_xor_sync(fft::kFull, v[j], o);
+        if (lane == 0) red[warp][j] = v[j];
       }
-      if (lane == 0 && (pix.x != 0.f || pix.y != 0.f)) {
-        atomicAdd(&A.u.pix[f].x, pix.x * A.u.pix_sign);
-        atomicAdd(&A.u.pix[f].y, pix.y * A.u.pix_sign);
+      __syncthreads();
+      float S[2] = {0.f, 0.f};
+#pragma unroll
+      for (int w = 0; w < kLBT / 32; ++w) {
+        S[0] += red[w][0];
+        S[1] += red[w][1];
+      }
+      const int k0 = pow2_exp_below_inverse(S[0] / static_cast<float>(Na));
+      const int k1 = pow2_exp_below_inverse(S[1] / static_cast<float>(Na));
+      const float s0 = exp2i(k0), s1 = exp2i(k1);            // s_f multiplies the cells
+      const size_t f0 = static_cast<size_t>(2 * p) * C + c, f1 = f0 + C;
+      if (tid < (two ? 2 : 1)) {
+        const int k = tid ? k1 : k0;
+        A.fscale[tid ? f1 : f0] = exp2i(k);
+        A.finv2[tid ? f1 : f0] = exp2i(-2 * k);              // 1 / s_f^2 multiplies |D|^2
+        if (A.u.do_cal) {
+          float2 q = make_float2(0.f, 0.f);
+          for (int w = 0; w < kLBT / 32; ++w) {
+            q.x += red[w][2 + 2 * tid];
+            q.y += red[w][3 + 2 * tid];
+          }
+          A.u.pix[tid ? f1 : f0] = q;
+        }
+      }
+      for (int b = 0; b < nb; ++b, ++it) {
+        const int slot = it & 1;
+        if (TS && tid == 0) {                                // the other slot was read out before the last barrier
+          if (b + 1 < nb) load_lists(c, b + 1, slot ^ 1);
+          else if (p + 1 < p_hi) load_lists(c, 0, slot ^ 1);
+          else if (more) load_lists(c + 1, 0, slot ^ 1);
+        }
+        T2* t0p = tile + static_cast<size_t>(slot) * 2 * rb * kc;
+        T2* t1p = t0p + rb * kc;
+        const unsigned char* lists = TS ? slists + static_cast<size_t>(slot) * A.max_lists
+                                        : A.lists + static_cast<size_t>(__ldg(A.lists_at + c * A.nb_max + b).x) * 16;
+        if (TS && !mbar_wait_bounded(smem_addr(bars + slot), (it >> 1) & 1u)) {
+          abort_flag = 1;
+          atomicExch(A.err, 1);
+        } else {
+          const BlockLists hd = *reinterpret_cast<const BlockLists*>(lists);
+          const int2* slice = reinterpret_cast<const int2*>(lists + sizeof(BlockLists));
+          const uint16_t* cell = reinterpret_cast<const uint16_t*>(lists + hd.cells);
+          const uint2* ent = reinterpret_cast<const uint2*>(lists + hd.ents);
+          for (int k = 0; k * (kLBT / 32) < hd.nslice; ++k) {
+            const int sl = slice_of(k, warp, kLBT / 32);
+            if (sl >= hd.nslice) break;
+            const int2 s = slice[sl];
+            const unsigned at = cell[sl * 32 + lane];
+            const Cf2 sum = sum_taps(ent + s.x + lane, s.y, Es);
+            if (at != 0xffffu) {
+              const float2 re = fft::f2_unpack(sum.re), im = fft::f2_unpack(sum.im);
+              store_lp(reinterpret_cast<T*>(t0p + at), re.x * s0, im.x * s0);
+              store_lp(reinterpret_cast<T*>(t1p + at), re.y * s1, im.y * s1);
+            }
+          }
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the tile before the bulk copies
+        if (tid == 0) bulk_store_wait_read();                // the other slot's copies have read it
+        __syncthreads();
+        if (*reinterpret_cast<volatile int*>(&abort_flag)) {
+          // let the lists in flight land (bounded) before the CTA exits
+          if (TS && tid == 0 && (b + 1 < nb || p + 1 < p_hi || more))
+            mbar_wait_bounded(smem_addr(bars + (slot ^ 1)), ((it + 1) >> 1) & 1u);
+          return;
+        }
+        if (tid == 0) {
+          const int rows = R - b * rb < rb ? R - b * rb : rb;
+          const uint32_t bytes = static_cast<uint32_t>(rows) * A.kr * sizeof(T);
+          bulk_store(gh + (f0 * A.r_alloc + b * rb) * A.kr, smem_addr(t0p), bytes);
+          if (two) bulk_store(gh + (f1 * A.r_alloc + b * rb) * A.kr, smem_addr(t1p), bytes);
+          bulk_store_commit();
+        }
       }
     }
   }
+  if (tid == 0) bulk_store_wait_all();
 }
 
 // ---------------------------------------------------------------------------
@@ -313,7 +366,8 @@ constexpr uint32_t kColTmemCols = 512;   // tc_cols, tc_rows, X-engine: two 256-
 // the CTA's resident DFT tile and the data ring.
 size_t tc_smem_bytes(int kp) {
   const size_t tile = static_cast<size_t>(kp / 64) * kChunkBytes;
-  return 1024 /*alignment slack*/ + tile + kColStages * kColChunkBytes + 256 /*barriers*/;
+  return 1024 /*alignment slack*/ + tile + kColStages * kColChunkBytes + 256 /*barriers*/ +
+         kEpiWarps * kTile * sizeof(float) /*frame weights*/;
 }
 
 // Column DFT GEMM.  A CTA owns one 128-row DFT tile (rows 2 ky + re/im),
@@ -467,30 +521,39 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     const int r = mb * kTile + q * 32 + lane;      // DFT row = 2 ky + (re, im)
     const int ky = r >> 1;
     int i = 0;
+    float* wts = reinterpret_cast<float*>(bars + 2 * S + 8) + (warp - 2) * kTile;   // 1 / s_t^2 of the tile's frames
     for (long long u = u0; u < dtiles; u += G, ++i) {
       const int acc = i & 1;
       const uint32_t ph = static_cast<uint32_t>((i >> 1) & 1);
-      if (!mbar_wait(smem_u32(bars + 2 * S + acc), ph, abort_flag, A.err)) break;
-      tc_fence_after();
-      const int tb = static_cast<int>(u % tbk);
-      const int ck = static_cast<int>(u / tbk) * 2 + half;
-      const int c = ck / N, kx = ck % N;
-      float sum = 0.f;
+      const int tb = static_cast<int>(static_cast<unsigned>(u) % static_cast<unsigned>(tbk));
+      const unsigned ck = static_cast<unsigned>(u) / static_cast<unsigned>(tbk) * 2 + half;
+      const int c = static_cast<int>(ck / N), kx = static_cast<int>(ck % N);
+      // the weights before the wait, for broadcast reads of four at a time
 #pragma unroll
       for (int ch = 0; ch < kTile / 32; ++ch) {
-        const int col = ch * 32;
-        const int t = tb * kTile + col + lane;
-        const float my_w = (t < nt) ? __ldg(A.finv2 + static_cast<size_t>(t) * C + c) : 0.f;
+        const int t = tb * kTile + ch * 32 + lane;
+        wts[ch * 32 + lane] = (t < nt) ? __ldg(A.finv2 + static_cast<size_t>(t) * C + c) : 0.f;
+      }
+      __syncwarp();
+      if (!mbar_wait(smem_u32(bars + 2 * S + acc), ph, abort_flag, A.err)) break;
+      tc_fence_after();
+      fft::f32x2 sum2 = 0ull;                      // even and odd frames
+#pragma unroll
+      for (int ch = 0; ch < kTile / 32; ++ch) {
         float v[32];
         tmem_ld32(tmem_base + (static_cast<uint32_t>(q * 32) << 16) +
-                      static_cast<uint32_t>(acc * kColN + half * kTile + col),
+                      static_cast<uint32_t>(acc * kColN + half * kTile + ch * 32),
                   v);
 #pragma unroll
-        for (int j = 0; j < 32; ++j) {
-          const float w = __shfl_sync(fft::kFull, my_w, j);
-          sum = fmaf(v[j] * v[j], w, sum);
+        for (int j = 0; j < 32; j += 4) {
+          const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(wts + ch * 32 + j);
+          const fft::f32x2 a = fft::f2_pack(v[j], v[j + 1]), b = fft::f2_pack(v[j + 2], v[j + 3]);
+          sum2 = fft::f2_fma(fft::f2_mul(a, a), w.x, sum2);
+          sum2 = fft::f2_fma(fft::f2_mul(b, b), w.y, sum2);
         }
       }
+      const float2 halves = fft::f2_unpack(sum2);
+      const float sum = halves.x + halves.y;
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(bars + 2 * S + 2 + acc));
@@ -922,11 +985,17 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       if (!mbar_wait(smem_u32(bars + 2 * S + acc), aph, abort_flag, A.err)) break;
       tc_fence_after();
       const int mt = static_cast<int>(u / nt2), ot = static_cast<int>(u % nt2);
-      const long long row = static_cast<long long>(mt) * kTile + q * 32 + lane;
-      const long long f = row / A.r_alloc;                 // frame tl * C + c
+      // 32-bit place arithmetic, once per tile (in 64 bits per store it was
+      // most of the epilogue: 92 -> 81 us at N = 128): the rows of a batch are fewer
+      // than 2^31 (each takes 128 bytes or more of Gh)
+      const unsigned row = static_cast<unsigned>(mt) * kTile + q * 32 + lane;
+      const unsigned f = row / static_cast<unsigned>(A.r_alloc);   // frame tl * C + c
       const int jw = static_cast<int>(row - f * A.r_alloc);
-      const int c = static_cast<int>(f % C), tl = static_cast<int>(f / C);
+      const int tl = static_cast<int>(f / static_cast<unsigned>(C)), c = static_cast<int>(f - static_cast<unsigned>(tl) * C);
       const bool live = row < rows && jw < __ldg(A.win4 + (row < rows ? c : 0)).y;
+      const int kx0 = (ot * kRowN + half * kTile) / 2;
+      T* dst = hh + ((static_cast<size_t>(c) * N + kx0) * A.tb_cap + tl) * A.kp + 2 * jw;
+      const size_t step = static_cast<size_t>(A.tb_cap) * A.kp;    // to the next column
 #pragma unroll
       for (int ch = 0; ch < kTile / 32; ++ch) {
         float v[32];
@@ -936,8 +1005,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         if (live) {
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
-            const int kx = (ot * kRowN + half * kTile + ch * 32) / 2 + j;
-            store_lp(hh + ((static_cast<size_t>(c) * N + kx) * A.tb_cap + tl) * A.kp + 2 * jw, v[2 * j], v[2 * j + 1]);
+            store_lp(dst, v[2 * j], v[2 * j + 1]);
+            dst += step;
           }
         }
       }
@@ -955,23 +1024,34 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   }
 }
 
-template <int N, typename T>
-cudaError_t grid_lp_n(const TcArgs& a, long long t0, int nt, int sms, cudaStream_t s) {
-  const size_t es_bytes = static_cast<size_t>(a.u.n_ant) * sizeof(float2);
-  cudaError_t e = cudaFuncSetAttribute(grid_lp_kernel<N, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(es_bytes));
+template <int FMT, typename T, bool TS>
+cudaError_t grid_lp_launch(const TcArgs& a, long long t0, int nt, int sms, cudaStream_t s) {
+  const size_t smem = tc_grid_smem(a.u.n_ant, a.rb, a.kr, TS ? a.max_lists : 0);
+  auto k = grid_lp_kernel<FMT, T, TS>;
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
   int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, grid_lp_kernel<N, T>, kLBT, es_bytes);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kLBT, smem);
   if (e != cudaSuccess) return e;
-  const long long frames = static_cast<long long>(nt) * a.u.n_chan;
-  long long rb = static_cast<long long>(per_sm > 0 ? per_sm : 1) * sms;
-  if (rb > frames) rb = frames;
-  grid_lp_kernel<N, T><<<static_cast<unsigned>(rb), kLBT, es_bytes, s>>>(a, t0, nt);
+  const long long pairs = static_cast<long long>((nt + 1) / 2) * a.u.n_chan;
+  const long long most = static_cast<long long>(per_sm > 0 ? per_sm : 1) * sms;
+  k<<<static_cast<unsigned>(pairs < most ? pairs : most), kLBT, smem, s>>>(a, t0, nt);
   return cudaGetLastError();
 }
 
+template <typename T>
+cudaError_t grid_lp(const TcArgs& a, long long t0, int nt, int sms, cudaStream_t s) {
+  if (a.lists_smem)
+    return a.u.input_fmt ? grid_lp_launch<1, T, true>(a, t0, nt, sms, s) : grid_lp_launch<0, T, true>(a, t0, nt, sms, s);
+  return a.u.input_fmt ? grid_lp_launch<1, T, false>(a, t0, nt, sms, s) : grid_lp_launch<0, T, false>(a, t0, nt, sms, s);
+}
+
 }  // namespace
+
+size_t tc_grid_smem(int n_ant, int rb, int kr, int max_lists) {
+  return static_cast<size_t>(4) * rb * kr * 2 + 2 * static_cast<size_t>(max_lists) +
+         (static_cast<size_t>(n_ant) + 1) * sizeof(fft::Cf2);
+}
 
 bool tc_supported(int n, int rows_alloc) { return (n == 128 || n == 256) && 2 * rows_alloc <= 256; }
 
@@ -1023,13 +1103,7 @@ bool tc_make_row_maps(void* gh, void* dftr, long long rows_cap, int n, int kr, b
 
 cudaError_t launch_tc_batch(const TcArgs& a, const void* tm_dft, const void* tm_data, long long t0, int nt,
                             int sms, cudaStream_t s) {
-  cudaError_t e = cudaSuccess;
-  if (a.u.do_cal) e = cudaMemsetAsync(a.u.pix, 0, static_cast<size_t>(nt) * a.u.n_chan * sizeof(float2), s);
-  if (e != cudaSuccess) return e;
-  if (a.bf16) e = (a.u.grid_n == 128) ? grid_lp_n<128, __nv_bfloat16>(a, t0, nt, sms, s)
-                                      : grid_lp_n<256, __nv_bfloat16>(a, t0, nt, sms, s);
-  else e = (a.u.grid_n == 128) ? grid_lp_n<128, __half>(a, t0, nt, sms, s)
-                               : grid_lp_n<256, __half>(a, t0, nt, sms, s);
+  cudaError_t e = a.bf16 ? grid_lp<__nv_bfloat16>(a, t0, nt, sms, s) : grid_lp<__half>(a, t0, nt, sms, s);
   if (e != cudaSuccess) return e;
   {
     const long long rows = static_cast<long long>(nt) * a.u.n_chan * a.r_alloc;

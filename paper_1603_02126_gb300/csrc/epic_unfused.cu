@@ -416,14 +416,35 @@ __device__ __forceinline__ void corr_item(const UnfusedArgs& A, long long t0, in
   const float vs = A.vscale ? __ldg(A.vscale + c) : 1.0f;
   const int tb = nt * sy / nsy, te = nt * (sy + 1) / nsy;
   float kr = 0.f, ki = 0.f, pp = 0.f;
-  for (int tl = tb; tl < te; ++tl) {
-    const size_t f = static_cast<size_t>(tl) * C + c;
-    const float2 p = __ldcg(A.pix + f);            // written by another SM (persistent form)
-    const float2 e0 = load_volt_u(A.volt, A.input_fmt, (static_cast<size_t>(t0 + tl) * C + c) * Na + a);
-    const float2 e = make_float2(e0.x * vs, e0.y * vs);
-    kr += e.x * p.x + e.y * p.y;
-    ki += e.y * p.x - e.x * p.y;
-    pp += e.x * e.x + e.y * e.y;
+  // the loads of kBatch samples in flight together (one after the other:
+  // 15.5 us for 128 samples of 64 x 256 voltages, 10 us so)
+  constexpr int kBatch = 8;
+  for (int t = tb; t < te; t += kBatch) {
+    RawU raw[kBatch];
+    float2 p[kBatch];
+#pragma unroll
+    for (int j = 0; j < kBatch; ++j) {
+      const int tl = t + j < te ? t + j : te - 1;
+      p[j] = __ldcg(A.pix + static_cast<size_t>(tl) * C + c);   // written by another SM (persistent form)
+    }
+    if (A.input_fmt == 0) {
+#pragma unroll
+      for (int j = 0; j < kBatch; ++j)
+        raw[j] = fetch_raw(A.volt, 0, (static_cast<size_t>(t0 + (t + j < te ? t + j : te - 1)) * C + c) * Na + a);
+    } else {
+#pragma unroll
+      for (int j = 0; j < kBatch; ++j)
+        raw[j] = fetch_raw(A.volt, 1, (static_cast<size_t>(t0 + (t + j < te ? t + j : te - 1)) * C + c) * Na + a);
+    }
+#pragma unroll
+    for (int j = 0; j < kBatch; ++j)
+      if (t + j < te) {
+        const float2 e0 = unpack_raw(raw[j], A.input_fmt);
+        const float2 e = make_float2(e0.x * vs, e0.y * vs);
+        kr += e.x * p[j].x + e.y * p[j].y;
+        ki += e.y * p[j].x - e.x * p[j].y;
+        pp += e.x * e.x + e.y * e.y;
+      }
   }
   if (nsy == 1) {
     A.kacc[i].x += kr;

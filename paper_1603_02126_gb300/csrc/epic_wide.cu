@@ -32,6 +32,7 @@
 #include "epic_bulk.cuh"
 #include "epic_fft.cuh"
 #include "epic_internal.h"
+#include "epic_lists.cuh"
 #include "epic_residue.cuh"
 
 #include <cstdint>
@@ -41,10 +42,7 @@ namespace {
 
 using fft::Cf2;
 using fft::cmul;
-using fft::f2_fma;
 using fft::f2_pack;
-using fft::f2_splat;
-using fft::f32x2;
 
 constexpr int kWBT = 128;          // threads of the row kernel; two CTAs per SM (255 registers each)
 constexpr int kWP = 32;            // outputs per task
@@ -68,32 +66,18 @@ __host__ __device__ inline int wide_stride(int rows) {
   return r4 % 8 ? r4 : r4 + 4;
 }
 
-// One row block's lists: header (slices, byte offsets of the cells and of
-// the entries), slices (first entry, taps), cells (place in the block; 0xffff
-// = none), entries (byte offset of E'_a, weight bits).
-struct BlockLists {
-  int nslice, cells, ents, unused;
-};
-
 __device__ __forceinline__ void grid_block(const unsigned char* lists, const Cf2* Es, Cf2* grid) {
   const BlockLists hd = *reinterpret_cast<const BlockLists*>(lists);
   const int2* slice = reinterpret_cast<const int2*>(lists + sizeof(BlockLists));
   const uint16_t* cell = reinterpret_cast<const uint16_t*>(lists + hd.cells);
   const uint2* ent = reinterpret_cast<const uint2*>(lists + hd.ents);
-  const int lane = threadIdx.x & 31;
-  for (int sl = threadIdx.x >> 5; sl < hd.nslice; sl += kWBT / 32) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int k = 0; k * (kWBT / 32) < hd.nslice; ++k) {
+    const int sl = slice_of(k, warp, kWBT / 32);
+    if (sl >= hd.nslice) break;
     const int2 s = slice[sl];
     const unsigned at = cell[sl * 32 + lane];
-    const uint2* e = ent + s.x + lane;
-    Cf2 sum{0ull, 0ull};
-#pragma unroll 2
-    for (int k = 0; k < s.y; ++k) {
-      const uint2 en = e[k * 32];
-      const Cf2 x = *reinterpret_cast<const Cf2*>(reinterpret_cast<const unsigned char*>(Es) + en.x);
-      const f32x2 w = f2_splat(__uint_as_float(en.y));
-      sum.re = f2_fma(w, x.re, sum.re);
-      sum.im = f2_fma(w, x.im, sum.im);
-    }
+    const Cf2 sum = sum_taps(ent + s.x + lane, s.y, Es);
     if (at != 0xffffu) grid[at] = sum;
   }
 }
