@@ -187,11 +187,14 @@ cudaError_t launch_image(int n, const ImageArgs& a, cudaStream_t s);
 constexpr int kPairMaxAnt = 4;   // antennas per thread
 int pair_threads(int n);
 // Row stride of the spectra for at most rows occupied rows.
-int pair_rs(int n, int rows);
+int pair_rs(int n, int rows, bool adjoint);
 // Dynamic shared memory, with the tap lists when max_slices > 0.
-size_t pair_smem_bytes(int n, int n_ant, int rows, int gs, int max_slices, int max_ent);
+size_t pair_smem_bytes(int n, int n_ant, int rows, int gs, int max_slices, int max_ent, bool adjoint);
 cudaError_t pair_prepare(int n, int n_ant, bool table, size_t smem, int* ctas_per_sm);
 cudaError_t launch_pair(int n, const ImageArgs& a, cudaStream_t s);
+// Adjoint in the same form, FP32 (epic_pair_adjoint.cu): adds dL/dconj(w) of
+// dldi [C][N][N] to dldw [C][Na].
+cudaError_t launch_adjoint_pair(int n, const ImageArgs& a, const double* dldi, double2* dldw, cudaStream_t s);
 // Owner of image pixel (kx, ky) in the column phase.
 bool pair_pixel_owner(int n, int kx, int ky, PixelOwner* out);
 int pair_col_rounds(int n);

@@ -26,36 +26,15 @@
 // 2000 samples 37.6 against 53.9 us (with the update).
 #include "epic_fft.cuh"
 #include "epic_internal.h"
-#include "epic_lists.cuh"
-#include "epic_residue.cuh"
+#include "epic_pair.cuh"
 
 #include <cstdint>
 
 namespace epic {
 namespace {
 
-using fft::Cf2;
 using fft::cmul;
 using fft::f2_pack;
-
-// Frame pairs per FP32 partial image (FP64 across): 128 roundings of a running
-// sum, image error 0.9e-7 against 64 bits over 10^4 samples (1.4e-7 at 256).
-constexpr int kPairRun = 128;
-
-// Gridding of one frame pair: slices of 32 cells, one cell per lane.
-template <int BT>
-__device__ __forceinline__ void grid_pair(const int* __restrict__ cell, const int2* __restrict__ slice,
-                                          const uint2* __restrict__ ent, int nslice, const Cf2* Es, Cf2* grid) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int k = 0; k * (BT / 32) < nslice; ++k) {
-    const int sl = slice_of(k, warp, BT / 32);
-    if (sl >= nslice) break;
-    const int2 s = slice[sl];
-    const int at = cell[sl * 32 + lane];
-    const Cf2 sum = sum_taps(ent + s.x + lane, s.y, Es);
-    if (at >= 0) grid[at] = sum;
-  }
-}
 
 // Multiple-pixel EPICal: the calibration pixels among a thread's outputs
 // (slot mask, index of its first tap) of frame pair p.
@@ -71,62 +50,6 @@ __device__ __forceinline__ void store_taps(const ImageArgs& A, const Cf2 (&y)[16
       const int pi = static_cast<int>(tb.y) + __popc(tb.x & ((1u << m) - 1u));
       store_pixel(y, m, __ldg(ph + pi), d0 + pi, d1 ? d1 + pi : nullptr);
     }
-}
-
-// Bring the voltages of frame pair p of channel c into L1.
-template <int FMT, int BT>
-__device__ __forceinline__ void prefetch_pair(const ImageArgs& A, long long p, int c) {
-  constexpr int esz = FMT == 0 ? 1 : 8;
-  const size_t bytes = static_cast<size_t>(A.n_ant) * esz;
-#pragma unroll
-  for (int f = 0; f < 2; ++f)
-    if (2 * p + f < A.n_time) {
-      const uintptr_t b0 = reinterpret_cast<uintptr_t>(A.volt) +
-                           (static_cast<size_t>(2 * p + f) * A.n_chan + c) * bytes;
-      for (uintptr_t q = (b0 & ~static_cast<uintptr_t>(127)) + static_cast<uintptr_t>(threadIdx.x) * 128; q < b0 + bytes;
-           q += BT * 128)
-        asm volatile("prefetch.global.L1 [%0];" ::"l"(q));
-    }
-}
-
-// A channel's tables and geometry, its tap lists in shared memory (TS) or
-// read through L1.
-struct Chan {
-  int R, R4, W4, nslice;
-  const int2* slice;
-  const int* cell;
-  const uint2* ent;
-  float vs;
-  float2 pph;
-  const float2* wg;
-};
-
-template <bool TS>
-__device__ __forceinline__ Chan channel(const ImageArgs& A, int c, const int2* sslice, const int* scell,
-                                        const uint2* sent) {
-  Chan q;
-  const int4 wn = __ldg(A.win4 + c);                       // (y0, rows, x0, cols)
-  q.R = wn.y;
-  q.R4 = (wn.y + 3) & ~3;
-  q.W4 = (wn.w + 3) & ~3;
-  const int sb = __ldg(A.psbase + c), eb = __ldg(A.pebase + c);
-  q.nslice = __ldg(A.psbase + c + 1) - sb;
-  q.slice = TS ? sslice : A.pslice + sb;
-  q.cell = TS ? scell : A.pcell + static_cast<size_t>(sb) * 32;
-  q.ent = TS ? sent : A.pent + eb;
-  q.vs = A.vscale ? __ldg(A.vscale + c) : 1.0f;
-  q.pph = A.do_cal ? __ldg(A.pixph + c) : make_float2(1.f, 0.f);
-  q.wg = A.wgain + static_cast<size_t>(c) * A.n_ant;
-  return q;
-}
-
-template <int BT>
-__device__ __forceinline__ void load_lists(const ImageArgs& A, int c, int2* sslice, int* scell, uint2* sent) {
-  const int sb = __ldg(A.psbase + c), eb = __ldg(A.pebase + c);
-  const int ns = __ldg(A.psbase + c + 1) - sb, ne = __ldg(A.pebase + c + 1) - eb;
-  for (int i = threadIdx.x; i < ns; i += BT) sslice[i] = __ldg(A.pslice + sb + i);
-  for (int i = threadIdx.x; i < ns * 32; i += BT) scell[i] = __ldg(A.pcell + static_cast<size_t>(sb) * 32 + i);
-  for (int i = threadIdx.x; i < ne; i += BT) sent[i] = __ldg(A.pent + eb + i);
 }
 
 // One antenna's EPICal sums over a run (FP32; FP64 across runs).
@@ -145,21 +68,6 @@ struct Corr {
     atomicAdd(&A.kacc[o].y, static_cast<double>(k.y));
     atomicAdd(A.pacc + o, static_cast<double>(p));
   }
-};
-
-template <int N> struct PCfg;
-template <> struct PCfg<16>  { static constexpr int BT = 32,  PER_SM = 8; };
-template <> struct PCfg<32>  { static constexpr int BT = 64,  PER_SM = 8; };
-template <> struct PCfg<64>  { static constexpr int BT = 256, PER_SM = 2; };
-template <> struct PCfg<128> { static constexpr int BT = 512, PER_SM = 1; };
-
-template <int N>
-struct PGeo {
-  static constexpr int BT = PCfg<N>::BT;
-  static constexpr int NR = N / 16;                  // residues = lanes per transform
-  static constexpr int TASKS = N * NR;               // column tasks
-  static constexpr int ROUNDS = TASKS < BT ? 1 : TASKS / BT;
-  static_assert(TASKS < BT || TASKS % BT == 0, "column tasks must fill the CTA");
 };
 
 // Two phases per frame pair, a CTA barrier after each:
@@ -370,19 +278,20 @@ bool pair_pixel_owner(int n, int kx, int ky, PixelOwner* out) {
   return true;
 }
 
-// Row stride of the spectra: room for the rows rounded up to 4, and a
+// Row stride of the spectra: room for the rows rounded up to 4 (to 8 for the
+// adjoint, whose way back permutes blocks of 8), and a
 // stride that keeps the row phase's stores free of bank conflicts (a quarter
 // warp stores NR columns of 8 / NR neighbouring rows, 16 bytes each).
-int pair_rs(int n, int rows) {
+int pair_rs(int n, int rows, bool adjoint) {
   const int nr = n / 16;
-  int rs = (rows + 3) & ~3;
+  int rs = adjoint ? (rows + 7) & ~7 : (rows + 3) & ~3;
   const int step = 8 / nr;                       // rows per quarter warp
   while (!(nr == 1 || (rs % step == 0 && (rs / step) % 2 == 1))) ++rs;
   return rs;
 }
 
-size_t pair_smem_bytes(int n, int n_ant, int rows, int gs, int max_slices, int max_ent) {
-  const size_t cells = static_cast<size_t>(n) * pair_rs(n, rows) + static_cast<size_t>(rows) * gs + n_ant + 1;
+size_t pair_smem_bytes(int n, int n_ant, int rows, int gs, int max_slices, int max_ent, bool adjoint) {
+  const size_t cells = static_cast<size_t>(n) * pair_rs(n, rows, adjoint) + static_cast<size_t>(rows) * gs + n_ant + 1;
   return cells * 16 + (2 * static_cast<size_t>(n) + 2) * sizeof(float2) +
          static_cast<size_t>(max_slices) * (sizeof(int2) + 32 * sizeof(int)) +
          static_cast<size_t>(max_ent) * sizeof(uint2);

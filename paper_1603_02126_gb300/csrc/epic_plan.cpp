@@ -715,7 +715,7 @@ epic::ImageArgs fused_args(epic_plan_t p, const void* d_volt, long long n_time, 
     a.gs = p->gs;
     a.max_slices = p->max_slices;
     a.max_ent = p->max_ent;
-    a.rs = epic::pair_rs(p->n, p->rows_alloc);
+    a.rs = epic::pair_rs(p->n, p->rows_alloc, false);
     // at least tune_units frame pairs per CTA
     const long long pairs = static_cast<long long>(p->nc) * ((n_time + 1) / 2);
     a.grid = static_cast<int>(std::max<long long>(1, std::min<long long>(pairs / p->tune_units, p->ctas)));
@@ -1328,10 +1328,10 @@ epic_status choose_path(epic_plan_s* p, const epic_plan_desc* d, bool fused_shap
     // with the tap lists beside them when they fit, else read through L1
     const int W4 = (*std::max_element(p->cols.begin(), p->cols.end()) + 3) & ~3;
     p->gs = W4 + 1;                          // odd: neighbouring rows in different banks
-    const size_t s0 = epic::pair_smem_bytes(N, Na, p->rows_alloc, p->gs, 0, 0);
+    const size_t s0 = epic::pair_smem_bytes(N, Na, p->rows_alloc, p->gs, 0, 0, false);
     if (Na <= epic::kPairMaxAnt * epic::pair_threads(N) && s0 <= static_cast<size_t>(smem_optin)) {
       build_cells(p, wts, p->gs, cells);
-      const size_t s1 = epic::pair_smem_bytes(N, Na, p->rows_alloc, p->gs, cells->max_slices, cells->max_ent);
+      const size_t s1 = epic::pair_smem_bytes(N, Na, p->rows_alloc, p->gs, cells->max_slices, cells->max_ent, false);
       p->gsmem = s1 <= static_cast<size_t>(smem_optin) ? 1 : 0;
       if (p->gsmem) {
         p->max_slices = cells->max_slices;
@@ -2532,6 +2532,25 @@ epic_status epic_image_backward(epic_plan_t p, const void* d_volt, long long n_t
     if (e != cudaSuccess) return fail(EPIC_ERR_OOM, "gradient scratch allocation failed");
   }
   EPIC_CUDA(cudaMemsetAsync(p->d_dldw.p, 0, n * sizeof(double2), p->stream));
+  if (p->pair && p->adjoint_precision == EPIC_PREC_FP32) {
+    // the frame-pair form where its shared memory fits, with the tap lists
+    // beside it if they do
+    epic::ImageArgs q = fused_args(p, d_volt, n_time, nullptr, 1.0 / static_cast<double>(n_time));
+    int most = 0;
+    EPIC_CUDA(cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device));
+    q.rs = epic::pair_rs(p->n, p->rows_alloc, true);
+    q.smem = epic::pair_smem_bytes(p->n, p->na, p->rows_alloc, p->gs, q.max_slices, q.max_ent, true);
+    if (q.gsmem && q.smem > static_cast<size_t>(most)) {
+      q.gsmem = q.max_slices = q.max_ent = 0;
+      q.smem = epic::pair_smem_bytes(p->n, p->na, p->rows_alloc, p->gs, 0, 0, true);
+    }
+    if (q.smem <= static_cast<size_t>(most)) {
+      EPIC_CUDA(epic::launch_adjoint_pair(p->n, q, d_dl_di, p->d_dldw.p, p->stream));
+      EPIC_CUDA(epic::launch_adjoint_finalize(p->nc, p->na, p->d_dldw.p, p->d_gain.p, p->d_phase.p, p->d_flags.p,
+                                              reinterpret_cast<double2*>(d_grad_g), p->stream));
+      return EPIC_OK;
+    }
+  }
   epic::AdjointArgs a{};
   a.volt = d_volt;
   a.input_fmt = p->input;
