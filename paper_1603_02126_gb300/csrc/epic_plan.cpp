@@ -180,6 +180,7 @@ struct epic_plan_s {
 
   // launch-shape parameters (autotuner) and the captured interval graph
   int tune_units = 4;           // fused: work units per CTA to aim for
+  int tune_pairs = 1;           // frame-pair form: least frame pairs per CTA
   int tune_nt = 0;              // unfused: time samples per batch (0 = budget)
   int tune_cols = 4;            // unfused: column units per SM to aim for
   int tune_row_table = -1;      // unfused row kernel: gather table -1 auto, 0 L1, 1 shared memory
@@ -716,9 +717,13 @@ epic::ImageArgs fused_args(epic_plan_t p, const void* d_volt, long long n_time, 
     a.max_slices = p->max_slices;
     a.max_ent = p->max_ent;
     a.rs = epic::pair_rs(p->n, p->rows_alloc, false);
-    // at least tune_units frame pairs per CTA
+    // at least tune_pairs frame pairs per CTA: 1, since short calls want every
+    // SM (100 pairs at N = 128: 31 us with 1, 47 with 4; 600 pairs of 4 channels
+    // at N = 32: 17 and 25), but at most 256 CTAs per channel, whose image they
+    // all add to (1000 pairs of one channel at N = 32: 250 CTAs 36 us, 500 40,
+    // 1000 56)
     const long long pairs = static_cast<long long>(p->nc) * ((n_time + 1) / 2);
-    a.grid = static_cast<int>(std::max<long long>(1, std::min<long long>(pairs / p->tune_units, p->ctas)));
+    a.grid = static_cast<int>(std::max<long long>(1, std::min<long long>({pairs / p->tune_pairs, p->ctas, 256LL * p->nc})));
   }
   return a;
 }
@@ -2365,14 +2370,15 @@ epic_status epic_autotune(epic_plan_t p, const void* d_volt, long long n_time, d
   epic_status st = EPIC_OK;
   const int reps = 3;
   if (p->path == EPIC_PATH_FUSED) {
-    const int def = p->tune_units;
+    int& knob = p->pair ? p->tune_pairs : p->tune_units;
+    const int def = knob;
     st = time_image(p, d_volt, n_time, d_image, reps, &r.ms_default);
     best = r.ms_default;
     r.units_target = def;
     const int cand[] = {1, 2, 4, 8, 16, 32};
     for (int k : cand) {
       if (st != EPIC_OK) break;
-      p->tune_units = k;
+      knob = k;
       double ms = 0;
       st = time_image(p, d_volt, n_time, d_image, reps, &ms);
       ++r.candidates;
@@ -2381,7 +2387,7 @@ epic_status epic_autotune(epic_plan_t p, const void* d_volt, long long n_time, d
         r.units_target = k;
       }
     }
-    p->tune_units = r.units_target;
+    knob = r.units_target;
   } else {
     const int def_nt = p->tune_nt, def_cols = p->tune_cols;
     st = time_image(p, d_volt, n_time, d_image, reps, &r.ms_default);
