@@ -177,6 +177,10 @@ struct epic_plan_s {
 
   // differentiation form
   DevBuf<double2> d_dldw;       // [C][Na] dL/dconj(w) accumulator
+  // one-frame fused kernel of a frame-pair plan with BF16 gradients
+  bool one_ready = false;
+  int one_steps = 1, one_gsmem = 0, one_ctas = 0;
+  size_t one_smem = 0;
 
   // launch-shape parameters (autotuner) and the captured interval graph
   int tune_units = 4;           // fused: work units per CTA to aim for
@@ -577,7 +581,7 @@ struct CellTables {
   int max_slices = 0, max_ent = 0;
 };
 
-void build_cells(const epic_plan_s* p, const std::vector<float>& wts, int gs, CellTables* t) {
+epic_status build_cells(const epic_plan_s* p, const std::vector<float>& wts, int gs, CellTables* t) {
   const int N = p->n;
   SliceLists l;
   std::vector<std::vector<Tap>> taps;
@@ -587,6 +591,8 @@ void build_cells(const epic_plan_s* p, const std::vector<float>& wts, int gs, Ce
     const int R = p->rows[c];
     block_taps(p, wts, c, gs, R, &taps);
     slice_lists(taps[0], R * gs, nullptr, p->na, &l);
+    if (!l.slice.empty() && l.slice[0].y > 255)
+      return fail(EPIC_ERR_UNSUPPORTED, "more than 255 gridding taps on one grid cell");
     t->cell.insert(t->cell.end(), l.cell.begin(), l.cell.end());
     t->slice.insert(t->slice.end(), l.slice.begin(), l.slice.end());
     t->ent.insert(t->ent.end(), l.ent.begin(), l.ent.end());
@@ -601,6 +607,7 @@ void build_cells(const epic_plan_s* p, const std::vector<float>& wts, int gs, Ce
   t->sbase.push_back(static_cast<int>(t->slice.size()));
   t->ebase.push_back(static_cast<int>(t->ent.size()));
   prefix_sums(&t->cost);
+  return EPIC_OK;
 }
 
 // Tap lists of the frame-pair forms that grid by blocks of rb window rows: per
@@ -662,6 +669,13 @@ epic_status build_wide_lists(const epic_plan_s* p, const std::vector<float>& wts
   return EPIC_OK;
 }
 
+// Whether fused calls take the frame-pair kernel.  A plan with BF16 gradients
+// keeps the one-frame kernel: the BF16 rounding of dL/dI turns a last-digit
+// difference of the image into one of 2e-5 and more of the gradient.
+bool uses_pair(const epic_plan_s* p) {
+  return p->pair && !(p->adjoint_precision == EPIC_PREC_BF16 && p->one_ready && !(p->cal && p->npix > 0));
+}
+
 // Arguments of one fused launch over a device batch.
 epic::ImageArgs fused_args(epic_plan_t p, const void* d_volt, long long n_time, double* d_image,
                            double img_scale) {
@@ -705,7 +719,7 @@ epic::ImageArgs fused_args(epic_plan_t p, const void* d_volt, long long n_time, 
   a.smem = p->smem;
   a.npix = 0;                              // epic_image arms the pixel taps itself
   a.wait_limit = p->wait_limit;
-  if (p->pair) {
+  if (uses_pair(p)) {
     a.pair = 1;
     a.pcell = p->d_pcell.p;
     a.pslice = p->d_pslice.p;
@@ -724,8 +738,59 @@ epic::ImageArgs fused_args(epic_plan_t p, const void* d_volt, long long n_time, 
     // 1000 56)
     const long long pairs = static_cast<long long>(p->nc) * ((n_time + 1) / 2);
     a.grid = static_cast<int>(std::max<long long>(1, std::min<long long>({pairs / p->tune_pairs, p->ctas, 256LL * p->nc})));
+  } else if (p->pair) {
+    a.gsmem = p->one_gsmem;
+    a.steps = p->one_steps;
+    a.smem = p->one_smem;
+    a.segs = choose_segments(p->nc, n_time, p->one_ctas, p->tune_units);
+    a.grid = static_cast<int>(std::min<long long>(static_cast<long long>(p->nc) * a.segs, p->one_ctas));
   }
   return a;
+}
+
+// Whether the FP32 adjoint takes the frame-pair form; its launch shape into q.
+bool pair_adjoint(const epic_plan_s* p, epic::ImageArgs* q) {
+  if (!p->pair) return false;
+  int most = 0;
+  if (cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device) != cudaSuccess) return false;
+  int slices = p->max_slices, ent = p->max_ent;
+  size_t smem = epic::pair_smem_bytes(p->n, p->na, p->rows_alloc, p->gs, slices, ent, true);
+  if (smem > static_cast<size_t>(most)) {                  // the tap lists through L1
+    slices = ent = 0;
+    smem = epic::pair_smem_bytes(p->n, p->na, p->rows_alloc, p->gs, 0, 0, true);
+  }
+  if (smem > static_cast<size_t>(most)) return false;
+  if (q) {
+    q->rs = epic::pair_rs(p->n, p->rows_alloc, true);
+    q->smem = smem;
+    q->gsmem = p->gsmem && slices > 0 ? 1 : 0;
+    q->max_slices = slices;
+    q->max_ent = ent;
+  }
+  return true;
+}
+
+// Absolute-column gather tables of the one-frame adjoint kernels (FP32 where
+// the frame-pair form does not fit, and BF16), once per plan.
+epic_status ensure_adjoint_tables(epic_plan_s* p, const std::vector<float>& wts) {
+  if (p->d_ugofs.p) return EPIC_OK;
+  std::vector<int> ofs, base;
+  std::vector<uint4> cnt;
+  std::vector<uint2> ent;
+  if (epic_status st = build_gather(p, wts, epic::image_fft_lanes(p->n), false, ofs, cnt, ent, base)) return st;
+  cudaError_t es[] = {p->d_ugcnt.alloc(cnt.size()), p->d_ugent.alloc(ent.size()), p->d_ugbase.alloc(base.size()),
+                      p->d_ugofs.alloc(ofs.size())};
+  for (cudaError_t e : es)
+    if (e != cudaSuccess) {
+      p->d_ugofs.release();
+      return e == cudaErrorMemoryAllocation ? fail(EPIC_ERR_OOM, "device allocation failed")
+                                            : cuda_fail(e, "table upload");
+    }
+  EPIC_CUDA(cudaMemcpy(p->d_ugofs.p, ofs.data(), ofs.size() * sizeof(int), cudaMemcpyHostToDevice));
+  EPIC_CUDA(cudaMemcpy(p->d_ugcnt.p, cnt.data(), cnt.size() * sizeof(uint4), cudaMemcpyHostToDevice));
+  EPIC_CUDA(cudaMemcpy(p->d_ugent.p, ent.data(), ent.size() * sizeof(uint2), cudaMemcpyHostToDevice));
+  EPIC_CUDA(cudaMemcpy(p->d_ugbase.p, base.data(), base.size() * sizeof(int), cudaMemcpyHostToDevice));
+  return EPIC_OK;
 }
 
 // Cluster path: one persistent launch of thread-block clusters.
@@ -1153,6 +1218,23 @@ epic_status validate_desc(const epic_plan_desc* d, epic::ImageKernelShape* shape
   return EPIC_OK;
 }
 
+// Taps of every unflagged antenna with the centring sign of Eq. 10 and 1/Na
+// folded in, [C][Na][K*K].
+void fold_weights(const epic_plan_s* p, std::vector<float>& wts) {
+  const int Na = p->na, K = p->k, KK = K * K, h = (K - 1) / 2;
+  for (int c = 0; c < p->nc; ++c)
+    for (int a = 0; a < Na; ++a) {
+      if (p->flags[a]) continue;
+      const size_t i = static_cast<size_t>(c) * Na + a;
+      const int bx = p->base[2 * i], by = p->base[2 * i + 1];
+      for (int dy = 0; dy < K; ++dy)
+        for (int dx = 0; dx < K; ++dx) {
+          const double sgn = ((bx + dx - h + by + dy - h) & 1) ? -1.0 : 1.0;
+          wts[i * KK + dy * K + dx] = static_cast<float>(p->w64[i * KK + dy * K + dx] * sgn / Na);
+        }
+    }
+}
+
 // Gridding tables of Eq. 9 in FP64 (stencil centres p->base, normalised
 // taps p->w64), every channel's occupied window (y0, rows, x0, cols), and
 // the device forms: cell0 [C][Na] = window row * N + absolute column of
@@ -1233,20 +1315,30 @@ epic_status build_grid_tables(epic_plan_s* p, std::vector<int>& cell0, std::vect
     for (int a = 0; a < Na; ++a) {
       if (p->flags[a]) continue;
       const size_t ob = (static_cast<size_t>(c) * Na + a) * 2;
-      const int bx = p->base[ob], by = p->base[ob + 1];
-      cell0[static_cast<size_t>(c) * Na + a] = (by - h - ymin) * N + (bx - h);
-      const double* w = &p->w64[(static_cast<size_t>(c) * Na + a) * KK];
-      float* wf = &wts[(static_cast<size_t>(c) * Na + a) * KK];
-      for (int dy = 0; dy < K; ++dy)
-        for (int dx = 0; dx < K; ++dx) {
-          const int jx = bx + dx - h, jy = by + dy - h;
-          const double sgn = ((jx + jy) & 1) ? -1.0 : 1.0;   // centring of Eq. 10
-          wf[dy * K + dx] = static_cast<float>(w[dy * K + dx] * sgn / Na);
-        }
+      cell0[static_cast<size_t>(c) * Na + a] = (p->base[ob + 1] - h - ymin) * N + (p->base[ob] - h);
     }
   }
-
+  fold_weights(p, wts);
   return EPIC_OK;
+}
+
+// Shape of the one-frame fused kernel: two frames per step, then one; the
+// gather table in shared memory when it fits (entries per channel <= Na K^2
+// taps), else read through L1.  False: no shape fits.
+bool one_frame_shape(const epic_plan_s* p, int smem_optin, int* steps_out, int* gsmem, size_t* smem) {
+  const int n1 = epic::image_fft_lanes(p->n);
+  const size_t tab = epic::image_table_bytes(p->rows_alloc, n1, static_cast<long long>(p->na) * p->k * p->k);
+  for (int steps = epic::image_max_steps(p->n); steps >= 1; --steps)
+    for (int ts = 1; ts >= 0; --ts) {
+      const size_t need = epic::image_smem_bytes(p->n, p->na, p->rs_fused, steps) + (ts ? tab : 0);
+      if (need <= static_cast<size_t>(smem_optin)) {
+        *smem = need;
+        *gsmem = ts;
+        *steps_out = steps;
+        return true;
+      }
+    }
+  return false;
 }
 
 // Tables and launch shape of the wide frame-pair form where a pair of one
@@ -1270,6 +1362,33 @@ epic_status plan_wide(epic_plan_s* p, const std::vector<float>& wts, WideTables*
   p->w_rows_ctas = rows_per_sm * p->sms;
   p->w_cols_ctas = cols_per_sm * p->sms;
   if (!p->wide) *wide = WideTables();
+  return EPIC_OK;
+}
+
+// The one-frame fused kernel's tables and launch shape of a frame-pair plan.
+epic_status ensure_one_frame(epic_plan_s* p) {
+  int most = 0, per_sm = 0;
+  EPIC_CUDA(cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device));
+  if (!one_frame_shape(p, most, &p->one_steps, &p->one_gsmem, &p->one_smem)) return EPIC_OK;
+  EPIC_CUDA(epic::image_kernel_prepare(p->n, p->one_smem, p->na, p->one_steps, &per_sm));
+  if (per_sm < 1) return EPIC_OK;
+  std::vector<float> wts(p->w64.size(), 0.0f);
+  fold_weights(p, wts);
+  std::vector<int> ofs, base;
+  std::vector<uint4> cnt;
+  std::vector<uint2> ent;
+  if (epic_status st = build_gather(p, wts, epic::image_fft_lanes(p->n), true, ofs, cnt, ent, base)) return st;
+  cudaError_t es[] = {p->d_gofs.alloc(ofs.size()), p->d_gcnt.alloc(cnt.size()), p->d_gent.alloc(ent.size()),
+                      p->d_gbase.alloc(base.size())};
+  for (cudaError_t e : es)
+    if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? fail(EPIC_ERR_OOM, "device allocation failed")
+                                                                : cuda_fail(e, "table upload");
+  EPIC_CUDA(cudaMemcpy(p->d_gofs.p, ofs.data(), ofs.size() * sizeof(int), cudaMemcpyHostToDevice));
+  EPIC_CUDA(cudaMemcpy(p->d_gcnt.p, cnt.data(), cnt.size() * sizeof(uint4), cudaMemcpyHostToDevice));
+  EPIC_CUDA(cudaMemcpy(p->d_gent.p, ent.data(), ent.size() * sizeof(uint2), cudaMemcpyHostToDevice));
+  EPIC_CUDA(cudaMemcpy(p->d_gbase.p, base.data(), base.size() * sizeof(int), cudaMemcpyHostToDevice));
+  p->one_ctas = per_sm * p->sms;
+  p->one_ready = true;
   return EPIC_OK;
 }
 
@@ -1335,7 +1454,7 @@ epic_status choose_path(epic_plan_s* p, const epic_plan_desc* d, bool fused_shap
     p->gs = W4 + 1;                          // odd: neighbouring rows in different banks
     const size_t s0 = epic::pair_smem_bytes(N, Na, p->rows_alloc, p->gs, 0, 0, false);
     if (Na <= epic::kPairMaxAnt * epic::pair_threads(N) && s0 <= static_cast<size_t>(smem_optin)) {
-      build_cells(p, wts, p->gs, cells);
+      if (epic_status st = build_cells(p, wts, p->gs, cells)) return st;
       const size_t s1 = epic::pair_smem_bytes(N, Na, p->rows_alloc, p->gs, cells->max_slices, cells->max_ent, false);
       p->gsmem = s1 <= static_cast<size_t>(smem_optin) ? 1 : 0;
       if (p->gsmem) {
@@ -1347,23 +1466,7 @@ epic_status choose_path(epic_plan_s* p, const epic_plan_desc* d, bool fused_shap
     }
   }
   if (fused && !p->piped && !p->pair) {
-    // shape preference: two frames per step, then one; the gather table in
-    // shared memory when it fits (entries per channel <= Na K^2 taps), else
-    // read through L1
-    const int n1 = epic::image_fft_lanes(N);
-    const long long gmax = static_cast<long long>(Na) * KK;
-    const size_t tab = epic::image_table_bytes(p->rows_alloc, n1, gmax);
-    bool placed = false;
-    for (int steps = epic::image_max_steps(N); steps >= 1 && !placed; --steps)
-      for (int ts = 1; ts >= 0 && !placed; --ts) {
-        const size_t need = epic::image_smem_bytes(N, Na, p->rs_fused, steps) + (ts ? tab : 0);
-        if (need <= static_cast<size_t>(smem_optin)) {
-          p->smem = need;
-          p->gsmem = ts;
-          p->steps = steps;
-          placed = true;
-        }
-      }
+    const bool placed = one_frame_shape(p, smem_optin, &p->steps, &p->gsmem, &p->smem);
     if (!placed) {
       const std::string msg = "array footprint needs " +
                               std::to_string(epic::image_smem_bytes(N, Na, p->rs_fused, 1)) +
@@ -1536,11 +1639,11 @@ epic_status epic_plan_create(epic_plan_t* out, const epic_plan_desc* d) {
       cellf[static_cast<size_t>(c) * Na + a] = (by - h - p->y0[c]) * ws + (bx - h - p->x0[c]);
     }
   // gridding gather tables (see build_gather): the fused kernel, the plain
-  // unfused path and the reduced-precision gridding use window columns, the
-  // fused path's adjoint absolute columns
-  std::vector<int> gofs, gbase, ugofs, ugbase;
-  std::vector<uint4> gcnt, ugcnt;
-  std::vector<uint2> gent, ugent;
+  // unfused path use window columns, the one-frame adjoint absolute columns
+  // (ensure_adjoint_tables)
+  std::vector<int> gofs, gbase;
+  std::vector<uint4> gcnt;
+  std::vector<uint2> gent;
   if (p->path == EPIC_PATH_FUSED ? !p->pair
                                  : (p->path == EPIC_PATH_UNFUSED && !p->wide && p->precision == EPIC_PREC_FP32)) {
     const int n1 = p->path == EPIC_PATH_FUSED ? epic::image_fft_lanes(N) : epic::unfused_fft_lanes(N);
@@ -1549,13 +1652,6 @@ epic_status epic_plan_create(epic_plan_t* out, const epic_plan_desc* d) {
       return st;
     }
     for (int c = 0; c < C; ++c) p->gmax = std::max(p->gmax, gbase[c + 1] - gbase[c]);
-  }
-  if (p->path == EPIC_PATH_FUSED) {
-    const int n1 = epic::image_fft_lanes(N);
-    if (epic_status st = build_gather(p, wts, n1, false, ugofs, ugcnt, ugent, ugbase)) {
-      epic_plan_destroy(p);
-      return st;
-    }
   }
   std::vector<float2> pixph(C, make_float2(1.0f, 0.0f));
   std::vector<int> rowcol, order;
@@ -1575,8 +1671,7 @@ epic_status epic_plan_create(epic_plan_t* out, const epic_plan_desc* d) {
                       up(p->d_cellf, cellf), up(p->d_pixph, pixph), up(p->d_rowcol, rowcol),
                       up(p->d_order, order), up(p->d_ranges, ranges), up(p->d_gofs, gofs),
                       up(p->d_gent, gent), up(p->d_gbase, gbase), up(p->d_gcnt, gcnt),
-                      up(p->d_ugofs, ugofs), up(p->d_ugcnt, ugcnt), up(p->d_ugent, ugent),
-                      up(p->d_ugbase, ugbase), up(p->d_pcell, cells.cell), up(p->d_pslice, cells.slice),
+                      up(p->d_pcell, cells.cell), up(p->d_pslice, cells.slice),
                       up(p->d_pent, cells.ent), up(p->d_psbase, cells.sbase), up(p->d_pebase, cells.ebase),
                       up(p->d_pcost, cells.cost), up(p->d_wlists, wide.lists), up(p->d_wat, wide.at),
                       up(p->d_wrcost, wide.row_cost), up(p->d_wccost, wide.col_cost)};
@@ -1596,6 +1691,11 @@ epic_status epic_plan_create(epic_plan_t* out, const epic_plan_desc* d) {
     epic_plan_destroy(p);
     return cuda_fail(e, "counter");
   }
+  if (p->path == EPIC_PATH_FUSED && !pair_adjoint(p, nullptr))
+    if (epic_status st = ensure_adjoint_tables(p, wts)) {
+      epic_plan_destroy(p);
+      return st;
+    }
   *out = p;
   return EPIC_OK;
 }
@@ -1732,7 +1832,8 @@ epic_status epic_image(epic_plan_t p, const void* d_volt, long long n_time, doub
   if (p->precision != EPIC_PREC_FP32) return image_tc(p, d_volt, n_time, d_image);
   if (p->path == EPIC_PATH_CLUSTER) return image_cluster(p, d_volt, n_time, d_image);
   if (p->path == EPIC_PATH_UNFUSED) return image_unfused(p, d_volt, n_time, d_image);
-  if (p->wide && !(p->cal && p->npix > 0) && wide_ready(p, n_time)) return image_wide(p, d_volt, n_time, d_image);
+  if (p->wide && p->adjoint_precision != EPIC_PREC_BF16 && !(p->cal && p->npix > 0) && wide_ready(p, n_time))
+    return image_wide(p, d_volt, n_time, d_image);
   epic::ImageArgs a = fused_args(p, d_volt, n_time, d_image, 1.0 / static_cast<double>(n_time));
   if (p->cal && p->npix > 0) {
     if (epic_status st = ensure_ptap(p, n_time)) return st;
@@ -2218,6 +2319,13 @@ epic_status epic_plan_set_adjoint_precision(epic_plan_t p, int precision) {
   if (epic_status s = check_plan(p)) return s;
   if (precision != EPIC_PREC_FP32 && precision != EPIC_PREC_BF16)
     return fail(EPIC_ERR_INVALID_ARG, "adjoint precision must be EPIC_PREC_FP32 or EPIC_PREC_BF16");
+  if (precision == EPIC_PREC_BF16 && p->path == EPIC_PATH_FUSED && !p->d_ugofs.p) {
+    std::vector<float> wts(p->w64.size(), 0.0f);
+    fold_weights(p, wts);
+    if (epic_status st = ensure_adjoint_tables(p, wts)) return st;
+  }
+  if (precision == EPIC_PREC_BF16 && p->pair && !p->one_ready)
+    if (epic_status st = ensure_one_frame(p)) return st;
   p->adjoint_precision = precision;
   return EPIC_OK;
 }
@@ -2370,7 +2478,7 @@ epic_status epic_autotune(epic_plan_t p, const void* d_volt, long long n_time, d
   epic_status st = EPIC_OK;
   const int reps = 3;
   if (p->path == EPIC_PATH_FUSED) {
-    int& knob = p->pair ? p->tune_pairs : p->tune_units;
+    int& knob = uses_pair(p) ? p->tune_pairs : p->tune_units;
     const int def = knob;
     st = time_image(p, d_volt, n_time, d_image, reps, &r.ms_default);
     best = r.ms_default;
@@ -2539,18 +2647,8 @@ epic_status epic_image_backward(epic_plan_t p, const void* d_volt, long long n_t
   }
   EPIC_CUDA(cudaMemsetAsync(p->d_dldw.p, 0, n * sizeof(double2), p->stream));
   if (p->pair && p->adjoint_precision == EPIC_PREC_FP32) {
-    // the frame-pair form where its shared memory fits, with the tap lists
-    // beside it if they do
     epic::ImageArgs q = fused_args(p, d_volt, n_time, nullptr, 1.0 / static_cast<double>(n_time));
-    int most = 0;
-    EPIC_CUDA(cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device));
-    q.rs = epic::pair_rs(p->n, p->rows_alloc, true);
-    q.smem = epic::pair_smem_bytes(p->n, p->na, p->rows_alloc, p->gs, q.max_slices, q.max_ent, true);
-    if (q.gsmem && q.smem > static_cast<size_t>(most)) {
-      q.gsmem = q.max_slices = q.max_ent = 0;
-      q.smem = epic::pair_smem_bytes(p->n, p->na, p->rows_alloc, p->gs, 0, 0, true);
-    }
-    if (q.smem <= static_cast<size_t>(most)) {
+    if (pair_adjoint(p, &q)) {
       EPIC_CUDA(epic::launch_adjoint_pair(p->n, q, d_dl_di, p->d_dldw.p, p->stream));
       EPIC_CUDA(epic::launch_adjoint_finalize(p->nc, p->na, p->d_dldw.p, p->d_gain.p, p->d_phase.p, p->d_flags.p,
                                               reinterpret_cast<double2*>(d_grad_g), p->stream));
@@ -2573,17 +2671,18 @@ epic_status epic_image_backward(epic_plan_t p, const void* d_volt, long long n_t
   a.dldi = d_dl_di;
   a.dldw = p->d_dldw.p;
   a.img_scale = 1.0 / static_cast<double>(n_time);
-  a.segs = choose_segments(p->nc, n_time, p->ctas, p->tune_units);
+  const bool bf16 = p->adjoint_precision == EPIC_PREC_BF16;
+  a.smem = epic::adjoint_smem_bytes(p->n, p->rows_alloc, p->rs, p->na, bf16);
+  const int ctas = !p->pair ? p->ctas : p->one_ctas ? p->one_ctas : p->sms;
+  a.segs = choose_segments(p->nc, n_time, ctas, p->tune_units);
   a.rows_alloc = p->rows_alloc;
   a.rs = p->rs;
   const long long units = static_cast<long long>(p->nc) * a.segs;
-  a.grid = static_cast<int>(std::min<long long>(units, p->ctas));
+  a.grid = static_cast<int>(std::min<long long>(units, ctas));
   a.gofs = p->d_ugofs.p;
   a.gcnt = p->d_ugcnt.p;
   a.gent = p->d_ugent.p;
   a.gbase = p->d_ugbase.p;
-  const bool bf16 = p->adjoint_precision == EPIC_PREC_BF16;
-  a.smem = epic::adjoint_smem_bytes(p->n, p->rows_alloc, p->rs, p->na, bf16);
   EPIC_CUDA(epic::launch_adjoint(p->n, a, bf16, p->stream));
   EPIC_CUDA(epic::launch_adjoint_finalize(p->nc, p->na, p->d_dldw.p, p->d_gain.p, p->d_phase.p, p->d_flags.p,
                                           reinterpret_cast<double2*>(d_grad_g), p->stream));
