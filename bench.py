@@ -48,9 +48,9 @@ TRAFFIC = {"kernel_sha": "ffbd609a2fe4", "bytes_per_launch": 182208512}
 
 def kernel_sha() -> str:
     """sha256 (first 12 hex) of the fused kernel's sources (kernel file and
-    the FFT helpers it inlines)."""
+    the helpers it inlines)."""
     h = hashlib.sha256()
-    for f in ("epic_kernels.cu", "epic_fft.cuh"):
+    for f in ("epic_pair.cu", "epic_pair.cuh", "epic_residue.cuh", "epic_lists.cuh", "epic_fft.cuh"):
         h.update(open(os.path.join(ROOT, "paper_1603_02126_gb300", "csrc", f), "rb").read())
     return h.hexdigest()[:12]
 
@@ -743,7 +743,7 @@ def main():
             "image_ms_without_epical": float(np.mean(nocal)),
             "roofline": {"bound": "alu", "achieved": achieved, "peak": alu_peak,
                          "unit": "TFLOP/s", "frac": achieved / alu_peak, "traffic": traffic,
-                         "kernel": "epic_image_fused<128,1>",
+                         "kernel": "epic_image_pair<128>",
                          "peak_source": "measured in this run: FP32 FMA microbenchmark "
                                         "(epic_measure_fma_peak, 152 x 8 CTAs x 256 threads, "
                                         "8 independent chains per thread, CUDA events)",
