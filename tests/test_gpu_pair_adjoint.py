@@ -59,3 +59,29 @@ def test_pair_adjoint(n, na, rows, cols, T, fmt, support):
     grad = p.image_backward(dev, dl).cpu().numpy()
     assert np.linalg.norm(grad - ref) / np.linalg.norm(ref) <= 1e-4
     assert np.all(grad[:, 2] == 0)
+
+
+@pytest.mark.parametrize("n,na,T", [(32, 40, 5), (64, 300, 33), (128, 60, 4)])
+def test_image_of_bf16_gradient_plan(n, na, T):
+    """Images and gains of a plan whose gradients are BF16 (the one-frame
+    kernel), and of the same plan set back to FP32.  Relative L2 <= 1e-5,
+    gains <= 1e-4."""
+    from paper_1603_02126_gb300 import Plan
+    rng = np.random.default_rng(70 + n)
+    half = 7 * 299792458.0 / 50e6
+    ant = rng.uniform(-half, half, (na, 2))
+    freqs = [50e6, 46.1e6]
+    sky = np.array([[0.0, 0.0, 4.0], [0.2, -0.15, 1.5]])
+    g0 = synth.true_gains(2, na, rng)
+    E = synth.voltages(ant, freqs, g0, sky, T, 0.3, rng).astype(np.complex64)
+    oplan = O.Plan(ant, freqs, n, 0.5, support=3, model_lmS=sky)
+    g_ref, _, _, ref, _ = O.epical_interval(oplan, E.astype(np.complex128), g0, 0.5)
+    dev = torch.from_numpy(E).cuda()
+    p = Plan(ant, freqs, n, 0.5, support=3, input="c64")
+    for precision in ("bf16", "fp32"):
+        p.set_adjoint_precision(precision)
+        p.configure((0.0, 0.0), sky, 0.5, g0=g0)
+        img = p.image(dev).cpu().numpy()
+        p.update()
+        assert np.linalg.norm(img - ref) / np.linalg.norm(ref) <= 1e-5
+        assert np.max(np.abs(p.gains() - g_ref) / np.abs(g_ref)) <= 1e-4
