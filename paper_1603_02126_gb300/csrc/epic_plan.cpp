@@ -15,6 +15,7 @@
 #include <string>
 #include <vector>
 
+#include "epic_batch.h"
 #include "epic_internal.h"
 
 namespace {
@@ -848,35 +849,8 @@ void wide_plan_args(const epic_plan_s* p, epic::WideArgs* w) {
   w->cols_ctas = p->w_cols_ctas;
 }
 
-// Batch of the wide frame-pair form: samples per batch and channels per
-// launch.  All samples that fit with every channel, or kWideTime of them with
-// fewer channels (an image block is added to once per batch and share).  The
-// whole scratch budget is used: a launch costs its start and its tail, and
-// batches that stay in L2 were slower (1024 antennas, 256 x 256: 48 MB 29.5,
-// 200 MB 20.7, 512 MB 17.9, 2 GB 16.6 ms).
-struct WideBatch {
-  long long nt = 0;
-  int nc = 0;
-  size_t spec_n = 0, need = 0;   // float2 of the spectra, of the whole scratch
-};
-
-WideBatch wide_batch(const epic_plan_s* p, long long n_time) {
-  constexpr long long kWideTime = 256;
-  const int C = p->nc, N = p->n;
-  const size_t chan_t = static_cast<size_t>(N) * p->rs * sizeof(float2);   // one sample of one channel
-  const size_t budget = p->workspace_budget;
-  WideBatch b;
-  b.nt = std::min<long long>((n_time + 1) / 2 * 2,
-                             std::max<long long>(kWideTime, static_cast<long long>(budget / (chan_t * C))));
-  if (p->tune_nt > 0) b.nt = std::max<long long>(2, std::min<long long>(b.nt, p->tune_nt / 2 * 2));
-  b.nt = std::max<long long>(2, std::min<long long>(b.nt, static_cast<long long>(budget / chan_t) / 2 * 2));
-  const long long fit = static_cast<long long>(budget / (chan_t * static_cast<size_t>(b.nt)));
-  const int most = static_cast<int>(std::max<long long>(1, std::min<long long>(fit, C)));
-  const int groups = (C + most - 1) / most;
-  b.nc = (C + groups - 1) / groups;
-  b.spec_n = static_cast<size_t>(b.nt) * b.nc * N * p->rs;
-  b.need = b.spec_n + static_cast<size_t>(b.nt) * C;
-  return b;
+epic::WideBatch wide_batch(const epic_plan_s* p, long long n_time) {
+  return epic::wide_batch(p->nc, p->n, p->rs, p->workspace_budget, p->tune_nt, n_time);
 }
 
 // Whether a fused plan can take the wide form for this call: its scratch is
@@ -898,7 +872,7 @@ bool wide_ready(epic_plan_t p, long long n_time) {
 // Frame-pair form of the plain path.
 epic_status image_wide(epic_plan_t p, const void* d_volt, long long n_time, double* d_image) {
   const int C = p->nc;
-  const WideBatch wb = wide_batch(p, n_time);
+  const epic::WideBatch wb = wide_batch(p, n_time);
   const long long nt = wb.nt;
   const int nc = wb.nc;
   const size_t spec_n = wb.spec_n, need = wb.need;
