@@ -86,7 +86,11 @@ typedef struct {
                                   (column DFT on tensor cores, UNFUSED/AUTO path) */
   void* cuda_stream;           /* cudaStream_t for all work; NULL = default */
   int path;                    /* epic_path */
-  size_t workspace_bytes;      /* UNFUSED batch scratch budget; 0 = 2 GiB */
+  size_t workspace_bytes;      /* batch scratch budget; 0 = 2 GiB.  UNFUSED: allocated by the first
+                                  call, grown by longer ones up to the budget.  FUSED, N = 128, where
+                                  the footprint leaves no room for two frames on one SM: allocated at
+                                  creation (at most 2 GiB, less where the device has less) and kept,
+                                  image calls allocate nothing; other FUSED plans hold none */
   const double* kernel_param_ant;  /* host [Na]: kernel_param per antenna (heterogeneous
                                       illumination patterns), or NULL = kernel_param for all */
   int batch_persistent;        /* UNFUSED FP32, N = 256 or 512: 1 = every epic_image call is one

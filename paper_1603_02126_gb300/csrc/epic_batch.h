@@ -39,4 +39,11 @@ inline WideBatch wide_batch(int C, int N, int rs, size_t budget, int tune_nt, lo
   return b;
 }
 
+// float2 of a scratch that every call of a plan fits, whatever its n_time.
+inline size_t wide_scratch(int C, int N, int rs, size_t budget) {
+  const size_t frames = budget / (static_cast<size_t>(N) * rs * 8);
+  const long long nt = wide_batch(C, N, rs, budget, 0, 1LL << 40).nt;
+  return frames * N * rs + static_cast<size_t>(nt) * C;
+}
+
 }  // namespace epic

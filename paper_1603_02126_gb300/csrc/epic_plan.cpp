@@ -90,6 +90,8 @@ float2 gain_multiplier_host(const std::vector<double2>& phase, size_t i, double 
 }
 }  // namespace
 
+constexpr size_t kDefaultWorkspace = static_cast<size_t>(2) << 30;
+
 struct epic_plan_s {
   // description
   int na = 0, nc = 0, n = 0, k = 0, input = 0, kernel = 0;
@@ -172,7 +174,7 @@ struct epic_plan_s {
 
   // path and unfused scratch
   int path = EPIC_PATH_FUSED;
-  size_t workspace_budget = static_cast<size_t>(2) << 30;
+  size_t workspace_budget = kDefaultWorkspace;
   DevBuf<float2> d_ws;          // unfused scratch: [nt*C] x (N*rs + 1)
   int ws_time = 0;              // time samples the scratch holds
 
@@ -853,22 +855,6 @@ epic::WideBatch wide_batch(const epic_plan_s* p, long long n_time) {
   return epic::wide_batch(p->nc, p->n, p->rs, p->workspace_budget, p->tune_nt, n_time);
 }
 
-// Whether a fused plan can take the wide form for this call: its scratch is
-// there, or can be allocated (not while the stream is being captured).
-bool wide_ready(epic_plan_t p, long long n_time) {
-  const size_t need = wide_batch(p, n_time).need;
-  if (p->d_ws.n >= need) return true;
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(p->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
-    cudaGetLastError();
-    return false;
-  }
-  if (cudaStreamSynchronize(p->stream) != cudaSuccess) return false;
-  if (p->d_ws.alloc(need) == cudaSuccess) return true;
-  cudaGetLastError();
-  return false;
-}
-
 // Frame-pair form of the plain path.
 epic_status image_wide(epic_plan_t p, const void* d_volt, long long n_time, double* d_image) {
   const int C = p->nc;
@@ -1339,6 +1325,25 @@ epic_status plan_wide(epic_plan_s* p, const std::vector<float>& wts, WideTables*
   return EPIC_OK;
 }
 
+// Scratch of a fused plan in its wide form, once, for calls of any length:
+// epic_image of a fused plan allocates nothing and does not wait, and what a
+// captured graph binds stays where it is.  At most the default budget, less
+// where the device has less; without room for a pair the plan keeps the
+// one-frame kernel.
+void hold_wide_scratch(epic_plan_s* p, WideTables* wide) {
+  if (!p->wide) return;
+  const size_t pair_bytes = 2 * static_cast<size_t>(p->n) * p->rs * sizeof(float2);
+  for (size_t budget = std::min(p->workspace_budget, kDefaultWorkspace); budget >= pair_bytes; budget /= 2) {
+    if (p->d_ws.alloc(epic::wide_scratch(p->nc, p->n, p->rs, budget)) == cudaSuccess) {
+      p->workspace_budget = budget;
+      return;
+    }
+    cudaGetLastError();
+  }
+  p->wide = false;
+  *wide = WideTables();
+}
+
 // The one-frame fused kernel's tables and launch shape of a frame-pair plan.
 epic_status ensure_one_frame(epic_plan_s* p) {
   int most = 0, per_sm = 0;
@@ -1489,10 +1494,12 @@ epic_status choose_path(epic_plan_s* p, const epic_plan_desc* d, bool fused_shap
     p->ctas = per_sm * p->sms;
     p->path = EPIC_PATH_FUSED;
     // footprints that leave no room for two frames on one SM: the spectra of
-    // a pair through HBM (N = 128); multiple-pixel EPICal and calls that may
-    // not allocate stay with the one-frame kernel
-    if (!p->pair && !p->piped)
+    // a pair through HBM (N = 128); multiple-pixel EPICal and
+    // epic_image_host_static stay with the one-frame kernel
+    if (!p->pair && !p->piped) {
       if (epic_status st = plan_wide(p, wts, wide)) return st;
+      hold_wide_scratch(p, wide);
+    }
   } else {
     p->smem = 0;
     p->ctas = p->sms;
@@ -1806,7 +1813,7 @@ epic_status epic_image(epic_plan_t p, const void* d_volt, long long n_time, doub
   if (p->precision != EPIC_PREC_FP32) return image_tc(p, d_volt, n_time, d_image);
   if (p->path == EPIC_PATH_CLUSTER) return image_cluster(p, d_volt, n_time, d_image);
   if (p->path == EPIC_PATH_UNFUSED) return image_unfused(p, d_volt, n_time, d_image);
-  if (p->wide && p->adjoint_precision != EPIC_PREC_BF16 && !(p->cal && p->npix > 0) && wide_ready(p, n_time))
+  if (p->wide && p->adjoint_precision != EPIC_PREC_BF16 && !(p->cal && p->npix > 0))
     return image_wide(p, d_volt, n_time, d_image);
   epic::ImageArgs a = fused_args(p, d_volt, n_time, d_image, 1.0 / static_cast<double>(n_time));
   if (p->cal && p->npix > 0) {
@@ -2547,7 +2554,7 @@ epic_status epic_graph_capture(epic_plan_t p, const void* d_volt, long long n_ti
   if (p->cal && p->frames != 0)
     return fail(EPIC_ERR_STATE, "update EPICal before capturing (frames are pending)");
   if (epic_status st = ensure_ptap(p, n_time)) return st;    // multiple-pixel taps
-  if (p->path == EPIC_PATH_UNFUSED || p->wide) {
+  if (p->path == EPIC_PATH_UNFUSED) {
     // allocate the batch scratch outside the capture
     const bool cal = p->cal;
     const long long frames = p->frames;

@@ -22,7 +22,7 @@ int main() {
   long long T;
   while (std::scanf("%d %d %d %llu %d %lld", &C, &N, &rs, &budget, &tune, &T) == 6) {
     const epic::WideBatch b = epic::wide_batch(C, N, rs, budget, tune, T);
-    std::printf("%lld %d %zu %zu\n", b.nt, b.nc, b.spec_n, b.need);
+    std::printf("%lld %d %zu %zu %zu\n", b.nt, b.nc, b.spec_n, b.need, epic::wide_scratch(C, N, rs, budget));
   }
   return 0;
 }
@@ -65,7 +65,7 @@ def _cases():
 
 def test_every_batch_fits_its_scratch(batch_of):
     cases = list(_cases())
-    for (C, N, rs, budget, tune, T), (nt, nc, spec_n, need) in zip(cases, batch_of(cases)):
+    for (C, N, rs, budget, tune, T), (nt, nc, spec_n, need, held) in zip(cases, batch_of(cases)):
         case = (C, N, rs, budget, tune, T, nt, nc)
         assert nt >= 2 and nt % 2 == 0, case
         assert 1 <= nc <= C, case
@@ -74,3 +74,4 @@ def test_every_batch_fits_its_scratch(batch_of):
         assert 2 * pairs * nc * N * rs <= spec_n, case      # spectra end before the pixels
         assert spec_n + max(sizes) * C <= need, case        # pixels end inside the scratch
         assert spec_n * 8 <= budget, case
+        assert need <= held, case                           # a scratch held for calls of any length
