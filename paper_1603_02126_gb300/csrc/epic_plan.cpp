@@ -55,6 +55,7 @@ template <typename T>
 struct DevBuf {
   T* p = nullptr;
   size_t n = 0;
+  bool bound = false;           // a captured call holds its address
   cudaError_t alloc(size_t count) {
     release();
     if (count == 0) return cudaSuccess;
@@ -67,6 +68,7 @@ struct DevBuf {
     if (p) cudaFree(p);
     p = nullptr;
     n = 0;
+    bound = false;
   }
 };
 
@@ -197,6 +199,7 @@ struct epic_plan_s {
   int adjoint_precision = EPIC_PREC_FP32;   // arithmetic of the adjoint's transforms
   DevBuf<unsigned> d_gbar;      // grid barrier {count, generation, abort}
   cudaGraph_t graph = nullptr;
+  std::vector<void*> retired;   // replaced buffers that a captured call holds (see drop)
   cudaGraphExec_t graph_exec = nullptr;
 
   // reduced-precision form (tensor-core column DFT)
@@ -380,16 +383,53 @@ float2 window_phase(epic_plan_t p, int c, int kx, int ky) {
 
 // Tap buffer of the multiple-pixel form for calls of up to n_time samples
 // (grown outside any stream capture: epic_graph_capture sizes it first).
+// Buffers that a later call may replace: when this call is being captured
+// (by epic_graph_capture or by the caller), its graph holds their addresses.
+void bind_captured(epic_plan_s* p) {
+  if (!p->d_ws.p && !p->d_ptap.p && !p->d_phase.p && !p->d_xe_z.p) return;
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(p->stream, &st) != cudaSuccess) {
+    cudaGetLastError();
+    return;
+  }
+  if (st == cudaStreamCaptureStatusNone) return;
+  p->d_ws.bound = p->d_ptap.bound = p->d_phase.bound = p->d_xe_z.bound = true;
+  p->d_ap.bound = p->d_dp.bound = p->d_kmp.bound = p->d_gdir.bound = p->d_ptab.bound = p->d_pph.bound = true;
+}
+
+// Gives a buffer up: freed, or kept to the plan's end where a graph holds it.
+template <typename T>
+void drop(epic_plan_s* p, DevBuf<T>& b) {
+  if (b.bound && b.p) {
+    p->retired.push_back(b.p);
+    b.p = nullptr;
+  }
+  b.release();
+}
+
+// Replaces a buffer by one of at least `need` entries (at most `most` unless
+// need is more); in place of one that a graph holds at least twice as large,
+// so that what is kept stays below the size of the last.
+template <typename T>
+cudaError_t grow(epic_plan_s* p, DevBuf<T>& b, size_t need, size_t most) {
+  const size_t twice = b.bound ? std::max(need, std::min(2 * b.n, most)) : need;
+  drop(p, b);
+  if (b.alloc(twice) == cudaSuccess) return cudaSuccess;
+  cudaGetLastError();
+  return b.alloc(need);
+}
+
 epic_status ensure_ptap(epic_plan_t p, long long n_time) {
   if (p->npix < 1 || p->ptap_time >= n_time) return EPIC_OK;
   cudaError_t e = cudaStreamSynchronize(p->stream);
   if (e != cudaSuccess) return cuda_fail(e, "stream sync before tap buffer growth");
-  e = p->d_ptap.alloc(static_cast<size_t>(n_time) * p->nc * p->npix);
+  const size_t per_t = static_cast<size_t>(p->nc) * p->npix;
+  e = grow(p, p->d_ptap, static_cast<size_t>(n_time) * per_t, SIZE_MAX);
   if (e != cudaSuccess) {
     p->ptap_time = 0;
     return fail(EPIC_ERR_OOM, "pixel tap buffer allocation failed");
   }
-  p->ptap_time = n_time;
+  p->ptap_time = static_cast<long long>(p->d_ptap.n / per_t);
   return EPIC_OK;
 }
 
@@ -865,7 +905,8 @@ epic_status image_wide(epic_plan_t p, const void* d_volt, long long n_time, doub
   if (p->d_ws.n < need) {
     cudaError_t e = cudaStreamSynchronize(p->stream);
     if (e != cudaSuccess) return cuda_fail(e, "stream sync before scratch growth");
-    if (p->d_ws.alloc(need) != cudaSuccess) return fail(EPIC_ERR_OOM, "unfused scratch allocation failed");
+    if (grow(p, p->d_ws, need, epic::wide_scratch(C, p->n, p->rs, p->workspace_budget)) != cudaSuccess)
+      return fail(EPIC_ERR_OOM, "unfused scratch allocation failed");
   }
   p->ws_time = static_cast<int>(std::max<long long>(1, nt * nc / C));   // samples of all channels the scratch holds
   epic::WideArgs w{};
@@ -916,12 +957,12 @@ epic_status image_unfused(epic_plan_t p, const void* d_volt, long long n_time, d
   if (p->ws_time < nt) {
     cudaError_t e = cudaStreamSynchronize(p->stream);
     if (e != cudaSuccess) return cuda_fail(e, "stream sync before scratch growth");
-    e = p->d_ws.alloc(per_t * static_cast<size_t>(nt));
+    e = grow(p, p->d_ws, per_t * static_cast<size_t>(nt), p->workspace_budget / sizeof(float2));
     if (e != cudaSuccess) {
       p->ws_time = 0;
       return fail(EPIC_ERR_OOM, "unfused scratch allocation failed");
     }
-    p->ws_time = static_cast<int>(nt);
+    p->ws_time = static_cast<int>(std::min<size_t>(p->d_ws.n / per_t, 1 << 20));
   }
   nt = std::min<long long>(nt, p->ws_time);
   epic::UnfusedArgs a{};
@@ -1751,6 +1792,7 @@ epic_status epic_plan_destroy(epic_plan_t p) {
   p->d_iters.release();
   if (p->graph_exec) cudaGraphExecDestroy(p->graph_exec);
   if (p->graph) cudaGraphDestroy(p->graph);
+  for (void* q : p->retired) cudaFree(q);
   delete p;
   return EPIC_OK;
 }
@@ -1809,6 +1851,7 @@ epic_status epic_image(epic_plan_t p, const void* d_volt, long long n_time, doub
   if (!d_volt || !d_image) return fail(EPIC_ERR_INVALID_ARG, "NULL device buffer");
   if (n_time < 1) return fail(EPIC_ERR_INVALID_ARG, "n_time must be >= 1");
   const size_t img_bytes = static_cast<size_t>(p->nc) * p->n * p->n * sizeof(double);
+  bind_captured(p);
   if (!accumulate) EPIC_CUDA(cudaMemsetAsync(d_image, 0, img_bytes, p->stream));
   if (p->precision != EPIC_PREC_FP32) return image_tc(p, d_volt, n_time, d_image);
   if (p->path == EPIC_PATH_CLUSTER) return image_cluster(p, d_volt, n_time, d_image);
@@ -1946,6 +1989,7 @@ epic_status epic_visibilities(epic_plan_t p, const void* d_volt, long long n_tim
   if (epic_status s = check_plan(p)) return s;
   if (!d_volt || !d_vis) return fail(EPIC_ERR_INVALID_ARG, "NULL device buffer");
   if (n_time < 1) return fail(EPIC_ERR_INVALID_ARG, "n_time must be >= 1");
+  bind_captured(p);
   const size_t nv = static_cast<size_t>(p->nc) * p->na * p->na;
   if (p->input == EPIC_IN_CI4) {
     // tensor cores: FP16 integers, exact; time in segments that keep the
@@ -1958,6 +2002,7 @@ epic_status epic_visibilities(epic_plan_t p, const void* d_volt, long long n_tim
     if (p->xe_tp < seg) {
       EPIC_CUDA(cudaStreamSynchronize(p->stream));
       if (p->xe_tp == 0) EPIC_CUDA(epic::xe_prepare());
+      drop(p, p->d_xe_z);
       if (p->d_xe_z.alloc(row_bytes / sizeof(uint16_t) * static_cast<size_t>(seg)) != cudaSuccess) {
         p->xe_tp = 0;
         return fail(EPIC_ERR_OOM, "X-engine operand scratch allocation failed");
@@ -2028,8 +2073,10 @@ epic_status epic_visibility_solve(epic_plan_t p, const double* d_vis, double* d_
     }
     DevBuf<double2> d_ph;
     DevBuf<double> d_flux;
-    cudaError_t es[] = {p->d_vm.alloc(nv), p->d_sw.alloc(np), p->d_sm2.alloc(np), p->d_uv.alloc(uv.size()), p->d_iters.alloc(C),
-                        d_ph.alloc(ph.size()), d_flux.alloc(flux.size())};
+    // the plan's buffers have one size for its life: a captured solve keeps them
+    const auto once = [](auto& b, size_t count) { return b.n == count ? cudaSuccess : b.alloc(count); };
+    cudaError_t es[] = {once(p->d_vm, nv), once(p->d_sw, np), once(p->d_sm2, np), once(p->d_uv, uv.size()),
+                        once(p->d_iters, C), d_ph.alloc(ph.size()), d_flux.alloc(flux.size())};
     for (cudaError_t x : es)
       if (x != cudaSuccess) return fail(EPIC_ERR_OOM, "model visibility allocation failed");
     EPIC_CUDA(cudaMemcpyAsync(d_ph.p, ph.data(), ph.size() * sizeof(double2), cudaMemcpyHostToDevice, p->stream));
@@ -2120,11 +2167,17 @@ epic_status epical_configure_pixels(epic_plan_t p, int n_pix, const double* pix_
   EPIC_CUDA(cudaStreamSynchronize(p->stream));
   for (size_t i = 0; i < n; ++i)
     for (int q = 0; q < n_pix; ++q) gd[i * n_pix + q] = g[i];
+  drop(p, p->d_ap);
+  drop(p, p->d_dp);
+  drop(p, p->d_kmp);
+  drop(p, p->d_gdir);
+  drop(p, p->d_ptab);
+  drop(p, p->d_pph);
   cudaError_t es[] = {p->d_ap.alloc(nap), p->d_dp.alloc(nap), p->d_kmp.alloc(n * n_pix),
                       p->d_gdir.alloc(n * n_pix), p->d_ptab.alloc(tab.size()), p->d_pph.alloc(pph.size())};
   for (cudaError_t x : es)
     if (x != cudaSuccess) return fail(EPIC_ERR_OOM, "multiple-pixel EPICal allocation failed");
-  p->d_ptap.release();
+  drop(p, p->d_ptap);
   p->ptap_time = 0;
   EPIC_CUDA(cudaMemcpyAsync(p->d_ap.p, ap.data(), nap * sizeof(double2), cudaMemcpyHostToDevice, p->stream));
   EPIC_CUDA(cudaMemcpyAsync(p->d_dp.p, dp.data(), nap * sizeof(double2), cudaMemcpyHostToDevice, p->stream));
@@ -2168,6 +2221,7 @@ epic_status epical_average_channels(epic_plan_t p, int c_lo, int c_hi) {
   if (epic_status s = check_plan(p)) return s;
   if (!(0 <= c_lo && c_lo < c_hi && c_hi <= p->nc))
     return fail(EPIC_ERR_INVALID_ARG, "channel band must satisfy 0 <= c_lo < c_hi <= C");
+  bind_captured(p);
   EPIC_CUDA(epic::launch_average_channels(p->na, c_lo, c_hi, p->d_flags.p, p->d_gain.p, p->d_wgain.p,
                                           p->d_phase.p, p->stream));
   return EPIC_OK;
@@ -2181,7 +2235,7 @@ epic_status epic_set_phase_centre(epic_plan_t p, double l0, double m0) {
   const size_t n = static_cast<size_t>(C) * Na;
   if (l0 == 0.0 && m0 == 0.0) {
     p->phase.clear();
-    p->d_phase.release();
+    drop(p, p->d_phase);
   } else {
     p->phase.resize(n);
     for (int c = 0; c < C; ++c)
@@ -2240,6 +2294,7 @@ epic_status epical_update(epic_plan_t p, double* d_gains_out, int* d_status) {
   if (epic_status s = check_plan(p)) return s;
   if (!p->cal) return fail(EPIC_ERR_STATE, "EPICal is not configured");
   if (p->frames < 1) return fail(EPIC_ERR_STATE, "no frames imaged since the last update");
+  bind_captured(p);
   if (p->npix > 0) {
     epic::MultiUpdateArgs m{};
     m.n_chan = p->nc;
@@ -2608,6 +2663,7 @@ epic_status epic_set_gains_device(epic_plan_t p, const double* d_gains) {
   const NvtxRange nvtx_range("epic_set_gains_device");
   if (epic_status s = check_plan(p)) return s;
   if (!d_gains) return fail(EPIC_ERR_INVALID_ARG, "d_gains is NULL");
+  bind_captured(p);
   EPIC_CUDA(epic::launch_set_gains(p->nc * p->na, reinterpret_cast<const double2*>(d_gains), p->d_gain.p,
                                    p->d_wgain.p, p->d_phase.p, p->stream));
   return EPIC_OK;
@@ -2619,6 +2675,7 @@ epic_status epic_image_backward(epic_plan_t p, const void* d_volt, long long n_t
   if (epic_status s = check_plan(p)) return s;
   if (!d_volt || !d_dl_di || !d_grad_g) return fail(EPIC_ERR_INVALID_ARG, "NULL device buffer");
   if (n_time < 1) return fail(EPIC_ERR_INVALID_ARG, "n_time must be >= 1");
+  bind_captured(p);
   if (p->path != EPIC_PATH_FUSED)
     return fail(EPIC_ERR_UNSUPPORTED, "the adjoint is built for the fused path (N <= 128)");
   const size_t n = static_cast<size_t>(p->nc) * p->na;
