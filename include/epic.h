@@ -417,8 +417,11 @@ epic_status epic_image_backward(epic_plan_t plan, const void* d_volt, long long 
  * pairs (gridding sums, degridding sums, the conj(E_a) products and the
  * accumulation stay FP32, the gradient sums FP64).  The BF16 gradient
  * carries the rounding of 8-bit significands through about 4 log2(N)
- * butterfly levels (a relative error of order 10^-2).  Host only; applies
- * to later calls.  Errors: INVALID_ARG (another precision). */
+ * butterfly levels (a relative error of order 10^-2).  With BF16 set,
+ * epic_image of a fused plan also takes the kernel that images one frame per
+ * FP32 value (except in the multiple-pixel form): the frame-pair kernel's
+ * image differs in its last digits, and the BF16 rounding of dL/dI makes 2e-5
+ * of that in the gradient.  Host only; applies to later calls.  Errors: INVALID_ARG (another precision). */
 epic_status epic_plan_set_adjoint_precision(epic_plan_t plan, int precision);
 
 /* Debug/test accessors (synchronous, host outputs). */

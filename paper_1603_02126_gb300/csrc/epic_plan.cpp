@@ -182,7 +182,7 @@ struct epic_plan_s {
 
   // differentiation form
   DevBuf<double2> d_dldw;       // [C][Na] dL/dconj(w) accumulator
-  // one-frame fused kernel of a frame-pair plan with BF16 gradients
+  // one-frame fused kernel of a frame-pair plan (calls with BF16 gradients)
   bool one_ready = false;
   int one_steps = 1, one_gsmem = 0, one_ctas = 0;
   size_t one_smem = 0;
@@ -451,10 +451,11 @@ epic_status build_gather(epic_plan_t p, const std::vector<float>& wts, int N1, b
   cnt.assign(static_cast<size_t>(C) * RA * N1 * CW, make_uint4(0, 0, 0, 0));
   base.assign(static_cast<size_t>(C) + 1, 0);
   ent.clear();
-  std::vector<std::vector<std::pair<int, float>>> bucket(static_cast<size_t>(RA) * N1 * N2);
-  for (int c = 0; c < C; ++c) {
-    base[c] = static_cast<int>(ent.size());
-    for (auto& l : bucket) l.clear();
+  // per channel a counting sort of the taps by (lane, j): antennas in order
+  // inside a group
+  const size_t groups = static_cast<size_t>(RA) * N1 * N2;
+  std::vector<int> at(groups + 1);
+  const auto each_tap = [&](int c, auto&& f) {
     for (int a = 0; a < Na; ++a) {
       if (p->flags[a]) continue;
       const size_t ob = (static_cast<size_t>(c) * Na + a) * 2;
@@ -463,28 +464,34 @@ epic_status build_gather(epic_plan_t p, const std::vector<float>& wts, int N1, b
       const float* wf = &wts[(static_cast<size_t>(c) * Na + a) * KK];
       for (int dy = 0; dy < K; ++dy)
         for (int dx = 0; dx < K; ++dx) {
-          const float w = wf[dy * K + dx];
-          if (w == 0.0f) continue;
           const int x = xa + dx;
-          bucket[(static_cast<size_t>(r0 + dy) * N1 + x % N1) * N2 + x / N1].emplace_back(a, w);
+          if (wf[dy * K + dx] != 0.0f) f((static_cast<size_t>(r0 + dy) * N1 + x % N1) * N2 + x / N1, a, wf[dy * K + dx]);
         }
     }
+  };
+  for (int c = 0; c < C; ++c) {
+    base[c] = static_cast<int>(ent.size());
+    std::fill(at.begin(), at.end(), 0);
+    each_tap(c, [&](size_t g, int, float) { ++at[g + 1]; });
     for (int li = 0; li < RA * N1; ++li) {
-      ofs[static_cast<size_t>(c) * RA * N1 + li] = static_cast<int>(ent.size()) - base[c];
       unsigned char cb[32] = {0};
       for (int j = 0; j < N2; ++j) {
-        const auto& l = bucket[static_cast<size_t>(li) * N2 + j];
-        if (l.size() > 255) return fail(EPIC_ERR_UNSUPPORTED, "more than 255 gridding taps on one grid cell");
-        cb[j] = static_cast<unsigned char>(l.size());
-        for (const auto& en : l) {
-          uint2 q;
-          q.x = static_cast<unsigned>(en.first);
-          std::memcpy(&q.y, &en.second, sizeof(float));
-          ent.push_back(q);
-        }
+        const int n = at[static_cast<size_t>(li) * N2 + j + 1];
+        if (n > 255) return fail(EPIC_ERR_UNSUPPORTED, "more than 255 gridding taps on one grid cell");
+        cb[j] = static_cast<unsigned char>(n);
       }
       std::memcpy(&cnt[(static_cast<size_t>(c) * RA * N1 + li) * CW], cb, sizeof(uint4) * CW);
     }
+    for (size_t g = 0; g < groups; ++g) at[g + 1] += at[g];
+    for (int li = 0; li < RA * N1; ++li)
+      ofs[static_cast<size_t>(c) * RA * N1 + li] = at[static_cast<size_t>(li) * N2];
+    ent.resize(ent.size() + at[groups]);
+    uint2* e = ent.data() + base[c];
+    each_tap(c, [&](size_t g, int a, float w) {
+      uint2& q = e[at[g]++];
+      q.x = static_cast<unsigned>(a);
+      std::memcpy(&q.y, &w, sizeof(float));
+    });
   }
   base[C] = static_cast<int>(ent.size());
   return EPIC_OK;
@@ -803,37 +810,12 @@ bool pair_adjoint(const epic_plan_s* p, epic::ImageArgs* q) {
     smem = epic::pair_smem_bytes(p->n, p->na, p->rows_alloc, p->gs, 0, 0, true);
   }
   if (smem > static_cast<size_t>(most)) return false;
-  if (q) {
-    q->rs = epic::pair_rs(p->n, p->rows_alloc, true);
-    q->smem = smem;
-    q->gsmem = p->gsmem && slices > 0 ? 1 : 0;
-    q->max_slices = slices;
-    q->max_ent = ent;
-  }
+  q->rs = epic::pair_rs(p->n, p->rows_alloc, true);
+  q->smem = smem;
+  q->gsmem = p->gsmem && slices > 0 ? 1 : 0;
+  q->max_slices = slices;
+  q->max_ent = ent;
   return true;
-}
-
-// Absolute-column gather tables of the one-frame adjoint kernels (FP32 where
-// the frame-pair form does not fit, and BF16), once per plan.
-epic_status ensure_adjoint_tables(epic_plan_s* p, const std::vector<float>& wts) {
-  if (p->d_ugofs.p) return EPIC_OK;
-  std::vector<int> ofs, base;
-  std::vector<uint4> cnt;
-  std::vector<uint2> ent;
-  if (epic_status st = build_gather(p, wts, epic::image_fft_lanes(p->n), false, ofs, cnt, ent, base)) return st;
-  cudaError_t es[] = {p->d_ugcnt.alloc(cnt.size()), p->d_ugent.alloc(ent.size()), p->d_ugbase.alloc(base.size()),
-                      p->d_ugofs.alloc(ofs.size())};
-  for (cudaError_t e : es)
-    if (e != cudaSuccess) {
-      p->d_ugofs.release();
-      return e == cudaErrorMemoryAllocation ? fail(EPIC_ERR_OOM, "device allocation failed")
-                                            : cuda_fail(e, "table upload");
-    }
-  EPIC_CUDA(cudaMemcpy(p->d_ugofs.p, ofs.data(), ofs.size() * sizeof(int), cudaMemcpyHostToDevice));
-  EPIC_CUDA(cudaMemcpy(p->d_ugcnt.p, cnt.data(), cnt.size() * sizeof(uint4), cudaMemcpyHostToDevice));
-  EPIC_CUDA(cudaMemcpy(p->d_ugent.p, ent.data(), ent.size() * sizeof(uint2), cudaMemcpyHostToDevice));
-  EPIC_CUDA(cudaMemcpy(p->d_ugbase.p, base.data(), base.size() * sizeof(int), cudaMemcpyHostToDevice));
-  return EPIC_OK;
 }
 
 // Cluster path: one persistent launch of thread-block clusters.
@@ -1385,33 +1367,6 @@ void hold_wide_scratch(epic_plan_s* p, WideTables* wide) {
   *wide = WideTables();
 }
 
-// The one-frame fused kernel's tables and launch shape of a frame-pair plan.
-epic_status ensure_one_frame(epic_plan_s* p) {
-  int most = 0, per_sm = 0;
-  EPIC_CUDA(cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device));
-  if (!one_frame_shape(p, most, &p->one_steps, &p->one_gsmem, &p->one_smem)) return EPIC_OK;
-  EPIC_CUDA(epic::image_kernel_prepare(p->n, p->one_smem, p->na, p->one_steps, &per_sm));
-  if (per_sm < 1) return EPIC_OK;
-  std::vector<float> wts(p->w64.size(), 0.0f);
-  fold_weights(p, wts);
-  std::vector<int> ofs, base;
-  std::vector<uint4> cnt;
-  std::vector<uint2> ent;
-  if (epic_status st = build_gather(p, wts, epic::image_fft_lanes(p->n), true, ofs, cnt, ent, base)) return st;
-  cudaError_t es[] = {p->d_gofs.alloc(ofs.size()), p->d_gcnt.alloc(cnt.size()), p->d_gent.alloc(ent.size()),
-                      p->d_gbase.alloc(base.size())};
-  for (cudaError_t e : es)
-    if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? fail(EPIC_ERR_OOM, "device allocation failed")
-                                                                : cuda_fail(e, "table upload");
-  EPIC_CUDA(cudaMemcpy(p->d_gofs.p, ofs.data(), ofs.size() * sizeof(int), cudaMemcpyHostToDevice));
-  EPIC_CUDA(cudaMemcpy(p->d_gcnt.p, cnt.data(), cnt.size() * sizeof(uint4), cudaMemcpyHostToDevice));
-  EPIC_CUDA(cudaMemcpy(p->d_gent.p, ent.data(), ent.size() * sizeof(uint2), cudaMemcpyHostToDevice));
-  EPIC_CUDA(cudaMemcpy(p->d_gbase.p, base.data(), base.size() * sizeof(int), cudaMemcpyHostToDevice));
-  p->one_ctas = per_sm * p->sms;
-  p->one_ready = true;
-  return EPIC_OK;
-}
-
 // Launch shape and path of the plan: the tensor-core form's K extent for
 // FP16/BF16, else the fused kernel's frames per step and gather-table
 // placement (or the warp-specialised form), the cluster form when asked
@@ -1534,6 +1489,13 @@ epic_status choose_path(epic_plan_s* p, const epic_plan_desc* d, bool fused_shap
                               : fail(EPIC_ERR_UNSUPPORTED, "image kernel cannot be resident");
     p->ctas = per_sm * p->sms;
     p->path = EPIC_PATH_FUSED;
+    // a frame-pair plan's one-frame kernel
+    if (p->pair && one_frame_shape(p, smem_optin, &p->one_steps, &p->one_gsmem, &p->one_smem)) {
+      e = epic::image_kernel_prepare(N, p->one_smem, Na, p->one_steps, &per_sm);
+      if (e != cudaSuccess) return cuda_fail(e, "image kernel attributes");
+      p->one_ready = per_sm > 0;
+      p->one_ctas = per_sm * p->sms;
+    }
     // footprints that leave no room for two frames on one SM: the spectra of
     // a pair through HBM (N = 128); multiple-pixel EPICal and
     // epic_image_host_static stay with the one-frame kernel
@@ -1660,13 +1622,14 @@ epic_status epic_plan_create(epic_plan_t* out, const epic_plan_desc* d) {
       const int bx = p->base[ob], by = p->base[ob + 1];
       cellf[static_cast<size_t>(c) * Na + a] = (by - h - p->y0[c]) * ws + (bx - h - p->x0[c]);
     }
-  // gridding gather tables (see build_gather): the fused kernel, the plain
-  // unfused path use window columns, the one-frame adjoint absolute columns
-  // (ensure_adjoint_tables)
-  std::vector<int> gofs, gbase;
-  std::vector<uint4> gcnt;
-  std::vector<uint2> gent;
-  if (p->path == EPIC_PATH_FUSED ? !p->pair
+  // gridding gather tables (see build_gather): the one-frame fused kernel and
+  // the plain unfused path use window columns, the fused path's one-frame
+  // adjoint kernels absolute columns.  Built for frame-pair plans too, so that
+  // epic_plan_set_adjoint_precision stays on the host.
+  std::vector<int> gofs, gbase, ugofs, ugbase;
+  std::vector<uint4> gcnt, ugcnt;
+  std::vector<uint2> gent, ugent;
+  if (p->path == EPIC_PATH_FUSED ? !p->pair || p->one_ready
                                  : (p->path == EPIC_PATH_UNFUSED && !p->wide && p->precision == EPIC_PREC_FP32)) {
     const int n1 = p->path == EPIC_PATH_FUSED ? epic::image_fft_lanes(N) : epic::unfused_fft_lanes(N);
     if (epic_status st = build_gather(p, wts, n1, true, gofs, gcnt, gent, gbase)) {
@@ -1675,6 +1638,11 @@ epic_status epic_plan_create(epic_plan_t* out, const epic_plan_desc* d) {
     }
     for (int c = 0; c < C; ++c) p->gmax = std::max(p->gmax, gbase[c + 1] - gbase[c]);
   }
+  if (fused)
+    if (epic_status st = build_gather(p, wts, epic::image_fft_lanes(N), false, ugofs, ugcnt, ugent, ugbase)) {
+      epic_plan_destroy(p);
+      return st;
+    }
   std::vector<float2> pixph(C, make_float2(1.0f, 0.0f));
   std::vector<int> rowcol, order;
   std::vector<int2> ranges;
@@ -1693,6 +1661,8 @@ epic_status epic_plan_create(epic_plan_t* out, const epic_plan_desc* d) {
                       up(p->d_cellf, cellf), up(p->d_pixph, pixph), up(p->d_rowcol, rowcol),
                       up(p->d_order, order), up(p->d_ranges, ranges), up(p->d_gofs, gofs),
                       up(p->d_gent, gent), up(p->d_gbase, gbase), up(p->d_gcnt, gcnt),
+                      up(p->d_ugofs, ugofs), up(p->d_ugcnt, ugcnt), up(p->d_ugent, ugent),
+                      up(p->d_ugbase, ugbase),
                       up(p->d_pcell, cells.cell), up(p->d_pslice, cells.slice),
                       up(p->d_pent, cells.ent), up(p->d_psbase, cells.sbase), up(p->d_pebase, cells.ebase),
                       up(p->d_pcost, cells.cost), up(p->d_wlists, wide.lists), up(p->d_wat, wide.at),
@@ -1713,11 +1683,6 @@ epic_status epic_plan_create(epic_plan_t* out, const epic_plan_desc* d) {
     epic_plan_destroy(p);
     return cuda_fail(e, "counter");
   }
-  if (p->path == EPIC_PATH_FUSED && !pair_adjoint(p, nullptr))
-    if (epic_status st = ensure_adjoint_tables(p, wts)) {
-      epic_plan_destroy(p);
-      return st;
-    }
   *out = p;
   return EPIC_OK;
 }
@@ -2355,13 +2320,6 @@ epic_status epic_plan_set_adjoint_precision(epic_plan_t p, int precision) {
   if (epic_status s = check_plan(p)) return s;
   if (precision != EPIC_PREC_FP32 && precision != EPIC_PREC_BF16)
     return fail(EPIC_ERR_INVALID_ARG, "adjoint precision must be EPIC_PREC_FP32 or EPIC_PREC_BF16");
-  if (precision == EPIC_PREC_BF16 && p->path == EPIC_PATH_FUSED && !p->d_ugofs.p) {
-    std::vector<float> wts(p->w64.size(), 0.0f);
-    fold_weights(p, wts);
-    if (epic_status st = ensure_adjoint_tables(p, wts)) return st;
-  }
-  if (precision == EPIC_PREC_BF16 && p->pair && !p->one_ready)
-    if (epic_status st = ensure_one_frame(p)) return st;
   p->adjoint_precision = precision;
   return EPIC_OK;
 }
