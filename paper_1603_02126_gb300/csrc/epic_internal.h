@@ -321,6 +321,7 @@ struct WideArgs {
   const int* row_cost;     // [C + 1] prefix sums of the row kernel's cost per pair
   const int* col_cost;     // [C + 1] prefix sums of the column kernel's cost per pair and block
   int rows_ctas, cols_ctas;
+  int rows_grid;           // CTAs of this row launch
 };
 bool wide_supported(int n);
 int wide_row_block(int n);   // grid rows per block of lists

@@ -139,6 +139,7 @@ struct epic_plan_s {
   DevBuf<int2> d_pslice;        // (first entry, taps) of each slice
   DevBuf<uint2> d_pent;         // entries (byte offset of E'_a, weight bits)
   DevBuf<int> d_psbase, d_pebase, d_pcost;   // [C + 1] first slice / first entry / cost prefix
+  DevBuf<int> d_peven;          // [C + 1] 0, 1, .. C: equal costs
   DevBuf<float2> d_pixph;       // [C] calibrator-pixel phase in window coordinates
   std::vector<int> x0, cols;    // [C] first occupied column, occupied columns
   int rs_fused = 0;
@@ -168,6 +169,8 @@ struct epic_plan_s {
   DevBuf<unsigned char> d_wlists;   // row blocks' tap lists
   DevBuf<int2> d_wat;               // [C][nb_max] (offset, bytes) / 16 of each block's lists
   DevBuf<int> d_wrcost, d_wccost;   // [C + 1] cost prefixes of the row and column kernels
+  DevBuf<int> d_wblocks;            // [C + 1] first row block of each channel
+  std::vector<int> w_blocks;        // the same on the host
   int w_nb_max = 0, w_max_lists = 0, w_gs = 0, w_rows_ctas = 0, w_cols_ctas = 0;
 
   // host-API staging
@@ -666,7 +669,7 @@ epic_status build_cells(const epic_plan_s* p, const std::vector<float>& wts, int
 struct WideTables {
   std::vector<unsigned char> lists;
   std::vector<int2> at;          // [C][nb_max] (offset, bytes) / 16
-  std::vector<int> row_cost, col_cost;
+  std::vector<int> row_cost, col_cost, blocks;
   int nb_max = 0, max_lists = 0;
 };
 
@@ -710,25 +713,29 @@ epic_status build_wide_lists(const epic_plan_s* p, const std::vector<float>& wts
     // gridding, and the row transforms where the same kernel runs them
     long long rows = 10 * listed + 20LL * p->na;
     if (p->precision == EPIC_PREC_FP32) rows += static_cast<long long>(R) * (N / 32) * task_cost(32, p->cols[c]);
+    t->blocks.push_back(static_cast<int>(taps.size()));
     t->row_cost.push_back(static_cast<int>(std::max<long long>(1, rows / 256)));
     t->col_cost.push_back(static_cast<int>(task_cost(32, R)));
   }
   t->max_lists = (t->max_lists + 127) & ~127;
+  prefix_sums(&t->blocks);
   prefix_sums(&t->row_cost);
   prefix_sums(&t->col_cost);
   return EPIC_OK;
 }
 
-// Whether fused calls take the frame-pair kernel.  A plan with BF16 gradients
-// keeps the one-frame kernel: the BF16 rounding of dL/dI turns a last-digit
-// difference of the image into one of 2e-5 and more of the gradient.
-bool uses_pair(const epic_plan_s* p) {
-  return p->pair && !(p->adjoint_precision == EPIC_PREC_BF16 && p->one_ready && !(p->cal && p->npix > 0));
+// Whether an image call of a fused plan takes the frame-pair forms.  A plan
+// with BF16 gradients keeps the one-frame kernel: the BF16 rounding of dL/dI
+// turns a last-digit difference of the image into one of 2e-5 and more of the
+// gradient.
+bool pair_call(const epic_plan_s* p, long long n_time) {
+  const bool one = p->adjoint_precision == EPIC_PREC_BF16;
+  return !one || (p->cal && p->npix > 0) || (p->pair && !p->one_ready);
 }
 
 // Arguments of one fused launch over a device batch.
 epic::ImageArgs fused_args(epic_plan_t p, const void* d_volt, long long n_time, double* d_image,
-                           double img_scale) {
+                           double img_scale, bool pair) {
   epic::ImageArgs a{};
   a.volt = d_volt;
   a.input_fmt = p->input;
@@ -769,7 +776,7 @@ epic::ImageArgs fused_args(epic_plan_t p, const void* d_volt, long long n_time, 
   a.smem = p->smem;
   a.npix = 0;                              // epic_image arms the pixel taps itself
   a.wait_limit = p->wait_limit;
-  if (uses_pair(p)) {
+  if (pair) {
     a.pair = 1;
     a.pcell = p->d_pcell.p;
     a.pslice = p->d_pslice.p;
@@ -788,6 +795,10 @@ epic::ImageArgs fused_args(epic_plan_t p, const void* d_volt, long long n_time, 
     // 1000 56)
     const long long pairs = static_cast<long long>(p->nc) * ((n_time + 1) / 2);
     a.grid = static_cast<int>(std::max<long long>(1, std::min<long long>({pairs / p->tune_pairs, p->ctas, 256LL * p->nc})));
+    // one pair per CTA: equal costs, or shares by the channels' costs would
+    // give some CTAs two pairs and others none (64 channels, 200 antennas,
+    // 32 x 32, 4 samples: 24.8 against 17.5 us)
+    if (a.grid == pairs) a.pcost = p->d_peven.p;
   } else if (p->pair) {
     a.gsmem = p->one_gsmem;
     a.steps = p->one_steps;
@@ -917,6 +928,10 @@ epic_status image_wide(epic_plan_t p, const void* d_volt, long long n_time, doub
     for (int c0 = 0; c0 < C; c0 += nc) {
       w.c0 = c0;
       w.nc = std::min(nc, C - c0);
+      // one row block per CTA of a short call: equal costs
+      const long long blocks = static_cast<long long>(p->w_blocks[c0 + w.nc] - p->w_blocks[c0]) * ((n + 1) / 2);
+      w.row_cost = blocks <= w.rows_ctas ? p->d_wblocks.p : p->d_wrcost.p;
+      w.rows_grid = static_cast<int>(std::min<long long>(blocks, w.rows_ctas));
       EPIC_CUDA(epic::launch_wide_batch(w, t0, n, p->stream));
     }
     if (p->cal) EPIC_CUDA(epic::launch_correlate(a, t0, n, p->stream));
@@ -1353,8 +1368,7 @@ epic_status plan_wide(epic_plan_s* p, const std::vector<float>& wts, WideTables*
 // captured graph binds stays where it is.  At most the default budget, less
 // where the device has less; without room for a pair the plan keeps the
 // one-frame kernel.
-void hold_wide_scratch(epic_plan_s* p, WideTables* wide) {
-  if (!p->wide) return;
+void hold_wide_scratch(epic_plan_s* p) {
   const size_t pair_bytes = 2 * static_cast<size_t>(p->n) * p->rs * sizeof(float2);
   for (size_t budget = std::min(p->workspace_budget, kDefaultWorkspace); budget >= pair_bytes; budget /= 2) {
     if (p->d_ws.alloc(epic::wide_scratch(p->nc, p->n, p->rs, budget)) == cudaSuccess) {
@@ -1364,7 +1378,6 @@ void hold_wide_scratch(epic_plan_s* p, WideTables* wide) {
     cudaGetLastError();
   }
   p->wide = false;
-  *wide = WideTables();
 }
 
 // Launch shape and path of the plan: the tensor-core form's K extent for
@@ -1501,7 +1514,8 @@ epic_status choose_path(epic_plan_s* p, const epic_plan_desc* d, bool fused_shap
     // epic_image_host_static stay with the one-frame kernel
     if (!p->pair && !p->piped) {
       if (epic_status st = plan_wide(p, wts, wide)) return st;
-      hold_wide_scratch(p, wide);
+      if (p->wide) hold_wide_scratch(p);
+      if (!p->wide) *wide = WideTables();
     }
   } else {
     p->smem = 0;
@@ -1647,6 +1661,9 @@ epic_status epic_plan_create(epic_plan_t* out, const epic_plan_desc* d) {
   std::vector<int> rowcol, order;
   std::vector<int2> ranges;
   if (p->path == EPIC_PATH_CLUSTER) build_cluster_tables(p, rowcol, order, ranges);
+  std::vector<int> even;
+  for (int c = 0; p->pair && c <= C; ++c) even.push_back(c);
+  p->w_blocks = wide.blocks;
   std::vector<double2> gain(static_cast<size_t>(C) * Na, make_double2(1.0, 0.0));
   std::vector<float2> wgain(static_cast<size_t>(C) * Na, make_float2(1.0f, 0.0f));
 
@@ -1665,7 +1682,8 @@ epic_status epic_plan_create(epic_plan_t* out, const epic_plan_desc* d) {
                       up(p->d_ugbase, ugbase),
                       up(p->d_pcell, cells.cell), up(p->d_pslice, cells.slice),
                       up(p->d_pent, cells.ent), up(p->d_psbase, cells.sbase), up(p->d_pebase, cells.ebase),
-                      up(p->d_pcost, cells.cost), up(p->d_wlists, wide.lists), up(p->d_wat, wide.at),
+                      up(p->d_pcost, cells.cost), up(p->d_peven, even), up(p->d_wblocks, wide.blocks),
+                      up(p->d_wlists, wide.lists), up(p->d_wat, wide.at),
                       up(p->d_wrcost, wide.row_cost), up(p->d_wccost, wide.col_cost)};
   for (cudaError_t x : es)
     if (x != cudaSuccess) {
@@ -1748,6 +1766,8 @@ epic_status epic_plan_destroy(epic_plan_t p) {
   p->d_psbase.release();
   p->d_pebase.release();
   p->d_pcost.release();
+  p->d_peven.release();
+  p->d_wblocks.release();
   p->d_wlists.release();
   p->d_wat.release();
   p->d_wrcost.release();
@@ -1821,9 +1841,10 @@ epic_status epic_image(epic_plan_t p, const void* d_volt, long long n_time, doub
   if (p->precision != EPIC_PREC_FP32) return image_tc(p, d_volt, n_time, d_image);
   if (p->path == EPIC_PATH_CLUSTER) return image_cluster(p, d_volt, n_time, d_image);
   if (p->path == EPIC_PATH_UNFUSED) return image_unfused(p, d_volt, n_time, d_image);
-  if (p->wide && p->adjoint_precision != EPIC_PREC_BF16 && !(p->cal && p->npix > 0))
+  const bool pair = pair_call(p, n_time);
+  if (p->wide && pair && !(p->cal && p->npix > 0))
     return image_wide(p, d_volt, n_time, d_image);
-  epic::ImageArgs a = fused_args(p, d_volt, n_time, d_image, 1.0 / static_cast<double>(n_time));
+  epic::ImageArgs a = fused_args(p, d_volt, n_time, d_image, 1.0 / static_cast<double>(n_time), p->pair && pair);
   if (p->cal && p->npix > 0) {
     if (epic_status st = ensure_ptap(p, n_time)) return st;
     a.npix = p->npix;
@@ -2472,7 +2493,7 @@ epic_status epic_autotune(epic_plan_t p, const void* d_volt, long long n_time, d
   epic_status st = EPIC_OK;
   const int reps = 3;
   if (p->path == EPIC_PATH_FUSED) {
-    int& knob = uses_pair(p) ? p->tune_pairs : p->tune_units;
+    int& knob = p->pair && pair_call(p, n_time) ? p->tune_pairs : p->tune_units;
     const int def = knob;
     st = time_image(p, d_volt, n_time, d_image, reps, &r.ms_default);
     best = r.ms_default;
@@ -2642,8 +2663,10 @@ epic_status epic_image_backward(epic_plan_t p, const void* d_volt, long long n_t
     if (e != cudaSuccess) return fail(EPIC_ERR_OOM, "gradient scratch allocation failed");
   }
   EPIC_CUDA(cudaMemsetAsync(p->d_dldw.p, 0, n * sizeof(double2), p->stream));
-  if (p->pair && p->adjoint_precision == EPIC_PREC_FP32) {
-    epic::ImageArgs q = fused_args(p, d_volt, n_time, nullptr, 1.0 / static_cast<double>(n_time));
+  const bool bf16 = p->adjoint_precision == EPIC_PREC_BF16;
+  const size_t one_smem = epic::adjoint_smem_bytes(p->n, p->rows_alloc, p->rs, p->na, bf16);
+  if (p->pair && !bf16) {
+    epic::ImageArgs q = fused_args(p, d_volt, n_time, nullptr, 1.0 / static_cast<double>(n_time), true);
     if (pair_adjoint(p, &q)) {
       EPIC_CUDA(epic::launch_adjoint_pair(p->n, q, d_dl_di, p->d_dldw.p, p->stream));
       EPIC_CUDA(epic::launch_adjoint_finalize(p->nc, p->na, p->d_dldw.p, p->d_gain.p, p->d_phase.p, p->d_flags.p,
@@ -2667,8 +2690,7 @@ epic_status epic_image_backward(epic_plan_t p, const void* d_volt, long long n_t
   a.dldi = d_dl_di;
   a.dldw = p->d_dldw.p;
   a.img_scale = 1.0 / static_cast<double>(n_time);
-  const bool bf16 = p->adjoint_precision == EPIC_PREC_BF16;
-  a.smem = epic::adjoint_smem_bytes(p->n, p->rows_alloc, p->rs, p->na, bf16);
+  a.smem = one_smem;
   const int ctas = !p->pair ? p->ctas : p->one_ctas ? p->one_ctas : p->sms;
   a.segs = choose_segments(p->nc, n_time, ctas, p->tune_units);
   a.rows_alloc = p->rows_alloc;
@@ -2711,7 +2733,7 @@ int image_batch_scaled(epic_plan_s* p, const void* d_volt, long long n_time, dou
     return fail(EPIC_ERR_UNSUPPORTED, "this call needs a plan on the fused path");
   if (p->cal && p->npix > 0)
     return fail(EPIC_ERR_UNSUPPORTED, "multiple-pixel EPICal needs its tap buffer (plan scratch)");
-  const ImageArgs a = fused_args(p, d_volt, n_time, d_image, img_scale);
+  const ImageArgs a = fused_args(p, d_volt, n_time, d_image, img_scale, p->pair && pair_call(p, n_time));
   cudaError_t e = launch_image(p->n, a, p->stream);
   if (e != cudaSuccess) return cuda_fail(e, "image launch");
   if (p->cal) p->frames += n_time;

@@ -325,9 +325,8 @@ cudaError_t prepare_n(const WideArgs& w, int fmt, int* rows_per_sm, int* cols_pe
 template <int N>
 cudaError_t launch_n(const WideArgs& w, long long t0, int nt, cudaStream_t s) {
   const long long pairs = static_cast<long long>((nt + 1) / 2) * w.nc;
-  const long long rg = pairs * w.nb_max < w.rows_ctas ? pairs * w.nb_max : w.rows_ctas;
-  if (w.u.input_fmt) wide_rows_kernel<N, 1><<<static_cast<unsigned>(rg), kWBT, rows_smem<N>(w), s>>>(w, t0, nt);
-  else wide_rows_kernel<N, 0><<<static_cast<unsigned>(rg), kWBT, rows_smem<N>(w), s>>>(w, t0, nt);
+  if (w.u.input_fmt) wide_rows_kernel<N, 1><<<w.rows_grid, kWBT, rows_smem<N>(w), s>>>(w, t0, nt);
+  else wide_rows_kernel<N, 0><<<w.rows_grid, kWBT, rows_smem<N>(w), s>>>(w, t0, nt);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const long long cu = pairs * WGeo<N>::CB;
