@@ -724,12 +724,20 @@ epic_status build_wide_lists(const epic_plan_s* p, const std::vector<float>& wts
   return EPIC_OK;
 }
 
+// Samples of a call up to which one frame per FP32 value is the faster form:
+// half of a single sample's pair is empty, and a pair has more latency than
+// two frames on small grids (one-frame against frame-pair, us: one sample of
+// 256 antennas, 64 channels, 128 x 128 24.8 and 28.9, of 248, 64 x 64, 14.5
+// and 18.6; two samples 31.0 and 28.9, 16.6 and 18.6; 12 antennas, 16 x 16, two
+// samples 8.4 and 10.3, three samples of 64 channels 12.4 and 14.5).
+long long one_frame_samples(int n) { return n <= 16 ? 3 : n <= 64 ? 2 : 1; }
+
 // Whether an image call of a fused plan takes the frame-pair forms.  A plan
 // with BF16 gradients keeps the one-frame kernel: the BF16 rounding of dL/dI
 // turns a last-digit difference of the image into one of 2e-5 and more of the
 // gradient.
 bool pair_call(const epic_plan_s* p, long long n_time) {
-  const bool one = p->adjoint_precision == EPIC_PREC_BF16;
+  const bool one = p->adjoint_precision == EPIC_PREC_BF16 || n_time <= one_frame_samples(p->n);
   return !one || (p->cal && p->npix > 0) || (p->pair && !p->one_ready);
 }
 
@@ -2665,7 +2673,13 @@ epic_status epic_image_backward(epic_plan_t p, const void* d_volt, long long n_t
   EPIC_CUDA(cudaMemsetAsync(p->d_dldw.p, 0, n * sizeof(double2), p->stream));
   const bool bf16 = p->adjoint_precision == EPIC_PREC_BF16;
   const size_t one_smem = epic::adjoint_smem_bytes(p->n, p->rows_alloc, p->rs, p->na, bf16);
-  if (p->pair && !bf16) {
+  int most = 0;
+  EPIC_CUDA(cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device));
+  // one sample fills half a pair: 32.8 against 41.0 us for 256 antennas,
+  // 128 x 128, 21.0 against 24.6 for 248, 64 x 64 (two samples 45.6 against
+  // 41.1, 27.3 against 24.7)
+  const bool one = n_time == 1 && one_smem <= static_cast<size_t>(most);
+  if (p->pair && !bf16 && !one) {
     epic::ImageArgs q = fused_args(p, d_volt, n_time, nullptr, 1.0 / static_cast<double>(n_time), true);
     if (pair_adjoint(p, &q)) {
       EPIC_CUDA(epic::launch_adjoint_pair(p->n, q, d_dl_di, p->d_dldw.p, p->stream));
