@@ -1371,6 +1371,18 @@ epic_status plan_wide(epic_plan_s* p, const std::vector<float>& wts, WideTables*
   return EPIC_OK;
 }
 
+// Whether a fused plan (N = 128) images faster in its wide form than frame by
+// frame on one SM.  The wide transforms cost more the more rows they sum,
+// and the row kernel loses half its warps where the antennas and a block's
+// lists leave room for one CTA per SM.  Time of the one-frame kernel over
+// the wide form's, 1000 samples of 16 channels: 99 rows 1.11 at 100 antennas,
+// 1.27 at 512, 1.11 at 900 (one CTA); 113 rows 1.00 at 100, 1.17 at 250, 1.23
+// at 512, 0.97 at 700 and 1.00 at 900 (one CTA); 127 rows 0.89 at 100, 1.05 at
+// 250, 0.84 at 512 and 0.89 at 900 (one CTA).
+bool wide_pays(const epic_plan_s* p) {
+  return p->rows_alloc <= 108 || (p->na >= 200 && p->w_rows_ctas >= 2 * p->sms);
+}
+
 // Scratch of a fused plan in its wide form, once, for calls of any length:
 // epic_image of a fused plan allocates nothing and does not wait, and what a
 // captured graph binds stays where it is.  At most the default budget, less
@@ -1522,6 +1534,7 @@ epic_status choose_path(epic_plan_s* p, const epic_plan_desc* d, bool fused_shap
     // epic_image_host_static stay with the one-frame kernel
     if (!p->pair && !p->piped) {
       if (epic_status st = plan_wide(p, wts, wide)) return st;
+      if (!wide_pays(p)) p->wide = false;
       if (p->wide) hold_wide_scratch(p);
       if (!p->wide) *wide = WideTables();
     }

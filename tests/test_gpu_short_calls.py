@@ -1,7 +1,8 @@
 """Calls of one to four samples, where the plan chooses between the one-frame
-and the frame-pair kernels and gives each CTA one pair, against the FP64
-oracle: image relative L2 <= 1e-5, gains and gradient <= 1e-4 (the bounds of
-the plain path)."""
+and the frame-pair kernels and gives each CTA one pair, and footprints on
+both sides of the line between the one-frame kernel and the wide form
+(N = 128), against the FP64 oracle: image relative L2 <= 1e-5, gains and
+gradient <= 1e-4 (the bounds of the plain path)."""
 import numpy as np
 import pytest
 
@@ -71,3 +72,15 @@ def test_gradient(n, na, rows, T, C, fmt):
     grad = p.image_backward(dev, dl).cpu().numpy()
     ref = O.chi2_gradient(oplan, E, g, M)
     assert np.linalg.norm(grad - ref) / np.linalg.norm(ref) <= 1e-4
+
+
+@pytest.mark.parametrize("na,rows,wide", [(100, 107, True), (100, 109, False), (250, 113, True), (700, 113, False)])
+def test_form_by_footprint(na, rows, wide):
+    p, dev, E, g0, sky, oplan = _setup(128, na, rows, 5, 2, "ci4")
+    p.configure((0.0, 0.0), sky, 0.5, g0=g0)
+    img = p.image(dev).cpu().numpy()
+    assert (p.info()["batch_time"] > 0) == wide
+    p.update()
+    g_ref, _, _, ref, _ = O.epical_interval(oplan, E, g0, 0.5)
+    assert np.linalg.norm(img - ref) / np.linalg.norm(ref) <= 1e-5
+    assert np.max(np.abs(p.gains() - g_ref) / np.abs(g_ref)) <= 1e-4
