@@ -308,11 +308,12 @@ epic_status epic_visibilities(epic_plan_t plan, const void* d_volt, long long n_
  * max_a |g_new - g| <= tol max_a |g_new| or max_iter iterations.  V^M is
  * formed in FP64 from the point-source model of the last epical_configure
  * (V^M_ab = sum_s S_s e^{-2 pi i (u_a - u_b) . s}) on the first solve after
- * it.  The pair products run in FP32 (V and V^M rounded to FP32; the plan
- * holds 2 x C x Na x Na complex64 for them), the sums over antennas, the
- * update, the averaging and the stopping test in FP64, so the solution
- * agrees with an FP64 solve to about 1e-6; the stopping tolerance used is
- * max(tol, 1e-6).  d_vis: device [C][Na][Na]
+ * it.  The pair products run in FP32 (V and V^M rounded to FP32, the model
+ * and the gains brought near 1 by powers of two, so units do not matter; the
+ * plan holds 2.5 x C x Na x Na complex64 for them), the sums over antennas in
+ * two-float FP32 (48 bits), the update, the averaging and the stopping test
+ * in FP64, so the solution agrees with an FP64 solve to about 1e-6; the
+ * stopping tolerance used is max(tol, 1e-6).  d_vis: device [C][Na][Na]
  * complex128 (as from epic_visibilities).  d_gains: device [C][Na]
  * complex128, the start on input and the solution on output; flagged
  * antennas and antennas with no usable pair keep their start value.

@@ -146,8 +146,9 @@ cudaError_t launch_model_vis(int n_chan, int n_ant, int n_src, const double2* ph
                              float2* vm, cudaStream_t s);
 struct StefcalArgs {
   int n_chan, n_ant;
-  float2* w;               // [C][Na][ld] scratch: pair terms V conj(V^M) in FP32
-  float* m2;               // [C][Na][ld] scratch: |V^M|^2
+  float2* w;               // [C][Na][ld] scratch: pair terms V conj(M) in FP32, M = vm_scale V^M
+  float* m2;               // [C][Na][ld] scratch: |M|^2
+  float vm_scale;          // power of two that brings the model near 1
   int ld, rows;            // row stride of both; antennas per CTA (set by the launch)
   const float2* vm;        // [C][Na][Na] model visibilities (FP32)
   const double2* uv;       // [C][Na] antenna positions in wavelengths

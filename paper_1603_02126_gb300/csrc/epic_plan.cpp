@@ -2101,6 +2101,11 @@ epic_status epic_visibility_solve(epic_plan_t p, const double* d_vis, double* d_
   a.w = p->d_sw.p;
   a.m2 = p->d_sm2.p;
   a.vm = p->d_vm.p;
+  // |V^M| is at most the sum of the fluxes
+  double flux = 0.0;
+  for (size_t i = 2; i < p->model.size(); i += 3) flux += std::fabs(p->model[i]);
+  const int e = flux > 0.0 ? std::ilogb(flux) : 0;
+  a.vm_scale = std::abs(e) <= 20 ? 1.0f : std::ldexp(1.0f, -std::min(120, std::max(-120, e)));
   a.uv = p->d_uv.p;
   a.flags = p->d_flags.p;
   a.min_baseline = min_baseline;

@@ -140,9 +140,11 @@ __global__ void model_vis_kernel(int n_chan, int n_ant, int n_src, const double2
 constexpr int kSThreads = 1024;
 constexpr double kStefcalMinTol = 1e-6;   // smallest stopping tolerance with FP32 pair products
 
-// Pair terms of the solve, once per call: W_ab = V_ab conj(V^M_ab) and
-// |V^M_ab|^2 in FP32, zero for the pairs that are left out (autos, flagged
-// antennas, baselines below the cut) and in the padding of a row.
+// Pair terms of the solve, once per call: W_ab = V_ab conj(M_ab) and |M_ab|^2
+// in FP32, M the model times a power of two that keeps its square in range
+// (a model in SI units is near 1e-26), zero for the pairs that are left out
+// (autos, flagged antennas, baselines below the cut) and in the padding of a
+// row.
 __global__ void __launch_bounds__(128) pair_terms_kernel(const StefcalArgs A, const double2* __restrict__ vis) {
   const int Na = A.n_ant, ld = A.ld;
   const long long row = blockIdx.x;                          // channel * Na + antenna
@@ -159,7 +161,8 @@ __global__ void __launch_bounds__(128) pair_terms_kernel(const StefcalArgs A, co
       use = !(dx * dx + dy * dy < mb2);
     }
     if (use) {
-      const float2 m = A.vm[row * Na + b];
+      float2 m = A.vm[row * Na + b];
+      m = make_float2(m.x * A.vm_scale, m.y * A.vm_scale);
       const double2 v = vis[row * Na + b];
       const float vr = static_cast<float>(v.x), vi = static_cast<float>(v.y);
       w = make_float2(fmaf(vr, m.x, vi * m.y), fmaf(vi, m.x, -vr * m.y));
@@ -170,7 +173,24 @@ __global__ void __launch_bounds__(128) pair_terms_kernel(const StefcalArgs A, co
   }
 }
 
-// A sum as hi + lo (FP32 each, error-free two-sum: about 48 bits).
+// Size of a gain, as a number that orders as it: the bits of its larger part;
+// 0 where it is not finite.
+__device__ __forceinline__ unsigned size_of(float2 f) {
+  const unsigned m = __float_as_uint(fmaxf(fabsf(f.x), fabsf(f.y)));
+  return isfinite(f.x) && isfinite(f.y) ? m : 0u;
+}
+
+// Power of two for gains of largest size m: 1 between 2^-20 and 2^20 (and for
+// 0), else one that brings large gains near 2^-16 and small ones near 2^16, so
+// that their squares stay in FP32's range and their products with W too, for
+// visibilities (of order |g|^2) from 2^-120 to 2^120.
+__device__ __forceinline__ float gain_scale(unsigned m) {
+  const int k = static_cast<int>(m >> 23) - 127;
+  if (m == 0u || (k >= -20 && k <= 20)) return 1.f;
+  return ldexpf(1.f, k > 0 ? -k - 16 : -k + 16 > 120 ? 120 : -k + 16);
+}
+
+// A sum as hi + lo (FP32 each, error-free two-sum (Knuth): about 48 bits).
 struct Sum2 {
   float hi, lo;
   __device__ __forceinline__ void add(float h, float l) {
@@ -179,6 +199,12 @@ struct Sum2 {
     hi = s;
   }
 };
+
+// Largest of the values so far (non-negative doubles order as their bits; NaN
+// is passed over).
+__device__ __forceinline__ void raise(unsigned long long* most, double v) {
+  if (v >= 0.0) atomicMax(most, static_cast<unsigned long long>(__double_as_longlong(v)));
+}
 
 // Sums over the warp of three values of four rows: lane 8 j ends with row j's.
 __device__ __forceinline__ void sum_rows(const float (&v)[4][3], Sum2 (&out)[3]) {
@@ -210,7 +236,8 @@ __device__ __forceinline__ void sum_rows(const float (&v)[4][3], Sum2 (&out)[3])
 // its FP32 rate, and the FP64 lane reductions took a third of an iteration),
 // one thread per antenna divides, averages and tests in FP64 and writes the
 // new gain, rounded to FP32, into every CTA's shared memory; one cluster
-// barrier per iteration.
+// barrier per iteration.  Gains far from 1 (|g|^2 alone would leave FP32's
+// range) are multiplied by a power of two before an iteration uses them.
 //
 // What bounds it: W and |V^M|^2 (12 bytes a pair) come through L2 once per
 // iteration, the division and a cluster barrier follow in series.
@@ -225,6 +252,7 @@ __global__ void __launch_bounds__(kSThreads) stefcal_kernel(const StefcalArgs A)
   float* sums = reinterpret_cast<float*>(g + rows);          // [rows][6] (hi, lo) of Re, Im, denominator
   __shared__ unsigned long long most[2][2];                  // by parity: largest |change|^2, |g|^2 of this CTA
   __shared__ unsigned long long all[2][2][8];                // the same of every CTA of the cluster
+  __shared__ unsigned size[2], sizes[2][8];                  // likewise the largest size of the gains in use
   const int cl = static_cast<int>(cluster.num_blocks()), q = static_cast<int>(cluster.block_rank());
   const int c = blockIdx.x / cl;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -232,6 +260,8 @@ __global__ void __launch_bounds__(kSThreads) stefcal_kernel(const StefcalArgs A)
   const float2* W = A.w + static_cast<size_t>(c) * Na * ld;
   const float* M = A.m2 + static_cast<size_t>(c) * Na * ld;
   double2* gio = A.gains + static_cast<size_t>(c) * Na;
+  if (threadIdx.x < 2) size[threadIdx.x] = 0u;
+  __syncthreads();
   for (int a = threadIdx.x; a < ld; a += kSThreads) {
     const double2 v = a < Na ? gio[a] : make_double2(0.0, 0.0);
     const bool live = a < Na && !A.flags[a];
@@ -240,14 +270,24 @@ __global__ void __launch_bounds__(kSThreads) stefcal_kernel(const StefcalArgs A)
     gf[ld + a] = make_float2(0.f, 0.f);
     g2[a] = fmaf(f.x, f.x, f.y * f.y);
     g2[ld + a] = 0.f;
+    atomicMax(&size[1], size_of(f));
     if (a >= a0 && a < a0 + na) g[a - a0] = v;
   }
   if (threadIdx.x < 4) most[threadIdx.x >> 1][threadIdx.x & 1] = 0ull;
   cluster.sync();                                            // every CTA is resident and has read the gains
   const double tol = fmax(A.tol, kStefcalMinTol), tol2 = tol * tol;
+  float t = gain_scale(size[1]);                             // of the whole start, in every CTA
   int it = 0;
   for (; it < A.max_iter;) {
     const int cur = it & 1, nxt = cur ^ 1;
+    if (t != 1.f) {                                          // of the whole cluster
+      for (int a = threadIdx.x; a < ld; a += kSThreads) {
+        const float2 f = make_float2(gf[cur * ld + a].x * t, gf[cur * ld + a].y * t);
+        gf[cur * ld + a] = f;
+        g2[cur * ld + a] = fmaf(f.x, f.x, f.y * f.y);
+      }
+      __syncthreads();
+    }
     const float4* gp = reinterpret_cast<const float4*>(gf + cur * ld);
     const float4* hp = reinterpret_cast<const float4*>(g2 + cur * ld);
     for (int r = 4 * warp; r < na; r += 4 * (kSThreads / 32)) {
@@ -293,17 +333,21 @@ __global__ void __launch_bounds__(kSThreads) stefcal_kernel(const StefcalArgs A)
       if (den > 0.0) {
         x.x = (static_cast<double>(s[0]) + static_cast<double>(s[1])) / den;
         x.y = (static_cast<double>(s[2]) + static_cast<double>(s[3])) / den;
+        if (t != 1.f || A.vm_scale != 1.f) {                 // the sums were those of s V^M and t g
+          const double st = static_cast<double>(A.vm_scale) * static_cast<double>(t);
+          x.x *= st;
+          x.y *= st;
+        }
       }
       if (it & 1) x = make_double2(0.5 * (x.x + o.x), 0.5 * (x.y + o.y));
       const double dx = x.x - o.x, dy = x.y - o.y;
       g[r] = x;
-      // non-negative doubles order as their bits; NaN is passed over
-      const double d2 = dx * dx + dy * dy, x2 = x.x * x.x + x.y * x.y;
-      if (d2 >= 0.0) atomicMax(&most[cur][0], static_cast<unsigned long long>(__double_as_longlong(d2)));
-      if (x2 >= 0.0) atomicMax(&most[cur][1], static_cast<unsigned long long>(__double_as_longlong(x2)));
+      raise(&most[cur][0], dx * dx + dy * dy);
+      raise(&most[cur][1], x.x * x.x + x.y * x.y);
       if (!A.flags[a0 + r]) {
         const float2 f = make_float2(static_cast<float>(x.x), static_cast<float>(x.y));
         const float h = fmaf(f.x, f.x, f.y * f.y);
+        atomicMax(&size[cur], size_of(f));
         for (int d = 0; d < cl; ++d) {
           cluster.map_shared_rank(gf, d)[nxt * ld + a0 + r] = f;
           cluster.map_shared_rank(g2, d)[nxt * ld + a0 + r] = h;
@@ -315,15 +359,20 @@ __global__ void __launch_bounds__(kSThreads) stefcal_kernel(const StefcalArgs A)
       unsigned long long(*dst)[2][8] = cluster.map_shared_rank(all, static_cast<int>(threadIdx.x));
       dst[cur][0][q] = most[cur][0];
       dst[cur][1][q] = most[cur][1];
+      cluster.map_shared_rank(sizes, static_cast<int>(threadIdx.x))[cur][q] = size[cur];
     }
     if (threadIdx.x < 2) most[nxt][threadIdx.x] = 0ull;
+    if (threadIdx.x == 2) size[nxt] = 0u;
     cluster.sync();
     ++it;
     unsigned long long d = 0, m = 0;
+    unsigned u = 0;
     for (int k = 0; k < cl; ++k) {
       d = all[cur][0][k] > d ? all[cur][0][k] : d;
       m = all[cur][1][k] > m ? all[cur][1][k] : m;
+      u = sizes[cur][k] > u ? sizes[cur][k] : u;
     }
+    t = gain_scale(u);
     // FP32 pair products: changes below ~1e-6 are rounding, not progress
     if (__longlong_as_double(static_cast<long long>(d)) <= tol2 * __longlong_as_double(static_cast<long long>(m))) break;
   }
