@@ -142,9 +142,9 @@ constexpr double kStefcalMinTol = 1e-6;   // smallest stopping tolerance with FP
 
 // Pair terms of the solve, once per call: W_ab = V_ab conj(M_ab) and |M_ab|^2
 // in FP32, M the model times a power of two that keeps its square in range
-// (a model in SI units is near 1e-26), zero for the pairs that are left out
+// (a model in SI units is near 1e-26).  For the pairs that are left out
 // (autos, flagged antennas, baselines below the cut) and in the padding of a
-// row.
+// row W is 0 and |M|^2 is -0, which adds nothing and tells them apart.
 __global__ void __launch_bounds__(128) pair_terms_kernel(const StefcalArgs A, const double2* __restrict__ vis) {
   const int Na = A.n_ant, ld = A.ld;
   const long long row = blockIdx.x;                          // channel * Na + antenna
@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(128) pair_terms_kernel(const StefcalArgs A, co
   const bool live = !A.flags[a];
   for (int b = threadIdx.x; b < ld; b += 128) {
     float2 w = make_float2(0.f, 0.f);
-    float m2 = 0.f;
+    float m2 = -0.f;
     bool use = live && b < Na && b != a && !A.flags[b];
     if (use && mb2 > 0.0) {
       const double2 ua = A.uv[row], ub = A.uv[static_cast<size_t>(c) * Na + b];
@@ -174,10 +174,11 @@ __global__ void __launch_bounds__(128) pair_terms_kernel(const StefcalArgs A, co
 }
 
 // Size of a gain, as a number that orders as it: the bits of its larger part;
-// 0 where it is not finite.
+// kNotFinite where it is not finite.
+constexpr unsigned kNotFinite = 0x7f800000u;
 __device__ __forceinline__ unsigned size_of(float2 f) {
   const unsigned m = __float_as_uint(fmaxf(fabsf(f.x), fabsf(f.y)));
-  return isfinite(f.x) && isfinite(f.y) ? m : 0u;
+  return isfinite(f.x) && isfinite(f.y) ? m : kNotFinite;
 }
 
 // Power of two for gains of largest size m: 1 between 2^-20 and 2^20 (and for
@@ -253,6 +254,7 @@ __global__ void __launch_bounds__(kSThreads) stefcal_kernel(const StefcalArgs A)
   __shared__ unsigned long long most[2][2];                  // by parity: largest |change|^2, |g|^2 of this CTA
   __shared__ unsigned long long all[2][2][8];                // the same of every CTA of the cluster
   __shared__ unsigned size[2], sizes[2][8];                  // likewise the largest size of the gains in use
+  __shared__ unsigned finite;                                // the same of the finite ones
   const int cl = static_cast<int>(cluster.num_blocks()), q = static_cast<int>(cluster.block_rank());
   const int c = blockIdx.x / cl;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -276,11 +278,25 @@ __global__ void __launch_bounds__(kSThreads) stefcal_kernel(const StefcalArgs A)
   if (threadIdx.x < 4) most[threadIdx.x >> 1][threadIdx.x & 1] = 0ull;
   cluster.sync();                                            // every CTA is resident and has read the gains
   const double tol = fmax(A.tol, kStefcalMinTol), tol2 = tol * tol;
-  float t = gain_scale(size[1]);                             // of the whole start, in every CTA
+  unsigned u = size[1];                                      // of the whole start, in every CTA
   int it = 0;
   for (; it < A.max_iter;) {
     const int cur = it & 1, nxt = cur ^ 1;
-    if (t != 1.f) {                                          // of the whole cluster
+    // a gain in use that is not finite reaches the pairs it is part of, but
+    // not, as 0 times it, those that are left out
+    const bool skip = u == kNotFinite;                       // of the whole cluster, as t
+    if (skip) {
+      if (threadIdx.x == 0) finite = 0u;
+      __syncthreads();
+      for (int a = threadIdx.x; a < ld; a += kSThreads) {
+        const unsigned m = size_of(gf[cur * ld + a]);
+        if (m != kNotFinite) atomicMax(&finite, m);
+      }
+      __syncthreads();
+      u = finite;
+    }
+    const float t = gain_scale(u);
+    if (t != 1.f) {
       for (int a = threadIdx.x; a < ld; a += kSThreads) {
         const float2 f = make_float2(gf[cur * ld + a].x * t, gf[cur * ld + a].y * t);
         gf[cur * ld + a] = f;
@@ -302,6 +318,18 @@ __global__ void __launch_bounds__(kSThreads) stefcal_kernel(const StefcalArgs A)
           const float4* wp = reinterpret_cast<const float4*>(W + static_cast<size_t>(row) * ld);
           const float4 w0 = __ldg(wp + 2 * b), w1 = __ldg(wp + 2 * b + 1);
           const float4 m = __ldg(reinterpret_cast<const float4*>(M + static_cast<size_t>(row) * ld) + b);
+          if (skip) {
+            const float wr[4] = {w0.x, w0.z, w1.x, w1.z}, wi[4] = {w0.y, w0.w, w1.y, w1.w}, mm[4] = {m.x, m.y, m.z, m.w};
+            const float xr[4] = {x0.x, x0.z, x1.x, x1.z}, xi[4] = {x0.y, x0.w, x1.y, x1.w}, yy[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+              if (!signbit(mm[j])) {
+                v[i][0] = fmaf(wr[j], xr[j], fmaf(-wi[j], xi[j], v[i][0]));
+                v[i][1] = fmaf(wr[j], xi[j], fmaf(wi[j], xr[j], v[i][1]));
+                v[i][2] = fmaf(mm[j], yy[j], v[i][2]);
+              }
+            continue;
+          }
           v[i][0] = fmaf(w0.x, x0.x, fmaf(-w0.y, x0.y, v[i][0]));
           v[i][1] = fmaf(w0.x, x0.y, fmaf(w0.y, x0.x, v[i][1]));
           v[i][0] = fmaf(w0.z, x0.z, fmaf(-w0.w, x0.w, v[i][0]));
@@ -313,14 +341,14 @@ __global__ void __launch_bounds__(kSThreads) stefcal_kernel(const StefcalArgs A)
           v[i][2] = fmaf(m.x, y.x, fmaf(m.y, y.y, fmaf(m.z, y.z, fmaf(m.w, y.w, v[i][2]))));
         }
       }
-      Sum2 t[3];
-      sum_rows(v, t);
+      Sum2 sum[3];
+      sum_rows(v, sum);
       const int row = r + (lane >> 3);
       if ((lane & 7) == 0 && row < na) {
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-          sums[row * 6 + 2 * k] = t[k].hi;
-          sums[row * 6 + 2 * k + 1] = t[k].lo;
+          sums[row * 6 + 2 * k] = sum[k].hi;
+          sums[row * 6 + 2 * k + 1] = sum[k].lo;
         }
       }
     }
@@ -366,13 +394,12 @@ __global__ void __launch_bounds__(kSThreads) stefcal_kernel(const StefcalArgs A)
     cluster.sync();
     ++it;
     unsigned long long d = 0, m = 0;
-    unsigned u = 0;
+    u = 0;
     for (int k = 0; k < cl; ++k) {
       d = all[cur][0][k] > d ? all[cur][0][k] : d;
       m = all[cur][1][k] > m ? all[cur][1][k] : m;
       u = sizes[cur][k] > u ? sizes[cur][k] : u;
     }
-    t = gain_scale(u);
     // FP32 pair products: changes below ~1e-6 are rounding, not progress
     if (__longlong_as_double(static_cast<long long>(d)) <= tol2 * __longlong_as_double(static_cast<long long>(m))) break;
   }
