@@ -386,6 +386,7 @@ struct TcArgs {
   const int2* lists_at;    // [C][nb_max] (offset, bytes) / 16 of each block's lists
   int nb_max, max_lists, rb;
   int lists_smem;          // 1: two blocks' lists fit in shared memory
+  int one;                 // 1: E' of a frame pair does not fit, one frame at a time
   const int* row_cost;     // [C + 1] prefix sums of a frame pair's cost
   const float2* pixel;     // [C][Na] response of the calibrator pixel without phasing
 };

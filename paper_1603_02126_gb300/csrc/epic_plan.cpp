@@ -218,6 +218,7 @@ struct epic_plan_s {
   alignas(64) unsigned char tm_data[128];
   int kr = 0;                   // K extent of the row DFT (2 x window columns, padded to 64)
   int tc_rb = 0, tc_lists_smem = 0;   // gridding: rows per block of lists, lists in shared memory
+  int tc_one = 0;                     // gridding: one frame at a time
   DevBuf<float2> d_tc_pixel;    // [C][Na] response of the calibrator pixel without phasing
   DevBuf<uint16_t> d_tc_gh;     // [tc_time*C*rows_alloc][kr] scaled window grid
   DevBuf<uint16_t> d_tc_dftr;   // [2N][kr] row DFT over window columns
@@ -1155,6 +1156,7 @@ epic_status image_tc(epic_plan_t p, const void* d_volt, long long n_time, double
   a.max_lists = p->w_max_lists;
   a.rb = p->tc_rb;
   a.lists_smem = p->tc_lists_smem;
+  a.one = p->tc_one;
   a.row_cost = p->d_wrcost.p;
   a.pixel = p->d_tc_pixel.p;
   a.gh = p->d_tc_gh.p;
@@ -1433,6 +1435,7 @@ epic_status choose_path(epic_plan_s* p, const epic_plan_desc* d, bool fused_shap
       p->tc_lists_smem = (p->tc_rb > 4 ? 4 : 1) * need <= static_cast<size_t>(smem_optin);
       if (p->tc_lists_smem || p->tc_rb <= 4) break;
     }
+    p->tc_one = epic::tc_grid_smem(Na, p->tc_rb, p->kr, 0) + 1024 > static_cast<size_t>(smem_optin);
     p->w_nb_max = wide->nb_max;
     p->w_max_lists = wide->max_lists;
   }

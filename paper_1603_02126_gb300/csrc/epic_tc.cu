@@ -241,6 +241,94 @@ __global__ void __launch_bounds__(kLBT) grid_lp_kernel(const TcArgs A, long long
   if (tid == 0) bulk_store_wait_all();
 }
 
+// The same for arrays whose E' of a frame pair does not fit shared memory (more
+// than about 13 500 antennas): one frame at a time, E' as 8 bytes per antenna
+// (28 900 antennas), the lists through L1 and the cells stored as they are
+// summed.  The slices of all blocks are dealt to the 32 warps in turn, since a
+// block has fewer slices than the CTA warps (each block's from warp 0: 2.7 times
+// the call).  Bound by the list entries and E' of a tap, read for one frame
+// only: calls of 128 samples, 8 channels at N = 256, 14 900 antennas 0.55 ms,
+// 28 900 0.91 (1.12 and 1.87 with lane lists and 8 warps).
+constexpr int kOBT = 1024;         // threads: one CTA per SM
+template <int FMT, typename T>
+__global__ void __launch_bounds__(kOBT) grid_lp_one_kernel(const TcArgs A, long long t0, int nt) {
+  extern __shared__ __align__(16) float2 glp_es[];           // [Na] E' of the frame
+  __shared__ float red[kOBT / 32];
+  const int C = A.u.n_chan, Na = A.u.n_ant, rb = A.rb, kc = A.kr / 2, tid = threadIdx.x;
+  const int lane = tid & 31, warp = tid >> 5;
+  T* gh = static_cast<T*>(A.gh);
+  const long long frames = static_cast<long long>(nt) * C;
+  for (long long it = blockIdx.x; it < frames; it += gridDim.x) {
+    const int c = static_cast<int>(it / nt), tl = static_cast<int>(it - static_cast<long long>(c) * nt);
+    const size_t f = static_cast<size_t>(tl) * C + c, ic = static_cast<size_t>(c) * Na;
+    const size_t i0 = (static_cast<size_t>(t0 + tl) * C + c) * Na;
+    const float vs = A.u.vscale ? __ldg(A.u.vscale + c) : 1.0f;
+    float v[3] = {0.f, 0.f, 0.f};                            // S_f and the calibrator pixel, as in the pair kernel
+#pragma unroll 4
+    for (int a = tid; a < Na; a += kOBT) {
+      const float2 e = fft::cmul(pair_volt<FMT>(A.u.volt, i0 + a, vs), __ldg(A.u.wgain + ic + a));
+      glp_es[a] = e;
+      if (__ldg(A.u.cell0 + ic + a) >= 0) {
+        v[0] += sqrtf(e.x * e.x + e.y * e.y);
+        if (A.u.do_cal) {
+          const float2 r = __ldg(A.pixel + ic + a);
+          v[1] = fmaf(r.x, e.x, fmaf(-r.y, e.y, v[1]));
+          v[2] = fmaf(r.x, e.y, fmaf(r.y, e.x, v[2]));
+        }
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) v[j] += __shfl_xor_sync(fft::kFull, v[j], o);
+      if (lane == 0) red[warp] = v[j];
+      __syncthreads();
+      v[j] = 0.f;
+#pragma unroll
+      for (int w = 0; w < kOBT / 32; ++w) v[j] += red[w];
+      __syncthreads();
+    }
+    const int k = pow2_exp_below_inverse(v[0] / static_cast<float>(Na));
+    const float sf = exp2i(k);                               // s_f multiplies the cells
+    if (tid == 0) {
+      A.fscale[f] = sf;
+      A.finv2[f] = exp2i(-2 * k);                            // 1 / s_f^2 multiplies |D|^2
+      if (A.u.do_cal) A.u.pix[f] = make_float2(v[1], v[2]);
+    }
+    const int4 wn = __ldg(A.win4 + c);                       // (y0, rows, x0, cols)
+    T* dst = gh + f * A.r_alloc * A.kr;
+    const int pad = kc - wn.w;                               // columns past this channel's window
+    for (int i = tid; i < wn.y * pad; i += kOBT) store_lp(dst + static_cast<size_t>(i / pad) * A.kr + 2 * (wn.w + i % pad), 0.f, 0.f);
+    const int nb = (wn.y + rb - 1) / rb;
+    int turn = warp;                                         // slices dealt to the warps across the blocks
+    for (int b = 0; b < nb; ++b) {
+      const unsigned char* lists = A.lists + static_cast<size_t>(__ldg(A.lists_at + c * A.nb_max + b).x) * 16;
+      const BlockLists hd = *reinterpret_cast<const BlockLists*>(lists);
+      const int2* slice = reinterpret_cast<const int2*>(lists + sizeof(BlockLists));
+      const uint16_t* cell = reinterpret_cast<const uint16_t*>(lists + hd.cells);
+      const uint2* ent = reinterpret_cast<const uint2*>(lists + hd.ents);
+      int n = turn;
+      for (; n < hd.nslice; n += kOBT / 32) {
+        const int2 sl = slice[n];
+        const unsigned at = cell[n * 32 + lane];
+        float2 sum = make_float2(0.f, 0.f);
+#pragma unroll 4
+        for (int m = 0; m < sl.y; ++m) {
+          const uint2 en = __ldg(ent + sl.x + m * 32 + lane);
+          // weight 0: behind the end of a shorter list, antenna Na
+          const float2 x = en.y ? glp_es[en.x / 16] : make_float2(0.f, 0.f);
+          const float w = __uint_as_float(en.y);
+          sum.x = fmaf(w, x.x, sum.x);
+          sum.y = fmaf(w, x.y, sum.y);
+        }
+        if (at != 0xffffu) store_lp(dst + static_cast<size_t>(b) * rb * A.kr + 2 * at, sum.x * sf, sum.y * sf);
+      }
+      turn = n - hd.nslice;
+    }
+    __syncthreads();                                         // E' is read out
+  }
+}
+
 // ---------------------------------------------------------------------------
 // tcgen05 / TMA / mbarrier helpers (inline PTX)
 // ---------------------------------------------------------------------------
@@ -1039,8 +1127,25 @@ cudaError_t grid_lp_launch(const TcArgs& a, long long t0, int nt, int sms, cudaS
   return cudaGetLastError();
 }
 
+template <int FMT, typename T>
+cudaError_t grid_lp_one_launch(const TcArgs& a, long long t0, int nt, int sms, cudaStream_t s) {
+  const size_t smem = static_cast<size_t>(a.u.n_ant) * sizeof(float2);
+  auto k = grid_lp_one_kernel<FMT, T>;
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  if (e != cudaSuccess) return e;
+  int per_sm = 0;
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kOBT, smem);
+  if (e != cudaSuccess) return e;
+  const long long frames = static_cast<long long>(nt) * a.u.n_chan;
+  const long long most = static_cast<long long>(per_sm > 0 ? per_sm : 1) * sms;
+  k<<<static_cast<unsigned>(frames < most ? frames : most), kOBT, smem, s>>>(a, t0, nt);
+  return cudaGetLastError();
+}
+
 template <typename T>
 cudaError_t grid_lp(const TcArgs& a, long long t0, int nt, int sms, cudaStream_t s) {
+  if (a.one)
+    return a.u.input_fmt ? grid_lp_one_launch<1, T>(a, t0, nt, sms, s) : grid_lp_one_launch<0, T>(a, t0, nt, sms, s);
   if (a.lists_smem)
     return a.u.input_fmt ? grid_lp_launch<1, T, true>(a, t0, nt, sms, s) : grid_lp_launch<0, T, true>(a, t0, nt, sms, s);
   return a.u.input_fmt ? grid_lp_launch<1, T, false>(a, t0, nt, sms, s) : grid_lp_launch<0, T, false>(a, t0, nt, sms, s);
