@@ -20,6 +20,7 @@
 #include <algorithm>
 
 #include "epic_internal.h"
+#include "epic_sum.cuh"
 
 namespace epic {
 namespace {
@@ -191,13 +192,12 @@ __device__ __forceinline__ float gain_scale(unsigned m) {
   return ldexpf(1.f, k > 0 ? -k - 16 : -k + 16 > 120 ? 120 : -k + 16);
 }
 
-// A sum as hi + lo (FP32 each, error-free two-sum (Knuth): about 48 bits).
+// A sum as hi + lo (FP32 each).
 struct Sum2 {
   float hi, lo;
   __device__ __forceinline__ void add(float h, float l) {
-    const float s = hi + h, t = s - hi;
-    lo += l + ((hi - (s - t)) + (h - t));
-    hi = s;
+    lo += l;
+    add_kept(hi, lo, h);
   }
 };
 
