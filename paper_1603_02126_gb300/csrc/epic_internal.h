@@ -62,6 +62,8 @@ struct ImageArgs {
   const int* psbase;       // [C + 1] first slice of each channel
   const int* pebase;       // [C + 1] first entry of each channel
   const int* pcost;        // [C + 1] prefix sums of the channels' cost per frame pair
+  int run;                 // frame pairs per FP32 partial image
+  int corr_mask;           // frame pairs per FP32 partial correlation, a power of two, minus 1
   int gs;                  // row stride of the grid (16-byte cells)
   int max_slices, max_ent; // most slices / entries of one channel (0: lists not in shared memory)
 };
@@ -323,6 +325,7 @@ struct WideArgs {
   const int* col_cost;     // [C + 1] prefix sums of the column kernel's cost per pair and block
   int rows_ctas, cols_ctas;
   int rows_grid;           // CTAs of this row launch
+  int run;                 // frame pairs per FP32 partial image
 };
 bool wide_supported(int n);
 int wide_row_block(int n);   // grid rows per block of lists

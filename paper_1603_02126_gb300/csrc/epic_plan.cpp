@@ -725,6 +725,27 @@ epic_status build_wide_lists(const epic_plan_s* p, const std::vector<float>& wts
   return EPIC_OK;
 }
 
+// Frame pairs per FP32 partial image of a call of P pairs.  A run of r pairs
+// rounds its sum r times, P / r runs are summed in FP64: r / sqrt(3 P) roundings
+// of the image.  Short calls need short runs to stay at what the one-frame
+// kernels' segments rounded (image error of 128 samples, 128 x 128: 8.3e-8
+// with runs of 27 pairs, 7.2e-8 with 16, 7.4e-8 in segments of 16 samples; of
+// 128 samples, 512 x 512: 1.64e-7 with 64, 1.38e-7 with 32, 1.45e-7), long ones
+// can save on adding the image blocks (10^4 samples: 16.5 ms with 16, 15.4
+// with 128).
+int run_pairs(long long pairs, int least) {
+  return static_cast<int>(std::min<long long>(128, std::max<long long>(least, pairs / 16)));
+}
+
+// Frame pairs per FP32 partial correlation of such a call: a power of two near
+// P / 40 (gain error of 128 samples: 5.2e-8 with 27, 3.2e-8 with 8; 3.3e-8 with
+// one frame per value).
+int corr_pairs(long long pairs) {
+  int r = 8;
+  while (r < 128 && 40LL * 2 * r <= pairs) r *= 2;
+  return r;
+}
+
 // Samples of a call up to which one frame per FP32 value is the faster form:
 // half of a single sample's pair is empty, and a pair has more latency than
 // two frames on small grids (one-frame against frame-pair, us: one sample of
@@ -787,6 +808,8 @@ epic::ImageArgs fused_args(epic_plan_t p, const void* d_volt, long long n_time, 
   a.wait_limit = p->wait_limit;
   if (pair) {
     a.pair = 1;
+    a.run = run_pairs((n_time + 1) / 2, 16);
+    a.corr_mask = corr_pairs((n_time + 1) / 2) - 1;
     a.pcell = p->d_pcell.p;
     a.pslice = p->d_pslice.p;
     a.pent = p->d_pent.p;
@@ -913,6 +936,7 @@ epic_status image_wide(epic_plan_t p, const void* d_volt, long long n_time, doub
   p->ws_time = static_cast<int>(std::max<long long>(1, nt * nc / C));   // samples of all channels the scratch holds
   epic::WideArgs w{};
   wide_plan_args(p, &w);
+  w.run = run_pairs((n_time + 1) / 2, 32);
   epic::UnfusedArgs& a = w.u;
   a.volt = d_volt;
   a.input_fmt = p->input;

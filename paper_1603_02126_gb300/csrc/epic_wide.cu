@@ -46,8 +46,6 @@ using fft::f2_pack;
 
 constexpr int kWBT = 128;          // threads of the row kernel; two CTAs per SM (255 registers each)
 constexpr int kWP = 32;            // outputs per task
-// Frame pairs per FP32 partial image (FP64 across), as in the fused form.
-constexpr int kWideRun = 128;
 
 template <int N>
 struct WGeo {
@@ -257,8 +255,8 @@ __global__ void __launch_bounds__(WGeo<N>::CT, 256 / WGeo<N>::CT) wide_cols_kern
     };
     const bool pix = A.do_cal && kx == A.k0x && r == A.k0y % NR;
     if (tid == 0) load(p_lo, it & 1);                        // both slots are free here
-    for (long long pa = p_lo; pa < p_hi; pa += kWideRun) {
-      const long long pb = pa + kWideRun < p_hi ? pa + kWideRun : p_hi;
+    for (long long pa = p_lo; pa < p_hi; pa += W.run) {
+      const long long pb = pa + W.run < p_hi ? pa + W.run : p_hi;
       float acc[kWP];
 #pragma unroll
       for (int m = 0; m < kWP; ++m) acc[m] = 0.f;
