@@ -25,7 +25,7 @@ CU_SOURCES = ["epic_kernels.cu", "epic_pair.cu", "epic_pair_adjoint.cu", "epic_w
 CXX_SOURCES = ["epic_plan.cpp"]
 HEADERS = [os.path.join(CSRC, "epic_internal.h"), os.path.join(CSRC, "epic_fft.cuh"),
            os.path.join(CSRC, "epic_fused_geo.cuh"), os.path.join(CSRC, "epic_residue.cuh"),
-           os.path.join(CSRC, "epic_batch.h"), os.path.join(CSRC, "epic_bulk.cuh"), os.path.join(CSRC, "epic_lists.cuh"), os.path.join(CSRC, "epic_sum.cuh"), os.path.join(CSRC, "epic_pair.cuh"),
+           os.path.join(CSRC, "epic_batch.h"), os.path.join(CSRC, "epic_bulk.cuh"), os.path.join(CSRC, "epic_lists.cuh"), os.path.join(CSRC, "epic_sum.cuh"), os.path.join(CSRC, "epic_smem.cuh"), os.path.join(CSRC, "epic_pair.cuh"),
            os.path.join(ROOT, "include", "epic.h")]
 
 

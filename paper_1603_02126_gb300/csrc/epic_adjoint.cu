@@ -10,6 +10,7 @@
 #include "epic_fft.cuh"
 #include "epic_fused_geo.cuh"
 #include "epic_internal.h"
+#include "epic_smem.cuh"
 
 #include <cstdint>
 
@@ -511,7 +512,7 @@ cudaError_t adjoint_n(const AdjointArgs& a, bool bf16, cudaStream_t s) {
   void (*k)(AdjointArgs);
   if (a.n_ant <= Cfg<N>::BT) k = bf16 ? epic_image_adjoint_b2<N, 1> : epic_image_adjoint<N, 1>;
   else k = bf16 ? epic_image_adjoint_b2<N, kMaxAntPerThread> : epic_image_adjoint<N, kMaxAntPerThread>;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(a.smem));
+  cudaError_t e = allow_smem(k);
   if (e != cudaSuccess) return e;
   k<<<a.grid, Cfg<N>::BT, a.smem, s>>>(a);
   return cudaGetLastError();

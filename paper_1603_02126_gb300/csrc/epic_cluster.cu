@@ -21,6 +21,7 @@
 
 #include "epic_fft.cuh"
 #include "epic_internal.h"
+#include "epic_smem.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -310,8 +311,7 @@ cudaError_t cluster_launch_n(const ClusterArgs& a, cudaStream_t s) {
 
 template <int N>
 cudaError_t cluster_prepare_n(size_t smem, int* clusters) {
-  cudaError_t e = cudaFuncSetAttribute(epic_image_cluster<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
+  cudaError_t e = allow_smem(epic_image_cluster<N>);
   if (e != cudaSuccess) return e;
   if (KCfg<N>::CS > 8) {
     e = cudaFuncSetAttribute(epic_image_cluster<N>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);

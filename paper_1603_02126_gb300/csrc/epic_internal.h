@@ -399,8 +399,7 @@ bool tc_make_row_maps(void* gh, void* dftr, long long rows_cap, int n, int kr, b
                       void* tm_fr);
 bool tc_supported(int n, int rows_alloc);
 int tc_kp(int rows_alloc);
-size_t tc_smem(int kp);
-cudaError_t tc_prepare(bool bf16, size_t smem);
+cudaError_t tc_prepare(bool bf16);
 bool tc_make_maps(void* dft, void* hh, int n, int n_chan, int tb_cap, int kp, bool bf16, void* tm_dft,
                   void* tm_data);
 cudaError_t launch_tc_batch(const TcArgs& a, const void* tm_dft, const void* tm_data, long long t0, int nt,

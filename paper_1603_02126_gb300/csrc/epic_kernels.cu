@@ -27,6 +27,7 @@
 #include "epic_fft.cuh"
 #include "epic_fused_geo.cuh"
 #include "epic_internal.h"
+#include "epic_smem.cuh"
 
 #include <cstdint>
 
@@ -602,17 +603,10 @@ __global__ void unpack_ci4_kernel(const unsigned char* __restrict__ in, float2* 
   }
 }
 
-// The shared-memory attribute belongs to the kernel, not to a plan: always the
-// device's limit, so that plans of different footprints can live side by side.
 template <int N, int MAXA, int F>
 cudaError_t prepare_nmf(size_t smem, int* ctas) {
-  int dev = 0, most = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(epic_image_fused<N, MAXA, true, F>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(epic_image_fused<N, MAXA, false, F>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  cudaError_t e = allow_smem(epic_image_fused<N, MAXA, true, F>);
+  if (e == cudaSuccess) e = allow_smem(epic_image_fused<N, MAXA, false, F>);
   if (e != cudaSuccess) return e;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas, epic_image_fused<N, MAXA, true, F>,
                                                        Cfg<N>::BT, smem);

@@ -27,6 +27,7 @@
 #include "epic_fft.cuh"
 #include "epic_internal.h"
 #include "epic_pair.cuh"
+#include "epic_smem.cuh"
 
 #include <cstdint>
 
@@ -311,16 +312,9 @@ size_t pair_smem_bytes(int n, int n_ant, int rows, int gs, int max_slices, int m
 }
 
 cudaError_t pair_prepare(int n, int n_ant, bool table, size_t smem, int* ctas_per_sm) {
-  // the attribute belongs to the kernel, not to a plan: always the device's
-  // limit, so that plans of different footprints can live side by side
-  int dev = 0, most = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   const int bt = pair_threads(n);
-  for (int k = 0; k < 4; ++k) {
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(pair_kernel(n, k & 1, n_ant > bt, table, k > 1), cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-  }
+  cudaError_t e = cudaSuccess;
+  for (int k = 0; k < 4 && e == cudaSuccess; ++k) e = allow_smem(pair_kernel(n, k & 1, n_ant > bt, table, k > 1));
   if (e != cudaSuccess) return e;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, pair_kernel(n, 0, n_ant > bt, table, false), bt, smem);
 }

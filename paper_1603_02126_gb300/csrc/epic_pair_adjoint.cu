@@ -33,6 +33,7 @@
 // bank (0.59 against 0.58 ms for 8192 frames), without unrolled taps 0.58
 // against 0.56.
 #include "epic_pair.cuh"
+#include "epic_smem.cuh"
 
 namespace epic {
 namespace {
@@ -323,10 +324,7 @@ template <int N>
 cudaError_t adj_launch(const ImageArgs& a, const double* dldi, double2* dldw, cudaStream_t s) {
   constexpr int BT = PCfg<N>::BT;
   const AdjKernel k = a.input_fmt ? adj_nf<N, 1>(a.n_ant > BT, a.gsmem != 0) : adj_nf<N, 0>(a.n_ant > BT, a.gsmem != 0);
-  int dev = 0, most = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  const cudaError_t e = allow_smem(k);
   if (e != cudaSuccess) return e;
   k<<<a.grid, BT, a.smem, s>>>(a, dldi, dldw);
   return cudaGetLastError();

@@ -17,6 +17,7 @@
 // waiting (results are then discarded by the host).
 #include "epic_fft.cuh"
 #include "epic_internal.h"
+#include "epic_smem.cuh"
 
 #include <cstdint>
 
@@ -399,7 +400,7 @@ __global__ void __launch_bounds__(kBT, 1) epic_image_piped(const ImageArgs A) {
 template <int N, bool TS>
 cudaError_t piped_launch_t(const ImageArgs& a, cudaStream_t s, bool prepare_only, size_t smem, int* ctas) {
   auto k = epic_image_piped<N, TS, 4, 2>;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  cudaError_t e = allow_smem(k);
   if (e != cudaSuccess) return e;
   if (prepare_only) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas, k, kBT, smem);
   k<<<a.grid, kBT, a.smem, s>>>(a);

@@ -1448,7 +1448,7 @@ epic_status choose_path(epic_plan_s* p, const epic_plan_desc* d, bool fused_shap
       return fail(EPIC_ERR_UNSUPPORTED, "FP16/BF16 form: grid_n must be 128 or 256 and the array "
                                         "footprint at most 128 grid rows");
     p->kp = epic::tc_kp(p->rows_alloc);
-    e = epic::tc_prepare(p->precision == EPIC_PREC_BF16, epic::tc_smem(p->kp));
+    e = epic::tc_prepare(p->precision == EPIC_PREC_BF16);
     if (e != cudaSuccess) return cuda_fail(e, "tensor-core kernel attributes");
     // gridding lists by blocks of rows small enough for four CTAs per SM;
     // through L1 where two blocks' lists of 4 rows are still too large

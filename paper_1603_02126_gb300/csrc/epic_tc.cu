@@ -44,6 +44,7 @@
 #include "epic_internal.h"
 #include "epic_lists.cuh"
 #include "epic_residue.cuh"
+#include "epic_smem.cuh"
 
 namespace epic {
 namespace {
@@ -1116,7 +1117,7 @@ template <int FMT, typename T, bool TS>
 cudaError_t grid_lp_launch(const TcArgs& a, long long t0, int nt, int sms, cudaStream_t s) {
   const size_t smem = tc_grid_smem(a.u.n_ant, a.rb, a.kr, TS ? a.max_lists : 0);
   auto k = grid_lp_kernel<FMT, T, TS>;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  cudaError_t e = allow_smem(k);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kLBT, smem);
@@ -1131,7 +1132,7 @@ template <int FMT, typename T>
 cudaError_t grid_lp_one_launch(const TcArgs& a, long long t0, int nt, int sms, cudaStream_t s) {
   const size_t smem = static_cast<size_t>(a.u.n_ant) * sizeof(float2);
   auto k = grid_lp_one_kernel<FMT, T>;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  cudaError_t e = allow_smem(k);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kOBT, smem);
@@ -1162,19 +1163,11 @@ bool tc_supported(int n, int rows_alloc) { return (n == 128 || n == 256) && 2 * 
 
 int tc_kp(int rows_alloc) { return ((2 * rows_alloc + 63) / 64) * 64; }
 
-size_t tc_smem(int kp) { return tc_smem_bytes(kp); }
 
-cudaError_t tc_prepare(bool bf16, size_t smem) {
-  cudaError_t e = bf16 ? cudaFuncSetAttribute(tc_rows_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              static_cast<int>(tc_rows_smem_bytes()))
-                       : cudaFuncSetAttribute(tc_rows_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              static_cast<int>(tc_rows_smem_bytes()));
+cudaError_t tc_prepare(bool bf16) {
+  cudaError_t e = bf16 ? allow_smem(tc_rows_kernel<true>) : allow_smem(tc_rows_kernel<false>);
   if (e != cudaSuccess) return e;
-  if (bf16)
-    return cudaFuncSetAttribute(tc_cols_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                static_cast<int>(smem));
-  return cudaFuncSetAttribute(tc_cols_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              static_cast<int>(smem));
+  return bf16 ? allow_smem(tc_cols_kernel<true>) : allow_smem(tc_cols_kernel<false>);
 }
 
 // Tensor maps over the window grid Gh [rows_cap][kr] and the row DFT [2N][kr].
@@ -1235,8 +1228,7 @@ cudaError_t launch_tc_batch(const TcArgs& a, const void* tm_dft, const void* tm_
 }
 
 cudaError_t xe_prepare() {
-  return cudaFuncSetAttribute(xengine_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              static_cast<int>(xe_smem_bytes()));
+  return allow_smem(xengine_tc_kernel);
 }
 
 bool xe_make_map(void* z, int n_chan, int na_p, int tp, void* tm) {

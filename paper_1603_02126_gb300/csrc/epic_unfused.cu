@@ -24,6 +24,7 @@
 #include "epic_bulk.cuh"
 #include "epic_fft.cuh"
 #include "epic_internal.h"
+#include "epic_smem.cuh"
 #include "epic_sum.cuh"
 
 #include <cstdint>
@@ -568,7 +569,7 @@ cudaError_t persistent_launch(const UnfusedArgs& a, long long n_time, int nt_bat
                               cudaStream_t s) {
   const size_t es = static_cast<size_t>(kRowFrames) * a.n_ant * sizeof(float2);
   auto kern = unfused_persistent_kernel<N, NZR, NZC>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(es));
+  cudaError_t e = allow_smem(kern);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kUBT, es);
@@ -624,16 +625,14 @@ cudaError_t rows_dispatch(const UnfusedArgs& a, long long t0, int nt, int sms, c
   int per_sm = 0;
   cudaError_t e = cudaSuccess;
   if (a.row_table != 0) {                           // -1: shared memory if that keeps the occupancy, 1: always
-    e = cudaFuncSetAttribute(rows_window_kernel<N, NZ, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(smem_ts));
+    e = allow_smem(rows_window_kernel<N, NZ, true>);
     if (e == cudaSuccess)
       e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rows_window_kernel<N, NZ, true>, kUBT, smem_ts);
     if (e == cudaSuccess && per_sm >= 1 && (a.row_table == 1 || per_sm >= (N <= 128 ? 3 : 2)))
       return rows_launch<N, NZ, true>(a, t0, nt, sms, smem_ts, per_sm, s);
     cudaGetLastError();
   }
-  e = cudaFuncSetAttribute(rows_window_kernel<N, NZ, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           static_cast<int>(es));
+  e = allow_smem(rows_window_kernel<N, NZ, false>);
   if (e != cudaSuccess) return e;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rows_window_kernel<N, NZ, false>, kUBT, es);
   if (e != cudaSuccess) return e;
@@ -647,8 +646,7 @@ cudaError_t cols_launch(const UnfusedArgs& a, int nt, int sms, cudaStream_t s) {
   constexpr int NCOL = N < GROUPS ? N : GROUPS;
   constexpr bool STAGE = N <= 256;
   const size_t smem = STAGE ? static_cast<size_t>(2) * NCOL * a.rs * sizeof(float2) : 0;
-  cudaError_t e = cudaFuncSetAttribute(cols_window_kernel<N, NZ, STAGE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
+  cudaError_t e = allow_smem(cols_window_kernel<N, NZ, STAGE>);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cols_window_kernel<N, NZ, STAGE>, kUBT, smem);

@@ -34,6 +34,7 @@
 #include "epic_internal.h"
 #include "epic_lists.cuh"
 #include "epic_residue.cuh"
+#include "epic_smem.cuh"
 
 #include <cstdint>
 
@@ -311,8 +312,8 @@ cudaError_t prepare_n(const WideArgs& w, int fmt, int* rows_per_sm, int* cols_pe
   const int room = most - 256;                               // static shared memory beside the dynamic
   if (rows_smem<N>(w) > static_cast<size_t>(room) || cols_smem<N>(w) > static_cast<size_t>(room)) return cudaSuccess;
   auto rk = fmt ? wide_rows_kernel<N, 1> : wide_rows_kernel<N, 0>;
-  e = cudaFuncSetAttribute(rk, cudaFuncAttributeMaxDynamicSharedMemorySize, room);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(wide_cols_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, room);
+  e = allow_smem(rk);
+  if (e == cudaSuccess) e = allow_smem(wide_cols_kernel<N>);
   if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(rows_per_sm, rk, kWBT, rows_smem<N>(w));
   if (e == cudaSuccess)
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(cols_per_sm, wide_cols_kernel<N>,

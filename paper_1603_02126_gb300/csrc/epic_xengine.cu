@@ -20,6 +20,7 @@
 #include <algorithm>
 
 #include "epic_internal.h"
+#include "epic_smem.cuh"
 #include "epic_sum.cuh"
 
 namespace epic {
@@ -449,7 +450,7 @@ cudaError_t launch_stefcal(const StefcalArgs& args, const double2* vis64, int sm
   pair_terms_kernel<<<static_cast<unsigned>(a.n_chan * a.n_ant), 128, 0, s>>>(a, vis64);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(stefcal_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024);
+  e = allow_smem(stefcal_kernel);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(a.n_chan * cl));
