@@ -95,8 +95,11 @@ typedef struct {
                                       illumination patterns), or NULL = kernel_param for all */
   int batch_persistent;        /* UNFUSED FP32, N = 256 or 512: 1 = every epic_image call is one
                                   persistent cooperative launch over all its batches (grid
-                                  barriers between the row, column and correlation phases);
-                                  0 = one launch per kernel and batch; epic_autotune may switch it */
+                                  barriers between the row, column and correlation phases; one
+                                  frame per FP32 value); 0 = one launch per kernel and batch, two
+                                  frames per value, the faster form (2048 antennas, 512 x 512,
+                                  256 channels: half the time).  epic_autotune may switch plans
+                                  created with 1, or without room for a frame pair in their scratch */
 } epic_plan_desc;
 
 /* Read-only facts about a plan (epic_plan_get_info). */
@@ -116,8 +119,10 @@ typedef struct {
 /* Result of epic_autotune. */
 typedef struct {
   int path;                    /* epic_path that was tuned */
-  int units_target;            /* FUSED: work units per CTA aimed for */
-  int batch_time;              /* UNFUSED: time samples per batch (0 = scratch budget) */
+  int units_target;            /* FUSED: least frame pairs per CTA; work units per CTA aimed for
+                                  where calls of this length image one frame per FP32 value */
+  int batch_time;              /* UNFUSED, and FUSED with scratch: time samples per batch (0 = the
+                                  scratch's) */
   int cols_target;             /* UNFUSED: column-FFT units per SM aimed for */
   double ms_default, ms_best;  /* epic_image time before / after tuning */
   int candidates;              /* launch shapes timed */
@@ -193,12 +198,14 @@ epic_status epic_image_host_static(epic_plan_t plan, const void* h_volt, long lo
                                    double* h_image, int accumulate);
 
 /* Batching form, autotuner: times candidate launch shapes of epic_image on
- * this batch (FUSED: work units per CTA, i.e. the time-segment length of a
- * persistent CTA's work unit; UNFUSED: time samples per batch and
- * column-FFT work units per SM, then for FP32 the row kernel's variant:
- * gather table in shared memory or read through L1, one or two frames per
- * step, and for N = 256 / 512 whether a call runs as one persistent
- * launch), keeps the fastest in the plan and reports it in *out (may be
+ * this batch (FUSED: frame pairs or work units per CTA; plans that image
+ * frame pairs through device memory, i.e. UNFUSED at N = 256 / 512 and FUSED
+ * with scratch: time samples per batch; other UNFUSED plans: time samples
+ * per batch and column-FFT work units per SM, then for FP32 the row kernel's
+ * variant, gather table in shared memory or read through L1, one or two
+ * frames per step, and for N = 256 / 512 with batch_persistent whether a call
+ * runs as one persistent launch), keeps the fastest in the plan and reports
+ * it in *out (may be
  * NULL).  d_image is overwritten; EPICal sums are left
  * untouched.  Synchronous.  The paper has no counterpart (run-time tuning
  * of this implementation). */

@@ -2545,7 +2545,32 @@ epic_status epic_autotune(epic_plan_t p, const void* d_volt, long long n_time, d
   double best = 0.0;
   epic_status st = EPIC_OK;
   const int reps = 3;
-  if (p->path == EPIC_PATH_FUSED) {
+  if (p->wide && (p->path == EPIC_PATH_UNFUSED || pair_call(p, n_time))) {
+    // the wide form reads the batch length alone
+    const int def = p->tune_nt;
+    st = time_image(p, d_volt, n_time, d_image, reps, &r.ms_default);
+    best = r.ms_default;
+    r.batch_time = def;
+    p->tune_nt = 0;
+    const long long full = wide_batch(p, n_time).nt;
+    for (long long nt = full / 4 * 2; nt >= 2 && st == EPIC_OK; nt = nt / 4 * 2) {
+      p->tune_nt = static_cast<int>(std::min<long long>(nt, 1 << 30));
+      double ms = 0;
+      st = time_image(p, d_volt, n_time, d_image, reps, &ms);
+      ++r.candidates;
+      if (st != EPIC_OK || ms > 2.0 * best) break;
+      if (ms < best) {
+        best = ms;
+        r.batch_time = p->tune_nt;
+      }
+    }
+    p->tune_nt = r.batch_time;
+    r.units_target = p->tune_units;
+    r.cols_target = p->tune_cols;
+    r.row_table = p->tune_row_table;
+    r.row_frames = p->tune_row_frames;
+    r.batch_persistent = p->persistent;
+  } else if (p->path == EPIC_PATH_FUSED) {
     int& knob = p->pair && pair_call(p, n_time) ? p->tune_pairs : p->tune_units;
     const int def = knob;
     st = time_image(p, d_volt, n_time, d_image, reps, &r.ms_default);
@@ -2593,7 +2618,7 @@ epic_status epic_autotune(epic_plan_t p, const void* d_volt, long long n_time, d
     // one or two frames per step
     r.row_table = p->tune_row_table;
     r.row_frames = p->tune_row_frames;
-    if (p->precision == EPIC_PREC_FP32 && !p->wide)
+    if (p->precision == EPIC_PREC_FP32)
       for (int tb : {0, 1})
         for (int rf : {1, 2}) {
           if (st != EPIC_OK) break;
@@ -2612,7 +2637,7 @@ epic_status epic_autotune(epic_plan_t p, const void* d_volt, long long n_time, d
     p->tune_row_frames = r.row_frames;
     // then one persistent launch per call against the batched launches
     r.batch_persistent = p->persistent;
-    if (p->precision == EPIC_PREC_FP32 && !p->wide && epic::persistent_supported(p->n) && st == EPIC_OK) {
+    if (p->precision == EPIC_PREC_FP32 && epic::persistent_supported(p->n) && st == EPIC_OK) {
       const int def_pers = p->persistent;
       p->persistent = 1 - def_pers;
       double ms = 0;
