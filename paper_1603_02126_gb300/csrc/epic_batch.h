@@ -1,8 +1,9 @@
-// Host arithmetic of the wide frame-pair form's batches (no CUDA).
+// Host arithmetic of the frame-pair forms' batches and shares (no CUDA).
 #pragma once
 
 #include <algorithm>
 #include <cstddef>
+#include <vector>
 
 namespace epic {
 
@@ -44,6 +45,21 @@ inline size_t wide_scratch(int C, int N, int rs, size_t budget) {
   const size_t frames = budget / (static_cast<size_t>(N) * rs * 8);
   const long long nt = wide_batch(C, N, rs, budget, 0, 1LL << 40).nt;
   return frames * N * rs + static_cast<size_t>(nt) * C;
+}
+
+// [n + 1] prefix sums of the costs by which CTAs share the channels, scaled
+// down together where their sum would not fit.
+inline std::vector<int> cost_prefix(const std::vector<long long>& cost) {
+  const auto sum_of = [&](int shift) {
+    long long s = 0;
+    for (long long c : cost) s += std::max(1LL, c >> shift);
+    return s;
+  };
+  int shift = 0;
+  while (sum_of(shift) > (1LL << 30) && shift < 40) ++shift;
+  std::vector<int> out{0};
+  for (long long c : cost) out.push_back(out.back() + static_cast<int>(std::max(1LL, c >> shift)));
+  return out;
 }
 
 }  // namespace epic

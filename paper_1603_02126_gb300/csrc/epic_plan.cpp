@@ -614,16 +614,6 @@ void block_taps(const epic_plan_s* p, const std::vector<float>& wts, int c, int 
   }
 }
 
-void prefix_sums(std::vector<int>* v) {
-  int sum = 0;
-  for (int& x : *v) {
-    const int w = x;
-    x = sum;
-    sum += w;
-  }
-  v->push_back(sum);
-}
-
 // Cost of one transform task of P outputs from L inputs and of the whole
 // transform of an N-point axis, in packed FP32 instructions of a thread.
 long long task_cost(int P, int L) { return 18LL * P + 5LL * std::max(0, ((L + 3) & ~3) - P); }
@@ -637,6 +627,7 @@ struct CellTables {
 
 epic_status build_cells(const epic_plan_s* p, const std::vector<float>& wts, int gs, CellTables* t) {
   const int N = p->n;
+  std::vector<long long> cost;
   SliceLists l;
   std::vector<std::vector<Tap>> taps;
   for (int c = 0; c < p->nc; ++c) {
@@ -656,11 +647,11 @@ epic_status build_cells(const epic_plan_s* p, const std::vector<float>& wts, int
     const long long work = static_cast<long long>(N) * (N / 16) * task_cost(16, R) +
                            static_cast<long long>(R) * (N / 16) * task_cost(16, p->cols[c]) +
                            12LL * static_cast<long long>(taps[0].size()) + 20LL * p->na;
-    t->cost.push_back(static_cast<int>(std::max<long long>(1, work / 256)));
+    cost.push_back(work / 256);
   }
   t->sbase.push_back(static_cast<int>(t->slice.size()));
   t->ebase.push_back(static_cast<int>(t->ent.size()));
-  prefix_sums(&t->cost);
+  t->cost = epic::cost_prefix(cost);
   return EPIC_OK;
 }
 
@@ -679,6 +670,7 @@ epic_status build_wide_lists(const epic_plan_s* p, const std::vector<float>& wts
   *t = WideTables();
   t->nb_max = (p->rows_alloc + rb - 1) / rb;
   t->at.assign(static_cast<size_t>(p->nc) * t->nb_max, make_int2(0, 0));
+  std::vector<long long> row_cost, col_cost, blocks;
   SliceLists l;
   std::vector<std::vector<Tap>> taps;
   std::vector<unsigned char> inside;
@@ -714,14 +706,14 @@ epic_status build_wide_lists(const epic_plan_s* p, const std::vector<float>& wts
     // gridding, and the row transforms where the same kernel runs them
     long long rows = 10 * listed + 20LL * p->na;
     if (p->precision == EPIC_PREC_FP32) rows += static_cast<long long>(R) * (N / 32) * task_cost(32, p->cols[c]);
-    t->blocks.push_back(static_cast<int>(taps.size()));
-    t->row_cost.push_back(static_cast<int>(std::max<long long>(1, rows / 256)));
-    t->col_cost.push_back(static_cast<int>(task_cost(32, R)));
+    blocks.push_back(static_cast<long long>(taps.size()));
+    row_cost.push_back(rows / 256);
+    col_cost.push_back(task_cost(32, R));
   }
   t->max_lists = (t->max_lists + 127) & ~127;
-  prefix_sums(&t->blocks);
-  prefix_sums(&t->row_cost);
-  prefix_sums(&t->col_cost);
+  t->blocks = epic::cost_prefix(blocks);
+  t->row_cost = epic::cost_prefix(row_cost);
+  t->col_cost = epic::cost_prefix(col_cost);
   return EPIC_OK;
 }
 
