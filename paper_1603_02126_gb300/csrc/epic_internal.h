@@ -38,7 +38,6 @@ struct ImageArgs {
   double img_scale;        // 1 / T_call
   int do_cal;              // accumulate K, P
   int k0x, k0y;            // calibrator pixel
-  float pix_sign;          // (-1)^(k0x+k0y): centring factor of the image
   double2* kacc;           // [C][Na] sum_t E_a conj(P(t))
   double* pacc;            // [C][Na] sum_t |E_a|^2
   int segs;                // time segments per channel (units = C * segs)
@@ -291,7 +290,6 @@ struct UnfusedArgs {
   double* image;           // [C][N][N]
   double img_scale;
   int do_cal, k0x, k0y;
-  float pix_sign;
   double2* kacc;
   double* pacc;
   int cols_target;         // column-FFT work units per SM to aim for

@@ -787,7 +787,6 @@ epic::ImageArgs fused_args(epic_plan_t p, const void* d_volt, long long n_time, 
   a.do_cal = p->cal ? 1 : 0;
   a.k0x = p->cal ? p->k0x : 0;
   a.k0y = p->cal ? p->k0y : 0;
-  a.pix_sign = ((a.k0x + a.k0y) & 1) ? -1.0f : 1.0f;
   a.kacc = p->d_kacc.p;
   a.pacc = p->d_pacc.p;
   a.segs = choose_segments(p->nc, n_time, p->ctas, p->tune_units);
@@ -1021,7 +1020,6 @@ epic_status image_unfused(epic_plan_t p, const void* d_volt, long long n_time, d
   a.do_cal = p->cal ? 1 : 0;
   a.k0x = p->cal ? p->k0x : 0;
   a.k0y = p->cal ? p->k0y : 0;
-  a.pix_sign = ((a.k0x + a.k0y) & 1) ? -1.0f : 1.0f;
   a.kacc = p->d_kacc.p;
   a.pacc = p->d_pacc.p;
   a.cols_target = p->tune_cols;
@@ -1155,7 +1153,6 @@ epic_status image_tc(epic_plan_t p, const void* d_volt, long long n_time, double
   u.do_cal = p->cal ? 1 : 0;
   u.k0x = p->cal ? p->k0x : 0;
   u.k0y = p->cal ? p->k0y : 0;
-  u.pix_sign = ((u.k0x + u.k0y) & 1) ? -1.0f : 1.0f;
   u.kacc = p->d_kacc.p;
   u.pacc = p->d_pacc.p;
   u.cols_target = p->tune_cols;
