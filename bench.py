@@ -43,7 +43,7 @@ FP32_LANES_PER_SM = 128
 # ncu dram__bytes_read.sum + dram__bytes_write.sum of one fused image launch
 # on this workload, with kernel_sha() of the sources it was taken at;
 # ignored when those sources have changed since.
-TRAFFIC = {"kernel_sha": "4d2c4aef8a7b", "bytes_per_launch": 178779904}
+TRAFFIC = {"kernel_sha": "4d1a0d27a194", "bytes_per_launch": 178615552}
 
 
 def kernel_sha() -> str:

@@ -14,16 +14,20 @@
 // Gridding (Eq. 9) gives each lane one grid cell, the cells sorted by their
 // number of taps so that the 32 lanes of a slice run equally long.
 //
-// What bounds it: the FP32 pipe.  A packed instruction takes two cycles (the
-// scalar rate) and three with three distinct operands; one transform task of
-// 40 inputs takes 252 SM cycles with 16 warps resident (DFT 75, twiddles 37,
-// square 20, the rest the input sum and its shared-memory loads), 42 tasks
-// per pair of the 256-antenna, 128 x 128 station.  64 channels x 10^4 4-bit
-// samples: 15.3 ms against 19.3 for one frame per FP32 value with an
-// exchange through shared memory (63 % of the issue slots, 42 % of the FP32
-// pipe); 128 samples 0.254 against 0.361 ms; 248 antennas, 64 x 64, 15
-// channels, 1023 complex64 samples 0.297 against 0.426; 32 antennas, 32 x 32,
-// 2000 samples 37.6 against 53.9 us (with the update).
+// What bounds it: no unit is full (64 channels x 4096 4-bit samples of 256
+// antennas, 128 x 128: issue slots 51 %, FP32 pipe 51 %, shared-memory pipe
+// 46 %); 16 warps wait in turn for the FP32 pipe and for the shared-memory
+// loads and dependent steps of their tasks (stalls per issue: wait 1.5, not
+// selected 1.3, math throttle 1.3, barrier 1.1, short scoreboard 1.1).  A
+// packed instruction takes two cycles (the scalar rate) and three with three
+// distinct operands; one transform task of 40 inputs takes 252 SM cycles with
+// 16 warps resident (DFT 75, twiddles 37, square 20, the rest the input sum and
+// its loads), 42 tasks per pair of the 256-antenna station: three quarters of
+// the time.  64 channels x 10^4 samples: 15.3 ms against 19.2 for one frame per
+// FP32 value with an exchange through shared memory (63 % of the issue slots,
+// 42 % of the FP32 pipe); 128 samples 0.264 against 0.363 ms; 248 antennas,
+// 64 x 64, 15 channels, 1023 complex64 samples 0.310 against 0.425; 32 antennas,
+// 32 x 32, 2000 samples 37.4 against 53.1 us (with the update).
 #include "epic_fft.cuh"
 #include "epic_internal.h"
 #include "epic_pair.cuh"

@@ -20,8 +20,8 @@
 // 8192 frames of 1024 antennas, 256 x 256: rows 0.47, columns 0.55 ms, HBM 2.7
 // and 2.6 TB/s.  16-output tasks would need twice the loads; three CTAs per SM
 // (168 registers) were slower in the row kernel (17.0 against 16.6 ms).  4096
-// samples of 32 channels: 16.6 ms against 38.1 for the one-frame kernels; 2048
-// antennas, 512 x 512, 128 complex64 samples of 256 channels 23.5 against 53.4;
+// samples of 32 channels: 16.8 ms against 38.2 for the one-frame kernels; 2048
+// antennas, 512 x 512, 128 complex64 samples of 256 channels 24.0 against 53.3;
 // 200 antennas on 76 of 128 grid rows, 16 channels, 2000 samples 1.34 against
 // 1.57 for the one-frame fused kernel.
 //
