@@ -216,8 +216,9 @@ epic_status epic_autotune(epic_plan_t plan, const void* d_volt, long long n_time
  * of d_volt (n_time samples, all channels) into d_image followed, when
  * EPICal is configured, by epical_update writing d_gains_out (may be NULL),
  * into a graph owned by the plan.  Buffers are bound at capture; the plan
- * stream must not be the legacy default stream.  Replace the graph by
- * capturing again.  Synchronous. */
+ * stream must not be the legacy default stream.  Later calls of the plan,
+ * also longer ones, leave the graph valid (scratch that it binds is kept).
+ * Replace the graph by capturing again.  Synchronous. */
 epic_status epic_graph_capture(epic_plan_t plan, const void* d_volt, long long n_time, double* d_image,
                                double* d_gains_out);
 

@@ -185,7 +185,7 @@ struct epic_plan_s {
 
   // differentiation form
   DevBuf<double2> d_dldw;       // [C][Na] dL/dconj(w) accumulator
-  // one-frame fused kernel of a frame-pair plan (calls with BF16 gradients)
+  // one-frame fused kernel of a frame-pair plan (see pair_call)
   bool one_ready = false;
   int one_steps = 1, one_gsmem = 0, one_ctas = 0;
   size_t one_smem = 0;
@@ -385,8 +385,6 @@ float2 window_phase(epic_plan_t p, int c, int kx, int ky) {
   return make_float2(static_cast<float>(sg * std::cos(th)), static_cast<float>(sg * std::sin(th)));
 }
 
-// Tap buffer of the multiple-pixel form for calls of up to n_time samples
-// (grown outside any stream capture: epic_graph_capture sizes it first).
 // Buffers that a later call may replace: when this call is being captured
 // (by epic_graph_capture or by the caller), its graph holds their addresses.
 void bind_captured(epic_plan_s* p) {
@@ -423,6 +421,8 @@ cudaError_t grow(epic_plan_s* p, DevBuf<T>& b, size_t need, size_t most) {
   return b.alloc(need);
 }
 
+// Tap buffer of the multiple-pixel form for calls of up to n_time samples
+// (grown outside any stream capture: epic_graph_capture sizes it first).
 epic_status ensure_ptap(epic_plan_t p, long long n_time) {
   if (p->npix < 1 || p->ptap_time >= n_time) return EPIC_OK;
   cudaError_t e = cudaStreamSynchronize(p->stream);
