@@ -458,6 +458,8 @@ epic_status build_gather(epic_plan_t p, const std::vector<float>& wts, int N1, b
   // per channel a counting sort of the taps by (lane, j): antennas in order
   // inside a group
   const size_t groups = static_cast<size_t>(RA) * N1 * N2;
+  int shift = 0;                           // N1 is a power of two
+  while ((1 << shift) < N1) ++shift;
   std::vector<int> at(groups + 1);
   const auto each_tap = [&](int c, auto&& f) {
     for (int a = 0; a < Na; ++a) {
@@ -469,7 +471,8 @@ epic_status build_gather(epic_plan_t p, const std::vector<float>& wts, int N1, b
       for (int dy = 0; dy < K; ++dy)
         for (int dx = 0; dx < K; ++dx) {
           const int x = xa + dx;
-          if (wf[dy * K + dx] != 0.0f) f((static_cast<size_t>(r0 + dy) * N1 + x % N1) * N2 + x / N1, a, wf[dy * K + dx]);
+          if (wf[dy * K + dx] != 0.0f)
+            f((static_cast<size_t>(r0 + dy) * N1 + (x & (N1 - 1))) * N2 + (x >> shift), a, wf[dy * K + dx]);
         }
     }
   };
@@ -607,10 +610,11 @@ void block_taps(const epic_plan_s* p, const std::vector<float>& wts, int c, int 
     const size_t ob = (static_cast<size_t>(c) * Na + a) * 2;
     const int r0 = p->base[ob + 1] - h - p->y0[c], x0 = p->base[ob] - h - p->x0[c];
     const float* wf = &wts[(static_cast<size_t>(c) * Na + a) * KK];
-    for (int dy = 0; dy < K; ++dy)
+    for (int dy = 0; dy < K; ++dy) {
+      const int b = (r0 + dy) / rb, cell = (r0 + dy - b * rb) * gs + x0;
       for (int dx = 0; dx < K; ++dx)
-        if (wf[dy * K + dx] != 0.0f)
-          (*blocks)[(r0 + dy) / rb].push_back(Tap{(r0 + dy) % rb * gs + x0 + dx, a, wf[dy * K + dx]});
+        if (wf[dy * K + dx] != 0.0f) (*blocks)[b].push_back(Tap{cell + dx, a, wf[dy * K + dx]});
+    }
   }
 }
 
